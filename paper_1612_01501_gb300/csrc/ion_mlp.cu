@@ -10,10 +10,10 @@
 // Training (ion_surrogate_train): samples V uniform in [v_lo, v_hi] and [Ca] log-uniform
 // are drawn on the device (splitmix64 in counter form, Steele-Lea-Flood 2014), labelled
 // by the exact FP32 rate functions of ion_model.cuh, and fitted by minibatch Adam.  Each
-// minibatch is one launch of mlp_grad_kernel (128 samples per CTA; forward and backward
-// in FP32 with activations in shared memory; each CTA writes its partial gradient) and
-// one launch of mlp_adam_kernel (sums the partials in a fixed order, then the Adam step
-// on FP32 master weights), so training is deterministic.
+// minibatch is one launch of mlp_fwdbwd_kernel (forward and backward in FP32; activations
+// and deltas to an L2-resident buffer) and one of mlp_wgrad_kernel (the gradient of every
+// parameter over 128-sample groups, the groups added in a fixed order, then the Adam step on
+// FP32 master weights), so training is deterministic.
 //
 // Inference runs on the tensor cores, BF16 weights and activations with FP32 accumulation:
 // by default on tcgen05 with TMEM accumulators (ion_mlp_tc.cu: ion_surrogate_eval and the
@@ -38,8 +38,7 @@ namespace ion {
 constexpr int MI = ION_MLP_IN, MH = ION_MLP_HID, MO = ION_MLP_OUT;
 constexpr int P_W1 = 0, P_B1 = P_W1 + MH * MI, P_W2 = P_B1 + MH, P_B2 = P_W2 + MH * MH, P_W3 = P_B2 + MH,
               P_B3 = P_W3 + MO * MH, P_TOTAL = P_B3 + MO;   // 5912 parameters, the order of ion_surrogate_weights
-constexpr int MB = 128;                                      // samples per CTA in training
-constexpr int HS = MH + 1;                                   // padded row stride of activation tiles
+constexpr int MB = 128;                                      // samples per partial sum in training
 constexpr float V_CENTER = -25.0f, V_HALF = 75.0f;
 constexpr float LOGIT_MAX = 15.0f;
 
@@ -140,9 +139,32 @@ __global__ void mlp_normalise_kernel(int64_t n, const float *V, const float *ca,
     for (int j = 0; j < MO; ++j) T[k * MO + j] = (T[k * MO + j] - shift[j]) / scale[j];
 }
 
-// ---- training: one minibatch, forward + backward per sample, partial gradients per CTA ----
+// ---- training: one minibatch in two launches ------------------------------------------------
 // Samples of the minibatch: local index j in [0, B) maps to sample (mul * (j0 + j) + add) mod n
 // (a bijection when gcd(mul, n) = 1: a cheap per-epoch reshuffle).
+//
+// The arithmetic of a minibatch is small (0.07 GFLOP at B = 1024) and its sums have a fixed
+// order, so the time is the latency of the dependent chains and the point is to have many of
+// them in flight.  The forward / backward launch takes GS = 8 samples per CTA (128 CTAs at
+// B = 1024), a thread per (sample pair, hidden unit), each dot product one 64-step chain; it
+// leaves the activations and the deltas in L2, one row per unit.  The gradient launch gives
+// every parameter and every 128-sample group a chain of its own: a CTA stages 8 activation and
+// 8 delta rows of up to 8 groups (64 KB, one round of 16-byte async copies) and holds two chains per
+// thread; it adds the groups in order and takes the Adam step.  One sample per
+// thread, 128 samples per CTA (8 CTAs at B = 1024) and the gradients in the same kernel
+// measured 75 us per minibatch of 1024; this split 14.8 us (fwd / bwd 4.3 and gradients 5.5
+// when each runs alone; the rest is the first read of what the other launch just wrote), with
+// every sum in the same order, so the weights are the same bits.
+constexpr int GS = 8;             // samples per CTA of the forward / backward launch
+constexpr int WP = MH + 4;        // row stride of the weight copies: conflict-free 16-byte rows
+constexpr int VEC_PARAMS = MH * MI + MH + MH + MO + 1;   // W1, b1, b2, b3 and the loss
+constexpr int WG_GROUPS = 8;      // 128-sample groups in flight per CTA of the gradient launch
+constexpr int WG_TILE = 8;        // a W2 / W3 gradient tile is 8 x 8 parameters
+constexpr int WG_TILES2 = (MH / WG_TILE) * (MH / WG_TILE), WG_TILES3 = (MO / WG_TILE) * (MH / WG_TILE);
+constexpr int WG_VEC = 16;        // of the other parameters per CTA
+constexpr int WG_CTAS = WG_TILES2 + WG_TILES3 + (VEC_PARAMS + WG_VEC - 1) / WG_VEC;
+constexpr int WG_GSTRIDE = MB + 4, WG_STRIDE = WG_GROUPS * WG_GSTRIDE + 4;   // staged group and row strides: distinct banks
+
 struct GradArgs {
     const float *params;   // P_TOTAL
     const float *X;        // n x 2 normalised inputs
@@ -153,132 +175,295 @@ struct GradArgs {
     int32_t B;
     uint64_t mul, add;
     float denom;           // B * sum(mask)
-    float *partial;        // gridDim.x x (P_TOTAL + 1): gradient, then the loss sum
+    int64_t rows;          // B rounded up to whole groups of MB samples (rows past B hold zeros)
+    float *work;           // mlp_work_floats(rows): the arrays below, one after the other
 };
+// activations and deltas [unit][rows], inputs [2][rows], loss [rows]
+__device__ __forceinline__ float *wk_h1(const GradArgs &a) { return a.work; }
+__device__ __forceinline__ float *wk_h2(const GradArgs &a) { return a.work + a.rows * MH; }
+__device__ __forceinline__ float *wk_d1(const GradArgs &a) { return a.work + a.rows * (2 * MH); }
+__device__ __forceinline__ float *wk_d2(const GradArgs &a) { return a.work + a.rows * (3 * MH); }
+__device__ __forceinline__ float *wk_d3(const GradArgs &a) { return a.work + a.rows * (4 * MH); }
+__device__ __forceinline__ float *wk_x(const GradArgs &a) { return a.work + a.rows * (4 * MH + MO); }
+__device__ __forceinline__ float *wk_loss(const GradArgs &a) { return a.work + a.rows * (4 * MH + MO + MI); }
+static size_t mlp_work_floats(int64_t rows) { return (size_t)rows * (4 * MH + MO + MI + 1); }
 
-__global__ void __launch_bounds__(MB) mlp_grad_kernel(const GradArgs a) {
-    extern __shared__ __align__(16) float sm[];
-    float *Wt = sm;                          // P_TOTAL
-    float *H1 = Wt + P_TOTAL;                // [MB][HS]
-    float *H2 = H1 + MB * HS;
-    float *D1 = H2 + MB * HS;
-    float *D2 = D1 + MB * HS;
-    float *D3 = D2 + MB * HS;                // [MB][MO + 1]
-    float *Xs = D3 + MB * (MO + 1);          // [MB][2]
-    __shared__ float red[MB];
-    const int s = threadIdx.x;
-    for (int p = s; p < P_TOTAL; p += MB) Wt[p] = a.params[p];
-    const int64_t jl = (int64_t)blockIdx.x * MB + s;
-    const bool valid = jl < a.B;
-    const int64_t k = valid ? (int64_t)((a.mul * (uint64_t)(a.j0 + jl) + a.add) % (uint64_t)a.n) : 0;
+__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gsrc) : "memory");
+}
+// the 64 threads (two warps) that share a sample pair
+__device__ __forceinline__ void pair_sync(int sg) { asm volatile("bar.sync %0, 64;" ::"r"(sg + 1) : "memory"); }
+
+// Forward and backward of GS samples: 256 threads, thread (sg, u) has unit u of samples 2 sg, 2 sg + 1.
+__global__ void __launch_bounds__(256) mlp_fwdbwd_kernel(const GradArgs a) {
+    __shared__ __align__(16) float w2s[MH * WP], w3s[MO * WP];
+    __shared__ __align__(16) float w1s[MH * MI], b1s[MH], b2s[MH], b3s[MO];
+    __shared__ __align__(16) float h1[GS][MH], h2[GS][MH], d1[GS][MH], d2[GS][MH], d3[GS][MO], es[GS][MO];
+    const int tid = threadIdx.x, u = tid & 63, sg = tid >> 6;
+    const int64_t row0 = (int64_t)blockIdx.x * GS + 2 * sg;
+    // the samples are constant data: read before the wait on the previous minibatch
+    float x0[2], x1[2];
+    bool valid[2];
+    int64_t k[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        valid[r] = row0 + r < a.B;
+        k[r] = valid[r] ? (int64_t)((a.mul * (uint64_t)(a.j0 + row0 + r) + a.add) % (uint64_t)a.n) : 0;
+        x0[r] = valid[r] ? a.X[2 * k[r]] : 0.0f;
+        x1[r] = valid[r] ? a.X[2 * k[r] + 1] : 0.0f;
+    }
+    const int so = u / MO, o = u - so * MO;   // layer 3: threads u < 48 have output o of sample 2 sg + so
+    const bool out3 = u < 2 * MO;
+    const bool vo = so == 0 ? valid[0] : valid[1];
+    const float tgt = out3 && vo ? a.T[(so == 0 ? k[0] : k[1]) * MO + o] : 0.0f;
+    const float msk = out3 ? a.mask[o] : 0.0f;
+    pdl_enter();
+    for (int i = tid; i < MH * MH / 4; i += 256)
+        cp_async16(w2s + (i >> 4) * WP + 4 * (i & 15), a.params + P_W2 + 4 * i);
+    for (int i = tid; i < MO * MH / 4; i += 256)
+        cp_async16(w3s + (i >> 4) * WP + 4 * (i & 15), a.params + P_W3 + 4 * i);
+    if (tid < MH * MI / 4) cp_async16(w1s + 4 * tid, a.params + P_W1 + 4 * tid);
+    else if (tid < MH * MI / 4 + MH / 4) cp_async16(b1s + 4 * (tid - 32), a.params + P_B1 + 4 * (tid - 32));
+    else if (tid < MH * MI / 4 + MH / 2) cp_async16(b2s + 4 * (tid - 48), a.params + P_B2 + 4 * (tid - 48));
+    else if (tid < MH * MI / 4 + MH / 2 + MO / 4) cp_async16(b3s + 4 * (tid - 64), a.params + P_B3 + 4 * (tid - 64));
+    cp_async_commit();
+    cp_async_wait_all();
     __syncthreads();
-    const float *w1 = Wt + P_W1, *b1 = Wt + P_B1, *w2 = Wt + P_W2, *b2 = Wt + P_B2, *w3 = Wt + P_W3, *b3 = Wt + P_B3;
-    float loss = 0.0f;
-    const float x0 = valid ? a.X[2 * k] : 0.0f, x1 = valid ? a.X[2 * k + 1] : 0.0f;
-    Xs[2 * s] = x0;
-    Xs[2 * s + 1] = x1;
-    for (int j = 0; j < MH; ++j) H1[s * HS + j] = tanhf(fmaf(w1[2 * j], x0, fmaf(w1[2 * j + 1], x1, b1[j])));
-    for (int j = 0; j < MH; ++j) {
-        float acc = b2[j];
-        for (int q = 0; q < MH; ++q) acc = fmaf(w2[j * MH + q], H1[s * HS + q], acc);
-        H2[s * HS + j] = tanhf(acc);
+    const int s0 = 2 * sg;
+    float h1v[2], h2v[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        h1v[r] = tanhf(fmaf(w1s[2 * u], x0[r], fmaf(w1s[2 * u + 1], x1[r], b1s[u])));
+        h1[s0 + r][u] = h1v[r];
     }
-    for (int o = 0; o < MO; ++o) {
-        float acc = b3[o];
-        for (int q = 0; q < MH; ++q) acc = fmaf(w3[o * MH + q], H2[s * HS + q], acc);
-        const float e = valid ? (acc - a.T[k * MO + o]) * a.mask[o] : 0.0f;
-        loss = fmaf(e, e, loss);
-        D3[s * (MO + 1) + o] = 2.0f * e / a.denom;
+    pair_sync(sg);
+    {
+        float a0 = b2s[u], a1 = a0;
+#pragma unroll
+        for (int q = 0; q < MH; q += 4) {
+            const float4 w = *reinterpret_cast<const float4 *>(w2s + u * WP + q);
+            const float4 p = *reinterpret_cast<const float4 *>(&h1[s0][q]);
+            const float4 v = *reinterpret_cast<const float4 *>(&h1[s0 + 1][q]);
+            a0 = fmaf(w.w, p.w, fmaf(w.z, p.z, fmaf(w.y, p.y, fmaf(w.x, p.x, a0))));
+            a1 = fmaf(w.w, v.w, fmaf(w.z, v.z, fmaf(w.y, v.y, fmaf(w.x, v.x, a1))));
+        }
+        h2v[0] = tanhf(a0);
+        h2v[1] = tanhf(a1);
+        h2[s0][u] = h2v[0];
+        h2[s0 + 1][u] = h2v[1];
     }
-    for (int q = 0; q < MH; ++q) {
-        float acc = 0.0f;
-        for (int o = 0; o < MO; ++o) acc = fmaf(w3[o * MH + q], D3[s * (MO + 1) + o], acc);
-        const float h = H2[s * HS + q];
-        D2[s * HS + q] = acc * (1.0f - h * h);
+    pair_sync(sg);
+    if (out3) {
+        float acc = b3s[o];
+#pragma unroll
+        for (int q = 0; q < MH; q += 4) {
+            const float4 w = *reinterpret_cast<const float4 *>(w3s + o * WP + q);
+            const float4 p = *reinterpret_cast<const float4 *>(&h2[s0 + so][q]);
+            acc = fmaf(w.w, p.w, fmaf(w.z, p.z, fmaf(w.y, p.y, fmaf(w.x, p.x, acc))));
+        }
+        const float e = vo ? (acc - tgt) * msk : 0.0f;
+        es[s0 + so][o] = e;
+        d3[s0 + so][o] = 2.0f * e / a.denom;
     }
-    for (int q = 0; q < MH; ++q) {
-        float acc = 0.0f;
-        for (int j = 0; j < MH; ++j) acc = fmaf(w2[j * MH + q], D2[s * HS + j], acc);
-        const float h = H1[s * HS + q];
-        D1[s * HS + q] = acc * (1.0f - h * h);
+    pair_sync(sg);
+    {
+        float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+        for (int q = 0; q < MO; q += 4) {
+            const float4 p = *reinterpret_cast<const float4 *>(&d3[s0][q]);
+            const float4 v = *reinterpret_cast<const float4 *>(&d3[s0 + 1][q]);
+            const float wa = w3s[q * WP + u], wb = w3s[(q + 1) * WP + u], wc = w3s[(q + 2) * WP + u],
+                        wd = w3s[(q + 3) * WP + u];
+            a0 = fmaf(wd, p.w, fmaf(wc, p.z, fmaf(wb, p.y, fmaf(wa, p.x, a0))));
+            a1 = fmaf(wd, v.w, fmaf(wc, v.z, fmaf(wb, v.y, fmaf(wa, v.x, a1))));
+        }
+        d2[s0][u] = a0 * (1.0f - h2v[0] * h2v[0]);
+        d2[s0 + 1][u] = a1 * (1.0f - h2v[1] * h2v[1]);
     }
-    red[s] = loss;
+    if (u < 2) {   // the sample's loss, in output order
+        float loss = 0.0f;
+#pragma unroll
+        for (int q = 0; q < MO; ++q) loss = fmaf(es[s0 + u][q], es[s0 + u][q], loss);
+        wk_loss(a)[row0 + u] = loss;
+        wk_x(a)[row0 + u] = u == 0 ? x0[0] : x0[1];
+        wk_x(a)[a.rows + row0 + u] = u == 0 ? x1[0] : x1[1];
+    }
+    pair_sync(sg);
+    {
+        float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+        for (int q = 0; q < MH; q += 4) {
+            const float4 p = *reinterpret_cast<const float4 *>(&d2[s0][q]);
+            const float4 v = *reinterpret_cast<const float4 *>(&d2[s0 + 1][q]);
+            const float wa = w2s[q * WP + u], wb = w2s[(q + 1) * WP + u], wc = w2s[(q + 2) * WP + u],
+                        wd = w2s[(q + 3) * WP + u];
+            a0 = fmaf(wd, p.w, fmaf(wc, p.z, fmaf(wb, p.y, fmaf(wa, p.x, a0))));
+            a1 = fmaf(wd, v.w, fmaf(wc, v.z, fmaf(wb, v.y, fmaf(wa, v.x, a1))));
+        }
+        d1[s0][u] = a0 * (1.0f - h1v[0] * h1v[0]);
+        d1[s0 + 1][u] = a1 * (1.0f - h1v[1] * h1v[1]);
+    }
     __syncthreads();
-    // weight gradients of this CTA: sums over its samples, in sample order
-    float *out = a.partial + (int64_t)blockIdx.x * (P_TOTAL + 1);
-    {   // W2, b2: thread -> column q = s % 64, rows j in [32 (s / 64), +32)
-        const int q = s % MH, jh = s / MH;
-        float acc[32];
-#pragma unroll
-        for (int r = 0; r < 32; ++r) acc[r] = 0.0f;
-        for (int t = 0; t < MB; ++t) {
-            const float h = H1[t * HS + q];
-#pragma unroll
-            for (int r = 0; r < 32; ++r) acc[r] = fmaf(D2[t * HS + jh * 32 + r], h, acc[r]);
-        }
-#pragma unroll
-        for (int r = 0; r < 32; ++r) out[P_W2 + (jh * 32 + r) * MH + q] = acc[r];
-    }
-    {   // W3, b3: thread -> column q, outputs o in [12 (s / 64), +12)
-        const int q = s % MH, oh = s / MH;
-        float acc[12];
-#pragma unroll
-        for (int r = 0; r < 12; ++r) acc[r] = 0.0f;
-        for (int t = 0; t < MB; ++t) {
-            const float h = H2[t * HS + q];
-#pragma unroll
-            for (int r = 0; r < 12; ++r) acc[r] = fmaf(D3[t * (MO + 1) + oh * 12 + r], h, acc[r]);
-        }
-#pragma unroll
-        for (int r = 0; r < 12; ++r) out[P_W3 + (oh * 12 + r) * MH + q] = acc[r];
-    }
-    {   // W1 (thread -> hidden unit j = s % 64, input i = s / 64), b1, b2, b3
-        const int j = s % MH, i = s / MH;
-        float acc = 0.0f, bacc = 0.0f, b2acc = 0.0f;
-        for (int t = 0; t < MB; ++t) {
-            acc = fmaf(D1[t * HS + j], Xs[2 * t + i], acc);
-            bacc += D1[t * HS + j];
-            b2acc += D2[t * HS + j];
-        }
-        out[P_W1 + j * MI + i] = acc;
-        if (i == 0) out[P_B1 + j] = bacc;
-        else out[P_B2 + j] = b2acc;
-        if (s < MO) {
-            float b3acc = 0.0f;
-            for (int t = 0; t < MB; ++t) b3acc += D3[t * (MO + 1) + s];
-            out[P_B3 + s] = b3acc;
-        }
-    }
-    if (s == 0) {
-        float L = 0.0f;
-        for (int t = 0; t < MB; ++t) L += red[t];
-        out[P_TOTAL] = L;
+    // a unit's 8 samples are one 32-byte sector of its row: two 16-byte stores, so that every
+    // sector is written once and whole (8-byte stores of each thread's own pair: 15.5 us per
+    // minibatch of 1024 instead of 14.8)
+    const int half = 4 * (tid & 1), unit = (tid >> 1) & 63;
+    const int64_t at = (int64_t)blockIdx.x * GS + half;
+    auto put = [&](float *dst, const float *src, int stride) {   // src: the unit's column, sample-major
+        *reinterpret_cast<float4 *>(dst + unit * a.rows + at) =
+            make_float4(src[half * stride], src[(half + 1) * stride], src[(half + 2) * stride], src[(half + 3) * stride]);
+    };
+    if (tid < 128) {
+        put(wk_h1(a), &h1[0][unit], MH);
+        put(wk_h2(a), &h2[0][unit], MH);
+        if (unit < MO) put(wk_d3(a), &d3[0][unit], MO);
+    } else {
+        put(wk_d1(a), &d1[0][unit], MH);
+        put(wk_d2(a), &d2[0][unit], MH);
     }
 }
 
-size_t mlp_grad_smem() { return (size_t)(P_TOTAL + 4 * MB * HS + MB * (MO + 1) + 2 * MB) * sizeof(float); }
+struct AdamArgs {
+    GradArgs g;
+    float *params, *m, *v;
+    float *grad;           // non-NULL: return the gradient, no Adam step
+    float lr, b1, b2, eps, c1, c2;
+    float *loss;           // non-NULL: += loss sum / denom
+};
 
-// Sum the CTA partials in a fixed order; then either return the gradient (grad != NULL)
-// or take an Adam step on params.  Thread P_TOTAL adds the loss (divided by denom) to *loss.
-__global__ void mlp_adam_kernel(const float *partial, int nblk, float *params, float *m, float *v, float *grad,
-                                float lr, float b1, float b2, float eps, float c1, float c2, float denom, float *loss) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > P_TOTAL) return;
+// sum over a group's samples of d times h, in sample order, and the plain sum
+__device__ __forceinline__ float group_dot(const float *d, const float *h) {
+    float acc = 0.0f;
+#pragma unroll 16
+    for (int t = 0; t < MB; t += 4) {
+        const float4 dd = *reinterpret_cast<const float4 *>(d + t), hh = *reinterpret_cast<const float4 *>(h + t);
+        acc = fmaf(dd.w, hh.w, fmaf(dd.z, hh.z, fmaf(dd.y, hh.y, fmaf(dd.x, hh.x, acc))));
+    }
+    return acc;
+}
+__device__ __forceinline__ float group_sum(const float *d) {
+    float acc = 0.0f;
+#pragma unroll 16
+    for (int t = 0; t < MB; t += 4) {
+        const float4 dd = *reinterpret_cast<const float4 *>(d + t);
+        acc += dd.x;
+        acc += dd.y;
+        acc += dd.z;
+        acc += dd.w;
+    }
+    return acc;
+}
+
+// one 4-sample step of a chain
+__device__ __forceinline__ float dot4(float4 d, float4 h, float acc) {
+    return fmaf(d.w, h.w, fmaf(d.z, h.z, fmaf(d.y, h.y, fmaf(d.x, h.x, acc))));
+}
+
+// Gradients and the Adam step: a warp per group, lane (1 x 2 parameters of the tile, or one of
+// the others).  CTAs 0..63 own an 8 x 8 tile of W2 each, 64..87 one of W3, the rest 16 of the
+// other parameters (and the loss) each.
+__global__ void __launch_bounds__(32 * WG_GROUPS) mlp_wgrad_kernel(const AdamArgs a) {
+    extern __shared__ __align__(16) float rows_s[];   // 16 staged rows: 8 deltas, then 8 activations
+    __shared__ float part[WG_GROUPS][64];
+    const int lt = threadIdx.x & 31, gi = threadIdx.x >> 5, blk = blockIdx.x;
+    const int64_t rows = a.g.rows;
+    const int nblk = (int)(rows / MB);
+    const bool tile = blk < WG_TILES2 + WG_TILES3;
+    const bool w2 = blk < WG_TILES2;
+    const int tb = w2 ? blk : blk - WG_TILES2;
+    const int j0 = tb / (MH / WG_TILE) * WG_TILE, q0 = tb % (MH / WG_TILE) * WG_TILE;
+    // this thread's parameter after the groups are added (threads < 64, < 16 of the vector CTAs)
+    const int np = tile ? 64 : WG_VEC;
+    int p = -1;                    // P_TOTAL: the loss
+    if ((int)threadIdx.x < np) {
+        if (tile) p = (w2 ? P_W2 : P_W3) + (j0 + (threadIdx.x >> 3)) * MH + q0 + (threadIdx.x & 7);
+        else p = (blk - WG_TILES2 - WG_TILES3) * WG_VEC + threadIdx.x;   // list position, mapped below
+    }
+    const int v = tile || lt >= WG_VEC ? -1 : (blk - WG_TILES2 - WG_TILES3) * WG_VEC + lt;
+    auto vec_param = [](int x) {
+        if (x < MH * MI) return P_W1 + x;
+        if (x < MH * MI + MH) return P_B1 + (x - MH * MI);
+        if (x < MH * MI + 2 * MH) return P_B2 + (x - MH * MI - MH);
+        if (x < VEC_PARAMS - 1) return P_B3 + (x - MH * MI - 2 * MH);
+        return x == VEC_PARAMS - 1 ? P_TOTAL : -1;
+    };
+    if (!tile && p >= 0) p = vec_param(p);
+    const int vp = v < 0 ? -1 : vec_param(v);
+    pdl_enter();
+    const bool adam = p >= 0 && p < P_TOTAL && a.grad == nullptr;
+    const float m0 = adam ? a.m[p] : 0.0f, v0 = adam ? a.v[p] : 0.0f, w0 = adam ? a.params[p] : 0.0f;
+    const float *dsrc = w2 ? wk_d2(a.g) : wk_d3(a.g), *hsrc = w2 ? wk_h1(a.g) : wk_h2(a.g);
     float g = 0.0f;
-    for (int b = 0; b < nblk; ++b) g += partial[(int64_t)b * (P_TOTAL + 1) + p];
+    for (int c0 = 0; c0 < nblk; c0 += WG_GROUPS) {
+        const int here = min(WG_GROUPS, nblk - c0);
+        if (tile) {
+            if (gi < here) {   // this warp's group: lane = 16-byte part of the 128 samples
+                const int64_t at = (int64_t)(c0 + gi) * MB + 4 * lt;
+                float *dst = rows_s + gi * WG_GSTRIDE + 4 * lt;
+#pragma unroll
+                for (int r = 0; r < WG_TILE; ++r) {
+                    cp_async16(dst + r * WG_STRIDE, dsrc + (j0 + r) * rows + at);
+                    cp_async16(dst + (WG_TILE + r) * WG_STRIDE, hsrc + (q0 + r) * rows + at);
+                }
+            }
+            cp_async_commit();
+            cp_async_wait_all();
+            __syncwarp();      // a warp reads what its own lanes staged
+            if (gi < here) {
+                const int jj = lt >> 2, qq = 2 * (lt & 3);
+                const float *d = rows_s + jj * WG_STRIDE + gi * WG_GSTRIDE,
+                            *h = rows_s + (WG_TILE + qq) * WG_STRIDE + gi * WG_GSTRIDE;
+                float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll 16
+                for (int t = 0; t < MB; t += 4) {
+                    const float4 dd = *reinterpret_cast<const float4 *>(d + t),
+                                 ha = *reinterpret_cast<const float4 *>(h + t),
+                                 hb = *reinterpret_cast<const float4 *>(h + WG_STRIDE + t);
+                    a0 = dot4(dd, ha, a0);
+                    a1 = dot4(dd, hb, a1);
+                }
+                part[gi][jj * WG_TILE + qq] = a0;
+                part[gi][jj * WG_TILE + qq + 1] = a1;
+            }
+        } else if (gi < here && vp >= 0) {
+            const int64_t t0 = (int64_t)(c0 + gi) * MB;
+            float acc;
+            if (vp == P_TOTAL) acc = group_sum(wk_loss(a.g) + t0);
+            else if (vp < P_B1) acc = group_dot(wk_d1(a.g) + (vp >> 1) * rows + t0, wk_x(a.g) + (vp & 1) * rows + t0);
+            else if (vp < P_W2) acc = group_sum(wk_d1(a.g) + (vp - P_B1) * rows + t0);
+            else if (vp < P_W3) acc = group_sum(wk_d2(a.g) + (vp - P_B2) * rows + t0);
+            else acc = group_sum(wk_d3(a.g) + (vp - P_B3) * rows + t0);
+            part[gi][lt] = acc;
+        }
+        __syncthreads();
+        if (p >= 0)
+            for (int b = 0; b < here; ++b) g += part[b][threadIdx.x];
+        __syncthreads();
+    }
+    if (p < 0) return;
     if (p == P_TOTAL) {
-        if (loss) *loss += g / denom;
+        if (a.loss) *a.loss += g / a.g.denom;
         return;
     }
-    if (grad) {
-        grad[p] = g;
+    if (a.grad) {
+        a.grad[p] = g;
         return;
     }
-    const float mm = b1 * m[p] + (1.0f - b1) * g;
-    const float vv = b2 * v[p] + (1.0f - b2) * g * g;
-    m[p] = mm;
-    v[p] = vv;
-    params[p] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+    const float mm = a.b1 * m0 + (1.0f - a.b1) * g;
+    const float vv = a.b2 * v0 + (1.0f - a.b2) * g * g;
+    a.m[p] = mm;
+    a.v[p] = vv;
+    a.params[p] = w0 - a.lr * (mm / a.c1) / (sqrtf(vv / a.c2) + a.eps);
+}
+
+constexpr size_t WG_SMEM = 2 * WG_TILE * WG_STRIDE * sizeof(float);
+static cudaError_t prepare_minibatch() {
+    return cudaFuncSetAttribute(mlp_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM);
+}
+static cudaError_t launch_minibatch(const AdamArgs &a, bool pdl, cudaStream_t st) {
+    cudaError_t e = launch_k(mlp_fwdbwd_kernel, dim3((unsigned)(a.g.rows / GS)), dim3(256), 0, st, pdl, a.g);
+    if (e == cudaSuccess) e = launch_k(mlp_wgrad_kernel, dim3(WG_CTAS), dim3(32 * WG_GROUPS), WG_SMEM, st, true, a);
+    return e;
 }
 
 // Glorot-uniform weights from the counter-based generator, zero biases
@@ -539,39 +724,38 @@ extern "C" ion_status ion_surrogate_train(const ion_train_cfg *cfg, ion_surrogat
         !(cfg->ca_lo > 0) || !(cfg->ca_hi > cfg->ca_lo))
         return ion_fail(nullptr, ION_ERR_INVALID_ARG, "ion_surrogate_train: bad configuration");
     cudaStream_t st = (cudaStream_t)cfg->cuda_stream;
-    const int nblk = B / MB;
-    const size_t smem = mlp_grad_smem();
-    float *V = nullptr, *ca = nullptr, *X = nullptr, *T = nullptr, *params = nullptr, *m = nullptr, *v = nullptr,
-          *partial = nullptr, *mask = nullptr, *shift = nullptr, *scale = nullptr, *loss = nullptr;
-    double *stat = nullptr;
+    float *V, *ca, *X, *T, *params, *m, *v, *work, *mask, *shift, *scale, *loss;
+    double *stat;
     const int sblk = 64;
-    std::vector<void *> bufs;
-    auto alloc = [&](void **p, size_t bytes) {
-        cudaError_t e = ion_alloc(p, bytes);
-        if (e == cudaSuccess) bufs.push_back(*p);
-        return e;
+    // one allocation for every buffer, cut into 256-byte aligned parts
+    size_t total_bytes = 0;
+    char *arena = nullptr;
+    auto part = [&](size_t bytes) {
+        const size_t at = total_bytes;
+        total_bytes += (bytes + 255) / 256 * 256;
+        return at;
     };
-    auto cleanup = [&]() {
-        for (void *p : bufs) cudaFree(p);
-    };
-    cudaError_t e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = alloc((void **)&V, n * 4);
-    if (e == cudaSuccess) e = alloc((void **)&ca, n * 4);
-    if (e == cudaSuccess) e = alloc((void **)&X, n * 8);
-    if (e == cudaSuccess) e = alloc((void **)&T, n * MO * 4);
-    if (e == cudaSuccess) e = alloc((void **)&params, P_TOTAL * 4);
-    if (e == cudaSuccess) e = alloc((void **)&m, P_TOTAL * 4);
-    if (e == cudaSuccess) e = alloc((void **)&v, P_TOTAL * 4);
-    if (e == cudaSuccess) e = alloc((void **)&partial, (size_t)nblk * (P_TOTAL + 1) * 4);
-    if (e == cudaSuccess) e = alloc((void **)&mask, MO * 4);
-    if (e == cudaSuccess) e = alloc((void **)&shift, MO * 4);
-    if (e == cudaSuccess) e = alloc((void **)&scale, MO * 4);
-    if (e == cudaSuccess) e = alloc((void **)&loss, 4);
-    if (e == cudaSuccess) e = alloc((void **)&stat, (size_t)MO * sblk * 2 * 8);
-    if (e != cudaSuccess) {
-        cleanup();
-        return ion_fail(nullptr, ION_ERR_OOM, "ion_surrogate_train: %s", cudaGetErrorString(e));
-    }
+    const size_t oV = part(n * 4), oca = part(n * 4), oX = part(n * 8), oT = part(n * MO * 4), oparams = part(P_TOTAL * 4),
+                 om = part(P_TOTAL * 4), ov = part(P_TOTAL * 4), owork = part(mlp_work_floats(B) * 4),
+                 omask = part(MO * 4), oshift = part(MO * 4), oscale = part(MO * 4), oloss = part(4),
+                 ostat = part((size_t)MO * sblk * 2 * 8);
+    cudaError_t e = prepare_minibatch();
+    if (e != cudaSuccess) return mlp_cuda(e, "ion_surrogate_train");
+    e = ion_alloc(&arena, total_bytes);
+    if (e != cudaSuccess) return ion_fail(nullptr, ION_ERR_OOM, "ion_surrogate_train: %s", cudaGetErrorString(e));
+    V = (float *)(arena + oV);
+    ca = (float *)(arena + oca);
+    X = (float *)(arena + oX);
+    T = (float *)(arena + oT);
+    params = (float *)(arena + oparams);
+    m = (float *)(arena + om);
+    v = (float *)(arena + ov);
+    work = (float *)(arena + owork);
+    mask = (float *)(arena + omask);
+    shift = (float *)(arena + oshift);
+    scale = (float *)(arena + oscale);
+    loss = (float *)(arena + oloss);
+    stat = (double *)(arena + ostat);
     float hmask[MO];
     for (int o = 0; o < MO; ++o) hmask[o] = (o == 2 * G_MS + 1 || o == 2 * G_MA + 1) ? 0.0f : 1.0f;
     const float lc_lo = logf(cfg->ca_lo), lc_hi = logf(cfg->ca_hi);
@@ -598,17 +782,15 @@ extern "C" ion_status ion_surrogate_train(const ion_train_cfg *cfg, ion_surrogat
         const uint64_t add = (uint64_t)(ep * 7919) % (uint64_t)n;
         if (ep == cfg->epochs - 1) e = cudaMemsetAsync(loss, 0, 4, st);
         for (int64_t b = 0; b < steps_per_epoch && e == cudaSuccess; ++b, ++step) {
-            GradArgs ga{params, X, T, mask, n, b * B, B, mul, add, denom, partial};
-            mlp_grad_kernel<<<nblk, MB, smem, st>>>(ga);
             // cosine decay of the step size to 1 % over the run
             const double frac = total > 1 ? (double)step / (double)(total - 1) : 1.0;
             const float lr = (float)(cfg->lr * (0.01 + 0.99 * 0.5 * (1.0 + cos(M_PI * frac))));
             const double k = (double)(step + 1);
             const float c1 = (float)(1.0 - pow(0.9, k)), c2 = (float)(1.0 - pow(0.999, k));
-            mlp_adam_kernel<<<(P_TOTAL + 1 + 255) / 256, 256, 0, st>>>(partial, nblk, params, m, v, nullptr, lr, 0.9f,
-                                                                        0.999f, 1e-8f, c1, c2, denom,
-                                                                        ep == cfg->epochs - 1 ? loss : nullptr);
-            e = cudaGetLastError();
+            AdamArgs aa{{params, X, T, mask, n, b * B, B, mul, add, denom, B, work},
+                        params, m, v, nullptr, lr, 0.9f, 0.999f, 1e-8f, c1, c2, ep == cfg->epochs - 1 ? loss : nullptr};
+            // the first launch reads the samples that the kernels before it wrote: an ordinary one
+            e = launch_minibatch(aa, step > 0, st);
         }
     }
     float hl = 0.0f;
@@ -617,7 +799,7 @@ extern "C" ion_status ion_surrogate_train(const ion_train_cfg *cfg, ion_surrogat
     if (e == cudaSuccess) e = cudaMemcpyAsync(w_out->out_scale, scale, MO * 4, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hl, loss, 4, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cleanup();
+    cudaFree(arena);
     if (e != cudaSuccess) return ion_fail(nullptr, ION_ERR_CUDA, "ion_surrogate_train: %s", cudaGetErrorString(e));
     // input normalisation: x' = (x - shift) * scale with x = (V, ln [Ca])
     w_out->in_shift[0] = V_CENTER;
@@ -632,16 +814,16 @@ extern "C" ion_status ion_surrogate_grad(const ion_surrogate_weights *w, const f
                                          const float *mask, int32_t B, ion_surrogate_weights *grad, float *loss) {
     if (!w || !x || !t || !mask || !grad || B < 1)
         return ion_fail(nullptr, ION_ERR_INVALID_ARG, "ion_surrogate_grad: bad arguments");
-    const int nblk = (B + MB - 1) / MB;
+    const int64_t rows = ((int64_t)B + MB - 1) / MB * MB;
     float msum = 0.0f;
     for (int o = 0; o < MO; ++o) msum += mask[o];
     if (!(msum > 0)) return ion_fail(nullptr, ION_ERR_INVALID_ARG, "ion_surrogate_grad: empty mask");
-    float *params = nullptr, *X = nullptr, *T = nullptr, *M = nullptr, *partial = nullptr, *g = nullptr, *L = nullptr;
+    float *params = nullptr, *X = nullptr, *T = nullptr, *M = nullptr, *work = nullptr, *g = nullptr, *L = nullptr;
     cudaError_t e = ion_alloc(&params, P_TOTAL * 4);
     if (e == cudaSuccess) e = ion_alloc(&X, (size_t)B * 8);
     if (e == cudaSuccess) e = ion_alloc(&T, (size_t)B * MO * 4);
     if (e == cudaSuccess) e = ion_alloc(&M, MO * 4);
-    if (e == cudaSuccess) e = ion_alloc(&partial, (size_t)nblk * (P_TOTAL + 1) * 4);
+    if (e == cudaSuccess) e = ion_alloc(&work, mlp_work_floats(rows) * 4);
     if (e == cudaSuccess) e = ion_alloc(&g, P_TOTAL * 4);
     if (e == cudaSuccess) e = ion_alloc(&L, 4);
     if (e == cudaSuccess) e = cudaMemcpy(params, w, P_TOTAL * 4, cudaMemcpyHostToDevice);
@@ -649,15 +831,11 @@ extern "C" ion_status ion_surrogate_grad(const ion_surrogate_weights *w, const f
     if (e == cudaSuccess) e = cudaMemcpy(T, t, (size_t)B * MO * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(M, mask, MO * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(L, 0, 4);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_grad_smem());
     const float denom = (float)B * msum;
+    if (e == cudaSuccess) e = prepare_minibatch();
     if (e == cudaSuccess) {
-        GradArgs ga{params, X, T, M, B, 0, B, 1, 0, denom, partial};
-        mlp_grad_kernel<<<nblk, MB, mlp_grad_smem()>>>(ga);
-        mlp_adam_kernel<<<(P_TOTAL + 1 + 255) / 256, 256>>>(partial, nblk, params, nullptr, nullptr, g, 0, 0, 0, 0, 1, 1,
-                                                             denom, L);
-        e = cudaGetLastError();
+        AdamArgs aa{{params, X, T, M, B, 0, B, 1, 0, denom, rows, work}, params, nullptr, nullptr, g, 0, 0, 0, 0, 1, 1, L};
+        e = launch_minibatch(aa, false, nullptr);
     }
     float hl = 0.0f;
     if (e == cudaSuccess) e = cudaMemcpy(grad, g, P_TOTAL * 4, cudaMemcpyDeviceToHost);
@@ -666,7 +844,7 @@ extern "C" ion_status ion_surrogate_grad(const ion_surrogate_weights *w, const f
     cudaFree(X);
     cudaFree(T);
     cudaFree(M);
-    cudaFree(partial);
+    cudaFree(work);
     cudaFree(g);
     cudaFree(L);
     if (e != cudaSuccess)

@@ -54,6 +54,30 @@ def test_training_gradients_match_fp64_oracle(cuda, B):
         assert err.max() <= 0.0, (k, worst, float(g[k][worst]), float(gr[k][worst]), scale)
 
 
+@pytest.mark.parametrize("B", [1, 7, 129, 1025, 2200])
+def test_training_gradients_at_group_edges(cuda, B):
+    # one sample, partial CTAs of 8 samples, partial 128-sample groups, and more groups than
+    # the gradient launch holds at once; the sums have at most B terms of one sign pattern, so
+    # an entry may be off by B * 2^-24 of its largest term (bounded as in the test above, with
+    # the floor grown by sqrt(B / 300) for the longer sums)
+    rng = np.random.default_rng(1000 + B)
+    p = mlp.init_params(6, scale=1.2)
+    x = rng.uniform(-1, 1, (B, 2)).astype(np.float32)
+    t = rng.normal(0, 1, (B, 24)).astype(np.float32)
+    mask = np.ones(24, np.float32)
+    mask[[11, 19]] = 0.0
+    w = ion.weights_from_dict({k: v.astype(np.float32) for k, v in p.items()})
+    L, g = ion.ion_surrogate_grad(w, x, t, mask)
+    p32 = {k: v.astype(np.float32).astype(np.float64) for k, v in p.items()}
+    Lr, gr = mlp.loss_and_grads(p32, x.astype(np.float64), t.astype(np.float64), mask.astype(np.float64))
+    assert L == pytest.approx(Lr, rel=1e-5)
+    floor = 1e-6 * max(1.0, np.sqrt(B / 300))
+    for k in ("w1", "b1", "w2", "b2", "w3", "b3"):
+        scale = np.abs(gr[k]).max()
+        err = np.abs(g[k] - gr[k]) - (1e-4 * np.abs(gr[k]) + floor * scale)
+        assert err.max() <= 0.0, (k, float(err.max()), scale)
+
+
 def _bf16(x):
     """Round to BF16 (nearest, ties to even) through FP32, as the device packs FP32 values."""
     f = np.ascontiguousarray(np.asarray(x, np.float64).astype(np.float32))
