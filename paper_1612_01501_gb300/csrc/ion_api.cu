@@ -319,55 +319,6 @@ void ion_csr_fill(const ion_sim *s, CsrArgs &a, bool staged) {
     a.w = s->d_w;
     a.g = s->g;
     a.col16 = csr_use16(s, staged) ? s->d_col16 : nullptr;
-    if (staged && s->d_col16p && a.col16 && s->pad_rows == s->csr_chunk_rows) {
-        a.col16p = s->d_col16p;
-        a.wp = s->d_wp;
-        a.segoff = s->d_segoff;
-    }
-}
-
-// The staged kernel's padded layout (see ion_sim): segment offsets on the host from the row
-// pointers and chunk boundaries, the columns and weights by a fill kernel.
-static ion_status build_padded_layout(ion_sim *s) {
-    const int n = s->n, C = s->n_chunks, rows = s->csr_chunk_rows;
-    std::vector<int32_t> rp((size_t)n + 1), mid((size_t)(C - 1) * n);
-    cudaError_t e = cudaMemcpyAsync(rp.data(), s->d_rowptr, rp.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, s->st);
-    if (e == cudaSuccess && C > 1)
-        e = cudaMemcpyAsync(mid.data(), s->d_mid, mid.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, s->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
-    if (e != cudaSuccess) return ion_fail(nullptr, ION_ERR_CUDA, "CSR padded layout: %s", cudaGetErrorString(e));
-    std::vector<int32_t> off((size_t)C * n + 1);
-    int64_t tot = 0;
-    for (int ch = 0; ch < C; ++ch)
-        for (int i = 0; i < n; ++i) {
-            const int64_t b = ch == 0 ? rp[i] : mid[(size_t)(ch - 1) * n + i];
-            const int64_t en = ch == C - 1 ? rp[i + 1] : mid[(size_t)ch * n + i];
-            off[(size_t)ch * n + i] = (int32_t)tot;
-            tot += (en - b + 7) & ~(int64_t)7;
-            if (tot >= INT32_MAX) return ION_OK;   // too large for 32-bit offsets: keep the unpadded layout
-        }
-    off[(size_t)C * n] = (int32_t)tot;
-    e = ion_alloc(&s->d_segoff, off.size() * sizeof(int32_t));
-    if (e == cudaSuccess) e = ion_alloc(&s->d_col16p, (size_t)std::max<int64_t>(tot, 8) * sizeof(uint16_t));
-    if (e == cudaSuccess && s->d_w) e = ion_alloc(&s->d_wp, (size_t)std::max<int64_t>(tot, 8) * sizeof(float));
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(s->d_segoff, off.data(), off.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s->st);
-    if (e == cudaSuccess)
-        e = launch_csr_pad_fill(s->d_rowptr, s->d_mid, s->d_col, s->d_w, n, C, rows, std::min(CSR_CHUNK, s->n_pad),
-                                s->d_segoff, s->d_col16p, s->d_wp, s->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);   // the host offsets are released on return
-    if (e != cudaSuccess) {
-        cudaFree(s->d_segoff);
-        cudaFree(s->d_col16p);
-        cudaFree(s->d_wp);
-        s->d_segoff = nullptr;
-        s->d_col16p = nullptr;
-        s->d_wp = nullptr;
-        return ion_fail(nullptr, e == cudaErrorMemoryAllocation ? ION_ERR_OOM : ION_ERR_CUDA, "CSR padded layout: %s",
-                        cudaGetErrorString(e));
-    }
-    s->pad_rows = rows;
-    return ION_OK;
 }
 
 ion_status ion_setup_csr_staging(ion_sim *s, int mode) {
@@ -377,8 +328,21 @@ ion_status ion_setup_csr_staging(ion_sim *s, int mode) {
     const bool on = mode == 2 || (mode == 0 && deg >= 64.0 && (csr_bytes > 96.0e6 || deg / chunks >= 32.0));
     s->csr_staged = 0;
     // staging relies on validated (sorted, in-range) columns: host-copied CSR only
-    // (the surrogate path computes its gap currents with the direct kernel)
-    if (!on || (s->flags & (ION_FLAG_SPLIT | ION_FLAG_SURROGATE)) || !s->own_csr || s->d_rev) return ION_OK;
+    if (!on || !s->own_csr || s->d_rev) return ION_OK;
+    // the compact layout runs the sliced kernel (which can also leave the currents to a
+    // separate update: SPLIT, SURROGATE); 32-bit columns, the bank order and layouts beyond
+    // 32-bit offsets the chunked one
+    if (s->d_col16 && !s->col16_bank) {
+        if (!s->sl.cols) {
+            const ion_status sp = ion_build_sliced(s, 0);
+            if (sp != ION_OK) return sp;
+        }
+        if (s->sl.cols) {
+            s->csr_staged = 1;
+            return ION_OK;
+        }
+    }
+    if (s->flags & (ION_FLAG_SPLIT | ION_FLAG_SURROGATE)) return ION_OK;
     s->n_chunks = (s->n_pad + CSR_CHUNK - 1) / CSR_CHUNK;
     int rows = (s->n + s->sms - 1) / s->sms;
     if (rows > 1024) rows = 1024;
@@ -394,19 +358,18 @@ ion_status ion_setup_csr_staging(ion_sim *s, int mode) {
             return ion_fail(nullptr, e == cudaErrorMemoryAllocation ? ION_ERR_OOM : ION_ERR_CUDA, "CSR staging setup: %s",
                             cudaGetErrorString(e));
     }
-    // The padded layout removes each segment's head and tail (up to 14 edges handled one by
-    // one); measured, it pays for segments of up to ~1000 edges with the exponential
-    // junction and at every length with the linear one, while exponential-junction rows of
-    // several thousand edges per chunk ran 4-9 % slower on it: those keep the unpadded layout.
-    const bool pad = (s->flags & ION_FLAG_SGJ) || deg / s->n_chunks <= 1024.0;
-    if (pad && s->d_col16 && !s->col16_bank && !s->d_col16p) {
-        const ion_status sp = build_padded_layout(s);
-        if (sp != ION_OK) return sp;
-    }
     const ion_status st = ion_prepare_csr_chunk(s);
     if (st != ION_OK) return st;
     s->csr_staged = 1;
     return ION_OK;
+}
+
+// The CSR step of the handle's layout: sliced, chunked or direct.
+cudaError_t ion_launch_csr(const ion_sim *s, const CsrArgs &a) {
+    if (s->csr_staged == 1)
+        return s->sl.cols ? launch_csr_sliced_step(a, s->sl, s->st)
+                          : launch_csr_chunk_step(a, s->csr_chunk_SW, s->csr_chunk_rows, s->d_mid, s->n_chunks, false, s->st);
+    return launch_csr_step(a, s->csr_SW, s->csr_rows, s->st);
 }
 
 // Allow the staged kernel of the current lanes-per-row choice its dynamic shared memory.
@@ -494,9 +457,7 @@ void ion_sim_free_device(ion_sim *s) {
     s->d_split = s->d_rev = nullptr;
     s->d_slot = s->d_icu = nullptr;
     cudaFree(s->d_mid);
-    cudaFree(s->d_col16p);
-    cudaFree(s->d_wp);
-    cudaFree(s->d_segoff);
+    ion_free_sliced(s);
     cudaFree(s->d_mlp);
     cudaFree(s->d_mlp_tc);
     s->d_mlp_tc = nullptr;
@@ -880,16 +841,13 @@ static cudaError_t enqueue_one_step(ion_sim *s, int k_off, const float *iapp) {
             // the compact CSR kernels with the linear term where the network has 16-bit
             // columns (staged or not, as for the exponential junction), else eight lanes
             // per row over the 32-bit columns
-            const bool staged = s->csr_staged == 1 && !split;
             CsrArgs a{};
             a.c = c;
-            ion_csr_fill(s, a, staged);
+            ion_csr_fill(s, a, s->csr_staged == 1);
             if (a.col16 != nullptr && !split) {
                 a.lin = 1;
                 a.fuse = 1;
-                e = staged ? launch_csr_chunk_step(a, s->csr_chunk_SW, s->csr_chunk_rows, s->d_mid, s->n_chunks, false,
-                                                   s->st)
-                           : launch_csr_step(a, s->csr_SW, s->csr_rows, s->st);
+                e = ion_launch_csr(s, a);
             } else {
                 a.col16 = nullptr;
                 e = launch_sgj_csr_step(a, s->st);
@@ -926,14 +884,11 @@ static cudaError_t enqueue_one_step(ion_sim *s, int k_off, const float *iapp) {
     } else if (s->kind == ION_CSR) {
         CsrArgs a{};
         a.c = c;
-        ion_csr_fill(s, a, s->csr_staged == 1 && !split);
+        ion_csr_fill(s, a, s->csr_staged == 1);
         a.fuse = split ? 0 : 1;
         a.ic_out = s->d_ic;
         a.vd_in = nullptr;
-        if (s->csr_staged == 1 && !split)
-            e = launch_csr_chunk_step(a, s->csr_chunk_SW, s->csr_chunk_rows, s->d_mid, s->n_chunks, false, s->st);
-        else
-            e = launch_csr_step(a, s->csr_SW, s->csr_rows, s->st);
+        e = ion_launch_csr(s, a);
         s->launches++;
         if (e == cudaSuccess && split) {
             CellArgs ca{c, s->d_ic, s->d_cellp};

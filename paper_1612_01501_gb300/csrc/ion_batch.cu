@@ -1193,18 +1193,24 @@ extern "C" ion_status ion_autotune(ion_sim *s, int32_t steps, ion_tune *chosen) 
         int bsw = s->csr_SW, brows = s->csr_rows, bstaged = s->csr_staged;
         int b_csw = s->csr_chunk_SW;
         const int sw0 = s->csr_SW;
+        int sl0 = 0;   // the sliced layout's own choice of lanes per row
         for (int staged = 0; staged <= 1 && st == ION_OK; ++staged) {
             if (staged) {
                 if (ion_setup_csr_staging(s, 2) != ION_OK || s->csr_staged == 0) break;
+                if (s->sl.cols) sl0 = 1 << s->sl.lsw;
             } else {
                 s->csr_staged = 0;
             }
             const int mode = s->csr_staged;
             for (int sw : SWs) {
-                if (sw * 4 < sw0 || sw > sw0 * 4) continue;   // near the degree-based choice
+                if (sl0 ? (sw * 2 < sl0 || sw > sl0 * 2) : (sw * 4 < sw0 || sw > sw0 * 4)) continue;   // near the default
                 for (int r : rows) {
                     if (staged && r != rows[0]) continue;     // staged: rows per CTA fixed by the SM count
-                    if (staged) {
+                    if (sl0) {   // the layout holds the lanes per row: built again
+                        s->csr_chunk_SW = sw;
+                        st = sw == 1 << s->sl.lsw ? ION_OK : ion_build_sliced(s, sw);
+                        if (st != ION_OK) break;
+                    } else if (staged) {
                         s->csr_chunk_SW = sw;
                         st = ion_prepare_csr_chunk(s);
                         if (st != ION_OK) break;
@@ -1232,8 +1238,11 @@ extern "C" ion_status ion_autotune(ion_sim *s, int32_t steps, ion_tune *chosen) 
         s->csr_rows = brows;
         s->csr_staged = bstaged;
         s->csr_chunk_SW = b_csw;
+        if (sl0 && st == ION_OK && (!bstaged || b_csw != 1 << s->sl.lsw))
+            st = ion_build_sliced(s, bstaged ? b_csw : sl0);   // the best lanes (or the default) again
+        if (sl0 && !s->sl.cols) s->csr_staged = 0;   // a failed rebuild: the direct kernel
         bt.csr_lanes_per_row = bstaged ? b_csw : bsw;
-        bt.csr_rows_per_cta = bstaged ? s->csr_chunk_rows : brows;
+        bt.csr_rows_per_cta = bstaged ? (sl0 ? s->sl.rows : s->csr_chunk_rows) : brows;
         bt.csr_staging = bstaged ? 2 : 1;
     }
     ion_drop_graphs(s);

@@ -262,10 +262,19 @@ struct CsrArgs {
     float *ic_out;
     const float *vd_in;
     int32_t lin;          // 1: linear junctions (SGJ use case); needs col16
-    // staged kernel, padded layout (see ion_sim): columns, weights, segment offsets
-    const uint16_t *col16p;
-    const float *wp;
-    const int32_t *segoff;
+};
+// The sliced layout of the staged CSR kernel (ion_csr_sliced.cu)
+struct SliceLayout {
+    const uint4 *cols;       // NULL: no such layout; per round 32 lanes x 8 columns
+    const float4 *w;         // NULL, or per round 2 x 32 lanes x 4 weights
+    const int32_t *off;      // first round of each slice, slices in (chunk, CTA, slice) order, and the end
+    const uint16_t *rowid;   // 32 / SW rows of each slice (within the CTA; 0xFFFF: none)
+    int32_t rows;            // rows per CTA (a multiple of 4)
+    int32_t lsw;             // log2 of the lanes per row
+    int32_t nsl;             // slices per (chunk, CTA)
+    int32_t n_chunks, chunk; // V_dend chunks and floats per chunk
+    int32_t nbuf;            // chunk buffers in shared memory
+    int32_t stage;           // 1: the rows' state words are staged in shared memory
 };
 struct PersistArgs {
     StepCommon c;         // k_off unused: the launch runs steps *t_dev .. *t_dev + n_steps - 1
@@ -321,9 +330,7 @@ cudaError_t launch_sgj_csr_step(const CsrArgs &a, cudaStream_t st);
 cudaError_t launch_csr_col16(const int32_t *col, int64_t nnz, int64_t n_alloc, uint16_t *col16, cudaStream_t st);
 cudaError_t launch_csr_half_step(const CsrArgs &a, int lanes_per_row, int rows_per_cta, const int32_t *split,
                                  const int32_t *rev, float *slot, float *icu, cudaStream_t st);
-cudaError_t launch_csr_pad_fill(const int32_t *row_ptr, const int32_t *mid, const int32_t *col, const float *w,
-                                 int32_t n, int n_chunks, int rows, int nb, const int32_t *off, uint16_t *col16p,
-                                 float *wp, cudaStream_t st);
+cudaError_t launch_csr_sliced_step(const CsrArgs &a, const SliceLayout &L, cudaStream_t st);
 cudaError_t launch_csr_chunk_bounds(const int32_t *row_ptr, const int32_t *col, int32_t n, int n_chunks,
                                     int32_t *mid, cudaStream_t st);
 size_t csr_chunk_smem_bytes(int n_pad, int rows);

@@ -932,10 +932,10 @@ static cudaError_t surrogate_step(ion_sim *s, int k_off, const float *iapp) {
     } else if (s->kind == ION_CSR) {
         CsrArgs a{};
         a.c = c;
-        ion_csr_fill(s, a, false);
+        ion_csr_fill(s, a, s->csr_staged == 1);
         a.fuse = 0;
         a.ic_out = s->d_ic;
-        e = launch_csr_step(a, s->csr_SW, s->csr_rows, s->st);
+        e = ion_launch_csr(s, a);
         s->launches++;
     }
     if (e != cudaSuccess) return e;
@@ -957,6 +957,5 @@ ion_status ion_setup_surrogate(ion_sim *s, const ion_params *p) {
     }
     s->step_override = surrogate_step;
     s->lps = s->kind == ION_NO_GJ ? 1 : 2;
-    s->csr_staged = 0;
     return ION_OK;
 }

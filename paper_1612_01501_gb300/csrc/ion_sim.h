@@ -71,14 +71,8 @@ struct ion_sim {
     int csr_staged = 0;             // 1: V_dend staged in shared memory chunk by chunk
     int csr_chunk_SW = 32, csr_chunk_rows = 0, n_chunks = 1;
     int32_t *d_mid = nullptr;       // interior chunk boundaries per row
-    // the staged kernel's padded layout: each (chunk, row) segment's columns chunk-relative
-    // and padded to whole 16-byte groups with entries that index the row's own V_dend
-    // (a pair with dV = 0 adds exactly 0); segments in chunk-major order from d_segoff
-    uint16_t *d_col16p = nullptr;
-    float *d_wp = nullptr;
-    int32_t *d_segoff = nullptr;
-    int32_t pad_rows = 0;           // rows per CTA the padding entries are numbered for
-    bool col16_bank = false;        // col16 holds the opt-in bank order (no padded layout)
+    ion::SliceLayout sl{};          // the staged kernel's sliced layout (cols NULL: the chunked kernel runs)
+    bool col16_bank = false;        // col16 holds the opt-in bank order (no sliced layout)
     // half-work CSR (ION_FLAG_HALF_WORK on a CSR network): first upper edge of each row, the
     // mirrored position of every upper edge, the per-edge slots, the rows' upper sums
     int32_t *d_split = nullptr, *d_rev = nullptr;
@@ -116,7 +110,10 @@ inline cudaError_t ion_alloc(T **p, size_t bytes) {
 
 // shared helpers (ion_api.cu)
 void ion_csr_fill(const ion_sim *s, ion::CsrArgs &a, bool staged);
+cudaError_t ion_launch_csr(const ion_sim *s, const ion::CsrArgs &a);
 ion_status ion_prepare_csr_chunk(ion_sim *s);
+ion_status ion_build_sliced(ion_sim *s, int lanes);   // ion_csr_sliced.cu (lanes per row, 0: choose)
+void ion_free_sliced(ion_sim *s);
 ion_status ion_fail(ion_sim *s, ion_status code, const char *fmt, ...);
 ion::ModelF ion_model_to_f32(const ion_model &m, double dt);
 ion_status ion_cell_params_to_f32(const float *cp, int32_t n, const ion_model &m, double dt, std::vector<float> &out);
