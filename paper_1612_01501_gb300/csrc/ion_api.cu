@@ -596,9 +596,9 @@ extern "C" ion_status ion_create(const ion_net *net, const ion_conn *conn, const
             e = cudaMemcpy2DAsync(s->d_W, (size_t)s->n_pad * sizeof(float), conn->weight, (size_t)s->n * sizeof(float),
                                   (size_t)s->n * sizeof(float), (size_t)s->n,
                                   conn->mem == ION_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s->st);
-        if (e == cudaSuccess) e = prepare_matrix_step(s->n_pad);
+        if (e == cudaSuccess) e = prepare_matrix_step();
         if (e != cudaSuccess) return fail(ion_fail(nullptr, ION_ERR_CUDA, "ion_create: matrix copy: %s", cudaGetErrorString(e)));
-        s->dense_R = matrix_default_R(s->n, sms);
+        s->dense_R = 4;
         const ion_tune *tu = (const ion_tune *)params->tune;
         if (tu && tu->dense_rows_per_warp > 0) s->dense_R = tu->dense_rows_per_warp;
         if (s->dense_R != 1 && s->dense_R != 2 && s->dense_R != 4)
@@ -829,7 +829,7 @@ static cudaError_t enqueue_one_step(ion_sim *s, int k_off, const float *iapp) {
         MatrixArgs a{};
         a.c = c;
         a.W = s->d_W;
-        e = launch_matrix_step(a, s->dense_R, s->st);
+        e = launch_matrix_step(a, s->dense_R, s->sms, s->st);
         s->launches++;
         return e;
     }

@@ -570,17 +570,25 @@ cudaError_t launch_csr_col16(const int32_t *col, int64_t nnz, int64_t n_alloc, u
 }
 
 // ---- stand-alone cell update (no gap junctions, or Ic computed by another launch) ----
+// Bound by memory once the state is larger than L2 (132 bytes per cell and step, 12 more with
+// pulses).  The CTAs walk the cells in opposite directions on even and odd steps: the cells a
+// step ends with are still in L2 when the next begins with them, so up to L2's worth of the
+// state is neither read from nor written back to HBM.  2^21 cells with
+// pulses on a fifth: 46.8 us per step (0.92 of the measured copy rate in the bytes above), 53.6
+// in one direction only, 61.8 before with the pulse table read after the state
 __global__ void __launch_bounds__(256) cell_step_kernel(const CellArgs a) {
-    pdl_enter();
     const StepCommon &c = a.c;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t b = c.par == 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const int64_t i = b * blockDim.x + threadIdx.x;
+    const PulseAhead pa = pulse_ahead(c.pulses, i, i < c.n);
+    pdl_enter();
     if (i >= c.n) return;
     const int64_t t = step_index(c);
     const float *vcur = vd_cur(c);
     float *vnext = vd_next(c);
     const Cell cell = load_cell(c.S, vcur, i);
     const float ic = a.ic != nullptr ? a.ic[i] : 0.0f;
-    float iapp = pulse_current(c.pulses, i, t);
+    float iapp = pulse_current(c.pulses, pa, t);
     if (c.iapp != nullptr) iapp += c.iapp[i];
     const CellNext o = a.cellp != nullptr ? cell_step(cell_model(c.P, a.cellp, c.S.stride, i), cell, ic, iapp)
                                           : cell_step(c.P, cell, ic, iapp);

@@ -320,9 +320,9 @@ cudaError_t launch_csr_step(const CsrArgs &a, int lanes_per_row, int rows_per_ct
 cudaError_t prepare_csr_step();
 cudaError_t launch_csr_chunk_step(const CsrArgs &a, int lanes_per_row, int rows_per_cta, const int32_t *mid,
                                   int n_chunks, bool prepare, cudaStream_t st);
-cudaError_t prepare_matrix_step(int n_pad);
-cudaError_t launch_matrix_step(const MatrixArgs &a, int R, cudaStream_t st);   // R: rows per warp, 1, 2 or 4
-int matrix_default_R(int n, int sms);
+cudaError_t prepare_matrix_step();
+// R: rows whose weights a warp has in flight, 1, 2 or 4
+cudaError_t launch_matrix_step(const MatrixArgs &a, int R, int sms, cudaStream_t st);
 int sgj_partials(int n);   // CTAs of the SGJ partial-sum launch (the update reads that many)
 constexpr int SGJ_ONE_LAUNCH = 16384;   // SGJ dense networks up to this size take one launch per step
 cudaError_t launch_sgj_dense_step(const StepCommon &c, float g, float *part, cudaStream_t st);
