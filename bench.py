@@ -843,7 +843,8 @@ def main():
                 "traffic": None,
                 # staged 16-bit columns run the sliced kernel, 32-bit ones the chunked one
                 "kernel": ("csr_sliced_step_kernel" if lay["index_bytes"] == 2 else "csr_chunk_step_kernel")
-                          if lay["staged"] else "csr_step_kernel",
+                          if lay["staged"] else ("csr_direct_step_kernel" if lay["index_bytes"] == 2 or nnz < 32 * n
+                                                 else "csr_step_kernel"),
                 "algorithmic_bytes_per_timestep": bytes_step,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs", "us_per_timestep": per_step_s * 1e6,
                 "note": "working set fits in L2 (129 MB)" if bytes_step < 100e6 else "streams from HBM",

@@ -210,9 +210,10 @@ typedef struct {
     int32_t csr_rows_per_cta;    /* rows per CTA of 256 threads, 1..256             */
     int32_t csr_lanes_scale;     /* batches: 0 = lanes per row from each network's
                                     mean degree, +1 = twice that, -1 = half        */
-    int32_t csr_staging;         /* single CSR networks: 0 = choose (stage when the
-                                    mean degree is 64 or more and at least 32 per
-                                    chunk, or the CSR exceeds 96 MB), 1 = gather V_dend
+    int32_t csr_staging;         /* single CSR networks: 0 = choose (from the cells, the
+                                    edges and the chunks V_dend would take; always
+                                    when the CSR exceeds 96 MB with rows of 64 or
+                                    more edges), 1 = gather V_dend
                                     through L1/L2, 2 = stage V_dend in shared memory,
                                     whole or in chunks (one CTA per SM)              */
     int32_t csr_bank_order;      /* single CSR networks with equal weights: 1 = store the

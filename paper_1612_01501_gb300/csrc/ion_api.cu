@@ -293,17 +293,38 @@ void ion_choose_csr_shape(double mean_deg, int *SW, int *rows) {
     *rows = r;
 }
 
+// The direct kernel: about four edges per lane (what it reads ahead of the step), and as many
+// rows per CTA as keep every CTA of the grid resident at once (up to 3.5 per SM), since a
+// second wave pays the whole chain of latencies again: 65 536 cells, k = 10: 5.6 us per step
+// with 128 rows per CTA, 6.5 with 64, 6.9 with 256; k = 24: 8.7 / 9.0.
+void ion_choose_direct_shape(int32_t n, double mean_deg, int sms, int *SW, int *rows) {
+    int sw = 1;
+    while (sw < 32 && 4 * sw < mean_deg) sw *= 2;
+    int r = 256 / sw;
+    while (r < 256 && (double)n / r > 3.5 * sms) r *= 2;
+    *SW = sw;
+    *rows = r;
+}
+
 // Shared-memory staging of V_dend for a CSR network (mode 0: choose, 1: off, 2: on).
-// Staging pays when rows are long: a warp's 32 random gathers then cost about 3.8
-// shared-memory wavefronts instead of 32 L1 lines.  Measured: the 65 536-cell network at
-// k = 1000 went from 0.45 to 0.69 of HBM bandwidth (32-bit columns), k = 100 from 20.6 to
-// 16.9 us per step (16-bit columns), and random networks of 10 000-13 000 cells at 25-50 %
-// density ran about twice as fast staged.  The default stages rows of 64 or more edges that
-// keep 32 or more per chunk, or any CSR too large for L2 (over 96 MB) with rows of 64 or
-// more edges; rows of ~10 edges stay on the direct kernel.  One CTA per SM owns ceil(n / SMs) rows (at most
-// 1024).  Only
-// CSR arrays copied from the host are staged: their columns were checked to be sorted
-// and in range, which the chunk boundaries rely on.
+// The sliced kernel pays per chunk of V_dend (about 1.7 us: the copy, the slices' bookkeeping),
+// the direct kernel per edge (a 32-byte sector from L2, 4.4 us per million; 1.8 where V_dend
+// fits L1 beside the rest); us per step direct / staged: 2 000 cells, k = 200: 3.1 / 4.2;
+// 10 000: 4.1 / 4.2 (k = 40), 5.1 / 4.3 (64); 20 000: 3.7 / 4.4 (10), 6.4 / 4.6 (40); 40 000:
+// 5.3 / 4.9 (10), 7.7 / 5.0 (24); 65 536: 5.8 / 8.1 (10), 9.1 / 8.3 (24).  Only CSR
+// arrays copied from the host are staged: their columns were checked to be sorted and in
+// range, which the chunk boundaries rely on.  32-bit columns (CSR_AS_GIVEN) stage rows of 64 or
+// more edges that keep 32 or more per 128 KB chunk, or any CSR too large for L2 (over 96 MB)
+// with rows of 64 or more.
+static bool stage_by_default(const ion_sim *s, double deg, double csr_bytes) {
+    if (deg >= 64.0 && csr_bytes > 96.0e6) return true;
+    const double chunks = (double)((s->n_pad + CSR_CHUNK - 1) / CSR_CHUNK);
+    if (!s->d_col16 || s->col16_bank) return deg >= 64.0 && deg / chunks >= 32.0;
+    const SliceLayout L = ion_plan_sliced(s->n, s->n_pad, s->nnz, s->sms, 0);
+    const double waves = std::ceil((double)s->n / L.rows / s->sms);
+    const double staged = 2.5 + 1.7 * L.n_chunks * waves + 2.0e-5 * s->n, direct = 2.2 + (s->n <= 4000 ? 1.8e-6 : 4.4e-6) * (double)s->nnz;
+    return staged < direct;
+}
 // The 16-bit columns serve the staged kernel (columns relative to a chunk of at most 2^16
 // cells) and the direct kernel when n <= 65 536 and rows are long enough (mean degree >= 32)
 // for its eight-edge groups; shorter rows read 32-bit columns four at a time.
@@ -324,8 +345,7 @@ void ion_csr_fill(const ion_sim *s, CsrArgs &a, bool staged) {
 ion_status ion_setup_csr_staging(ion_sim *s, int mode) {
     const double deg = s->n > 0 ? (double)s->nnz / s->n : 0.0;
     const double csr_bytes = (double)((s->d_col16 ? 2 : 4) + (s->d_w ? 4 : 0)) * (double)s->nnz;
-    const double chunks = (double)((s->n_pad + CSR_CHUNK - 1) / CSR_CHUNK);
-    const bool on = mode == 2 || (mode == 0 && deg >= 64.0 && (csr_bytes > 96.0e6 || deg / chunks >= 32.0));
+    const bool on = mode == 2 || (mode == 0 && stage_by_default(s, deg, csr_bytes));
     s->csr_staged = 0;
     // staging relies on validated (sorted, in-range) columns: host-copied CSR only
     if (!on || !s->own_csr || s->d_rev) return ION_OK;
@@ -369,6 +389,9 @@ cudaError_t ion_launch_csr(const ion_sim *s, const CsrArgs &a) {
     if (s->csr_staged == 1)
         return s->sl.cols ? launch_csr_sliced_step(a, s->sl, s->st)
                           : launch_csr_chunk_step(a, s->csr_chunk_SW, s->csr_chunk_rows, s->d_mid, s->n_chunks, false, s->st);
+    // 16-bit columns, linear junctions and short rows; long rows of 32-bit columns take 16-byte loads
+    if (a.col16 != nullptr || a.lin || s->nnz < 32 * (int64_t)s->n)
+        return launch_csr_direct_step(a, s->csr_SW, s->csr_rows, s->st);
     return launch_csr_step(a, s->csr_SW, s->csr_rows, s->st);
 }
 
@@ -657,7 +680,10 @@ extern "C" ion_status ion_create(const ion_net *net, const ion_conn *conn, const
             if (hs != ION_OK) return fail(hs);
         }
         int SW, rows;
-        ion_choose_csr_shape((double)s->nnz / s->n, &SW, &rows);
+        if (!s->d_rev && (csr_use16(s, false) || (s->flags & ION_FLAG_SGJ) || s->nnz < 32 * (int64_t)s->n))
+            ion_choose_direct_shape(s->n, (double)s->nnz / s->n, sms, &SW, &rows);
+        else
+            ion_choose_csr_shape((double)s->nnz / s->n, &SW, &rows);
         const ion_tune *tu = (const ion_tune *)params->tune;
         if (tu && tu->csr_lanes_per_row > 0) SW = tu->csr_lanes_per_row;
         if (tu && tu->csr_rows_per_cta > 0) rows = tu->csr_rows_per_cta;
@@ -838,20 +864,14 @@ static cudaError_t enqueue_one_step(ion_sim *s, int k_off, const float *iapp) {
             e = launch_sgj_dense_step(c, s->g, s->d_sgj, s->st);
             s->launches += s->lps;
         } else {
-            // the compact CSR kernels with the linear term where the network has 16-bit
-            // columns (staged or not, as for the exponential junction), else eight lanes
-            // per row over the 32-bit columns
             CsrArgs a{};
             a.c = c;
             ion_csr_fill(s, a, s->csr_staged == 1);
-            if (a.col16 != nullptr && !split) {
-                a.lin = 1;
-                a.fuse = 1;
-                e = ion_launch_csr(s, a);
-            } else {
-                a.col16 = nullptr;
-                e = launch_sgj_csr_step(a, s->st);
-            }
+            a.lin = 1;
+            a.fuse = 1;
+            // the chunked kernel has the linear term on 16-bit columns only
+            const bool chunked32 = s->csr_staged == 1 && !s->sl.cols && a.col16 == nullptr;
+            e = chunked32 ? launch_csr_direct_step(a, s->csr_SW, s->csr_rows, s->st) : ion_launch_csr(s, a);
             s->launches++;
         }
         return e;

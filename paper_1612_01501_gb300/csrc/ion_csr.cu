@@ -21,11 +21,11 @@
 namespace ion {
 
 // One CTA of 256 threads owns `rows` consecutive rows (rows <= 256).  Phase 1: groups of
-// SW lanes take the rows round-robin; phase 2: thread t updates row t.  LIN: linear
-// junctions (the SGJ use case), on the 16-bit column layout only.
-template <int SW, bool VEC, bool HAS_W, bool C16, bool LIN = false>
+// SW lanes take the rows round-robin; phase 2: thread t updates row t.  For 32-bit columns in
+// long rows (16-byte loads of four) and the stand-alone primitive; short rows and 16-bit
+// columns run csr_direct_step_kernel.
+template <int SW, bool VEC, bool HAS_W>
 __global__ void __launch_bounds__(256) csr_step_kernel(const CsrArgs a, int rows) {
-    static_assert(!LIN || C16, "linear junctions run on the 16-bit column layout");
     __shared__ float ic_s[256];
     pdl_enter();
     const StepCommon &c = a.c;
@@ -56,12 +56,8 @@ __global__ void __launch_bounds__(256) csr_step_kernel(const CsrArgs a, int rows
         const float vi = vin;
         bounds(it + 1, e0n, e1n, vin);
         float acc = 0.0f;
-        if (e1 > e0) {   // rows past the end (and empty rows) have e0 == e1
-            if (C16)
-                acc = csr_row_sum16<SW, HAS_W, false, LIN>(a.col16, a.w, e0, e1, vi, li, VjGlobal{vcur});
-            else
-                acc = csr_row_sum<SW, VEC, HAS_W>(vcur, a.col, a.w, e0, e1, vi, li);
-        }
+        if (e1 > e0)   // rows past the end (and empty rows) have e0 == e1
+            acc = csr_row_sum<SW, VEC, HAS_W>(vcur, a.col, a.w, e0, e1, vi, li);
 #pragma unroll
         for (int off = SW / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
         if (li == 0 && rr < rows) ic_s[rr] = (HAS_W ? acc : acc * a.g) * (1.0f / GJ_SCALE);
@@ -82,20 +78,13 @@ __global__ void __launch_bounds__(256) csr_step_kernel(const CsrArgs a, int rows
     finish_cell(c, t, vnext, i, o);
 }
 
-template <int SW, bool VEC, bool HAS_W, bool C16 = false, bool LIN = false>
+template <int SW, bool VEC, bool HAS_W>
 static cudaError_t launch_csr_T(const CsrArgs &a, int rows, cudaStream_t st) {
     const int grid = (a.c.n + rows - 1) / rows;
-    return launch_k(csr_step_kernel<SW, VEC, HAS_W, C16, LIN>, dim3(grid), dim3(256), 0, st, a.c.pdl != 0, a, rows);
+    return launch_k(csr_step_kernel<SW, VEC, HAS_W>, dim3(grid), dim3(256), 0, st, a.c.pdl != 0, a, rows);
 }
 template <int SW>
 static cudaError_t launch_csr_SW(const CsrArgs &a, int rows, cudaStream_t st) {
-    if (a.lin) {
-        if (a.col16 == nullptr) return cudaErrorInvalidValue;
-        return a.w != nullptr ? launch_csr_T<SW, true, true, true, true>(a, rows, st)
-                              : launch_csr_T<SW, true, false, true, true>(a, rows, st);
-    }
-    if (a.col16 != nullptr)   // 16-byte aligned indices (and weights, checked at creation)
-        return a.w != nullptr ? launch_csr_T<SW, true, true, true>(a, rows, st) : launch_csr_T<SW, true, false, true>(a, rows, st);
     const bool vec = ((uintptr_t)a.col % 16 == 0) && (a.w == nullptr || (uintptr_t)a.w % 16 == 0);
     if (a.w != nullptr) return vec ? launch_csr_T<SW, true, true>(a, rows, st) : launch_csr_T<SW, false, true>(a, rows, st);
     return vec ? launch_csr_T<SW, true, false>(a, rows, st) : launch_csr_T<SW, false, false>(a, rows, st);
@@ -118,14 +107,10 @@ cudaError_t launch_csr_step(const CsrArgs &a, int SW, int rows, cudaStream_t st)
 // Prefer L1 over shared memory for the V_dend gathers (the kernel uses 1 KB of shared).
 template <int SW>
 static void carveout_SW() {
-    cudaFuncSetAttribute(csr_step_kernel<SW, true, true, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    cudaFuncSetAttribute(csr_step_kernel<SW, false, true, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    cudaFuncSetAttribute(csr_step_kernel<SW, true, false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    cudaFuncSetAttribute(csr_step_kernel<SW, false, false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    cudaFuncSetAttribute(csr_step_kernel<SW, true, true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    cudaFuncSetAttribute(csr_step_kernel<SW, true, false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    cudaFuncSetAttribute(csr_step_kernel<SW, true, true, true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    cudaFuncSetAttribute(csr_step_kernel<SW, true, false, true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    cudaFuncSetAttribute(csr_step_kernel<SW, true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    cudaFuncSetAttribute(csr_step_kernel<SW, false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    cudaFuncSetAttribute(csr_step_kernel<SW, true, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    cudaFuncSetAttribute(csr_step_kernel<SW, false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
 }
 cudaError_t prepare_csr_step() {
     carveout_SW<1>();
@@ -135,6 +120,126 @@ cudaError_t prepare_csr_step() {
     carveout_SW<16>();
     carveout_SW<32>();
     return cudaGetLastError();
+}
+
+// ---- the direct step: V_dend gathered through L1 / L2 ---------------------------------------
+// Where it runs (short rows, small networks) a step is a few dependent memory latencies long,
+// so everything that does not change between steps (the row's bounds, its first SHORT_E columns
+// and weights per lane, its pulse) is read before the wait on the previous step; after it the
+// V_dend gathers and the rows' state words (cp.async) go out together.  256 threads, SW lanes
+// per row, four gathers in flight per lane; then one thread per row runs the update.  C16:
+// 16-bit columns.  LIN: linear junctions, w (V_i - V_j).
+// 65 536 cells, k = 10: 5.6 us per step (4 lanes, 128 rows per CTA); the kernel that read
+// bounds, columns, gathers, state and pulses one after the other took 9.5 (7.1 tuned).
+constexpr int SHORT_E = 4;
+
+template <int SW, bool HAS_W, bool LIN, bool C16>
+__global__ void __launch_bounds__(256) csr_direct_step_kernel(const CsrArgs a, int rows) {
+    extern __shared__ __align__(16) float sh_smem[];
+    float *ic_s = sh_smem, *cs = sh_smem + 256;
+    const StepCommon &c = a.c;
+    const int n = c.n, row0 = blockIdx.x * rows;
+    const int sub = threadIdx.x / SW, li = threadIdx.x % SW;
+    constexpr int NSUB = 256 / SW;
+    uint32_t e = 0, e1 = 0;   // unsigned: the look-ahead below may pass 2^31
+    int j[SHORT_E];
+    float w[HAS_W ? SHORT_E : 1];
+    auto column = [&](uint32_t q) { return C16 ? (int)__ldg(a.col16 + q) : __ldg(a.col + q); };
+    auto columns = [&]() {      // SHORT_E columns and weights from e on
+#pragma unroll
+        for (int k = 0; k < SHORT_E; ++k)
+            if (e + k * SW < e1) {
+                j[k] = column(e + k * SW);
+                if (HAS_W) w[k] = __ldg(a.w + e + k * SW);
+            }
+    };
+    auto head = [&](int rr) {   // bounds, first columns and weights of row rr of the CTA
+        const int i = row0 + rr;
+        e = e1 = 0;
+        if (rr < rows && i < n) {
+            e = (uint32_t)__ldg(a.row_ptr + i) + li;
+            e1 = (uint32_t)__ldg(a.row_ptr + i + 1);
+        }
+        columns();
+    };
+    auto edge = [&](float vi, float vj, float wt) {
+        if (LIN) return HAS_W ? wt * (vi - vj) : vi - vj;
+        return gj_edge(vi, vj, wt);
+    };
+    head(sub);
+    const int mine = threadIdx.x;
+    const bool has_row = mine < rows && row0 + mine < n;
+    const PulseAhead pa = pulse_ahead(c.pulses, row0 + mine, has_row && a.fuse);
+    pdl_enter();
+    const int64_t t = step_index(c);
+    const float *vcur = vd_cur(c);
+    if (a.fuse && has_row) {
+#pragma unroll
+        for (int q = 0; q < NCW; ++q)
+            cp_async4(cs + q * rows + mine, (q == 0 ? vcur : c.S.f(cell_word_field(q))) + row0 + mine);
+    }
+    cp_async_commit();
+    for (int rr = sub; rr - sub < rows; rr += NSUB) {   // the same trip count in every lane
+        if (rr != sub) head(rr);
+        const int i = row0 + rr;
+        const float vi = rr < rows && i < n ? vcur[i] : 0.0f;
+        float acc = 0.0f;
+        while (e < e1) {
+            float v[SHORT_E];
+#pragma unroll
+            for (int k = 0; k < SHORT_E; ++k)
+                if (e + k * SW < e1) v[k] = __ldg(vcur + j[k]);
+#pragma unroll
+            for (int k = 0; k < SHORT_E; ++k)
+                if (e + k * SW < e1) acc += edge(vi, v[k], HAS_W ? w[k] : 1.0f);
+            e += SHORT_E * SW;
+            columns();
+        }
+#pragma unroll
+        for (int off = SW / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (li == 0 && rr < rows) ic_s[rr] = (HAS_W ? acc : acc * a.g) * (LIN ? 1.0f : 1.0f / GJ_SCALE);
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    if (!has_row) return;
+    const int i = row0 + mine;
+    if (!a.fuse) {
+        a.ic_out[i] = ic_s[mine];
+        return;
+    }
+    float iapp = pulse_current(c.pulses, pa, t);
+    if (c.iapp != nullptr) iapp += c.iapp[i];
+    const CellNext o = cell_step(c.P, staged_cell(cs, rows, mine), ic_s[mine], iapp);
+    finish_cell(c, t, vd_next(c), i, o);
+}
+
+template <int SW, bool C16>
+static cudaError_t launch_direct_T(const CsrArgs &a, int rows, cudaStream_t st) {
+    const dim3 grid((a.c.n + rows - 1) / rows), block(256);
+    const size_t smem = (256 + (size_t)NCW * rows) * sizeof(float);
+    const bool pdl = a.c.pdl != 0;
+    if (a.lin)
+        return a.w != nullptr ? launch_k(csr_direct_step_kernel<SW, true, true, C16>, grid, block, smem, st, pdl, a, rows)
+                              : launch_k(csr_direct_step_kernel<SW, false, true, C16>, grid, block, smem, st, pdl, a, rows);
+    return a.w != nullptr ? launch_k(csr_direct_step_kernel<SW, true, false, C16>, grid, block, smem, st, pdl, a, rows)
+                          : launch_k(csr_direct_step_kernel<SW, false, false, C16>, grid, block, smem, st, pdl, a, rows);
+}
+template <int SW>
+static cudaError_t launch_direct_SW(const CsrArgs &a, int rows, cudaStream_t st) {
+    return a.col16 != nullptr ? launch_direct_T<SW, true>(a, rows, st) : launch_direct_T<SW, false>(a, rows, st);
+}
+// rows: rows per CTA (1..256); SW: lanes per row.
+cudaError_t launch_csr_direct_step(const CsrArgs &a, int SW, int rows, cudaStream_t st) {
+    if (rows < 1 || rows > 256) return cudaErrorInvalidValue;
+    switch (SW) {
+        case 1: return launch_direct_SW<1>(a, rows, st);
+        case 2: return launch_direct_SW<2>(a, rows, st);
+        case 4: return launch_direct_SW<4>(a, rows, st);
+        case 8: return launch_direct_SW<8>(a, rows, st);
+        case 16: return launch_direct_SW<16>(a, rows, st);
+        case 32: return launch_direct_SW<32>(a, rows, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 // ---- column-chunked variant: V_dend staged in shared memory -------------------------------
@@ -426,41 +531,6 @@ cudaError_t launch_sgj_dense_step(const StepCommon &c, float g, float *part, cud
                     (const float *)part, n_part, g);
 }
 int sgj_partials(int n) { return std::min(256, std::max(1, (n + 4095) / 4096)); }
-
-// CSR: eight lanes per row, 32 rows per CTA, then the cell update of the CTA's rows.
-__global__ void __launch_bounds__(256) sgj_csr_step_kernel(const CsrArgs a) {
-    __shared__ float ic_s[32];
-    pdl_enter();
-    const StepCommon &c = a.c;
-    const int64_t t = step_index(c);
-    const float *vcur = vd_cur(c);
-    float *vnext = vd_next(c);
-    const int sub = threadIdx.x >> 3, li = threadIdx.x & 7;
-    const int i = blockIdx.x * 32 + sub;
-    float acc = 0.0f;
-    if (i < c.n) {
-        const float vi = vcur[i];
-        for (int e = a.row_ptr[i] + li; e < a.row_ptr[i + 1]; e += 8) {
-            const float dv = vi - __ldg(vcur + __ldg(a.col + e));
-            acc = a.w != nullptr ? fmaf(__ldg(a.w + e), dv, acc) : acc + dv;
-        }
-    }
-#pragma unroll
-    for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (li == 0) ic_s[sub] = a.w != nullptr ? acc : acc * a.g;
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
-    const int r = blockIdx.x * 32 + threadIdx.x;
-    if (r >= c.n) return;
-    const Cell cell = load_cell(c.S, vcur, r);
-    float iapp = pulse_current(c.pulses, r, t);
-    if (c.iapp != nullptr) iapp += c.iapp[r];
-    const CellNext o = cell_step(c.P, cell, ic_s[threadIdx.x], iapp);
-    finish_cell(c, t, vnext, r, o);
-}
-cudaError_t launch_sgj_csr_step(const CsrArgs &a, cudaStream_t st) {
-    return launch_k(sgj_csr_step_kernel, dim3((a.c.n + 31) / 32), dim3(256), 0, st, a.c.pdl != 0, a);
-}
 
 // ---- half-work CSR (each stored pair evaluated once) ------------------------------------
 // The pair term is odd in dV and the weights are symmetric, so the term of the stored edge

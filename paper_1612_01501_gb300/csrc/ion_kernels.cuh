@@ -261,7 +261,7 @@ struct CsrArgs {
     int32_t fuse;
     float *ic_out;
     const float *vd_in;
-    int32_t lin;          // 1: linear junctions (SGJ use case); needs col16
+    int32_t lin;          // 1: linear junctions (SGJ use case); not in csr_step_kernel
 };
 // The sliced layout of the staged CSR kernel (ion_csr_sliced.cu)
 struct SliceLayout {
@@ -317,6 +317,7 @@ struct CellArgs {
 // launchers (return the CUDA launch status)
 cudaError_t launch_dense_step(const DenseArgs &a, int rows_per_warp, int warps, int col_splits, cudaStream_t st);
 cudaError_t launch_csr_step(const CsrArgs &a, int lanes_per_row, int rows_per_cta, cudaStream_t st);
+cudaError_t launch_csr_direct_step(const CsrArgs &a, int lanes_per_row, int rows_per_cta, cudaStream_t st);
 cudaError_t prepare_csr_step();
 cudaError_t launch_csr_chunk_step(const CsrArgs &a, int lanes_per_row, int rows_per_cta, const int32_t *mid,
                                   int n_chunks, bool prepare, cudaStream_t st);
@@ -326,7 +327,6 @@ cudaError_t launch_matrix_step(const MatrixArgs &a, int R, int sms, cudaStream_t
 int sgj_partials(int n);   // CTAs of the SGJ partial-sum launch (the update reads that many)
 constexpr int SGJ_ONE_LAUNCH = 16384;   // SGJ dense networks up to this size take one launch per step
 cudaError_t launch_sgj_dense_step(const StepCommon &c, float g, float *part, cudaStream_t st);
-cudaError_t launch_sgj_csr_step(const CsrArgs &a, cudaStream_t st);
 cudaError_t launch_csr_col16(const int32_t *col, int64_t nnz, int64_t n_alloc, uint16_t *col16, cudaStream_t st);
 cudaError_t launch_csr_half_step(const CsrArgs &a, int lanes_per_row, int rows_per_cta, const int32_t *split,
                                  const int32_t *rev, float *slot, float *icu, cudaStream_t st);

@@ -112,6 +112,7 @@ inline cudaError_t ion_alloc(T **p, size_t bytes) {
 void ion_csr_fill(const ion_sim *s, ion::CsrArgs &a, bool staged);
 cudaError_t ion_launch_csr(const ion_sim *s, const ion::CsrArgs &a);
 ion_status ion_prepare_csr_chunk(ion_sim *s);
+ion::SliceLayout ion_plan_sliced(int32_t n, int32_t n_pad, int64_t nnz, int sms, int lanes);
 ion_status ion_build_sliced(ion_sim *s, int lanes);   // ion_csr_sliced.cu (lanes per row, 0: choose)
 void ion_free_sliced(ion_sim *s);
 ion_status ion_fail(ion_sim *s, ion_status code, const char *fmt, ...);
