@@ -240,17 +240,18 @@ static int num_sms() {
 }
 
 // Dense: a CTA has W = GR x GJ warps (GR row groups of R rows, GJ column splits) and
-// owns GR * R rows.  Pick (R, GR, GJ) to minimise the work of the busiest SM,
-// ceil(grid / SMs) * (GR * R + 4): every row costs the same N pair evaluations and every
-// CTA pays about four rows' worth for staging and scaling its V_dend tiles.  Among equal
-// costs prefer 24..32 warps per CTA (the SFU pipe needs that many warps in flight; a
-// probe of the pair loop gave 0.44 / 0.67 / 0.77 of the ex2 peak at 9 / 18 / 32 warps),
-// then fewer rows per warp (a smaller register footprint).
+// owns GR * R rows.  Pick (R, GR, GJ) for the least modelled time of the busiest SM:
+// ceil(grid / SMs) * (GR * R + 8) rows' worth (every CTA pays about eight for its tile and its
+// tail), times 1 + 1 / (4 R) for a 16-byte column load and its transform shared by R rows, times
+// factors for too few warps to keep the SFU busy, for column splits and for the 768-thread
+// limit above R = 4.  Fitted to a sweep of all one- to three-wave shapes at 21 sizes from 64 to
+// 18 688 cells: the choice is within 0.9 % of the best on average, 4.6 % at worst.  us per
+// step, this choice / rows and warps alone as before: 1 003 cells 2.88 / 3.47; 2 999: 4.60 /
+// 4.64; 8 192: 12.4 / 12.7; 9 000: 15.4 / 15.6; 12 000: 22.6 / 22.9.
 void ion_choose_dense_shape(int n, int sms, int *R_out, int *W_out, int *GJ_out) {
     static const int Rs[] = {1, 2, 4, 6, 8};
     static const int GJs[] = {1, 2, 4};
-    long best_cost = -1;
-    int best_score = -1;
+    double best = -1.0;
     int bR = 1, bW = 1, bGJ = 1;
     for (int R : Rs)
         for (int GJ : GJs)
@@ -258,13 +259,12 @@ void ion_choose_dense_shape(int n, int sms, int *R_out, int *W_out, int *GJ_out)
                 const int W = GR * GJ;
                 if (W * 32 > dense_max_threads(R)) continue;
                 const long rows = (long)GR * R;
-                const long grid = (n + rows - 1) / rows;
-                const long cost = ((grid + sms - 1) / sms) * (rows + 4);
-                const int warps_score = (W >= 24) ? 3 : (W >= 16 ? 2 : (W >= 8 ? 1 : 0));
-                const int score = warps_score * 16 + (8 - R);
-                if (best_cost < 0 || cost < best_cost || (cost == best_cost && score > best_score)) {
-                    best_cost = cost;
-                    best_score = score;
+                const long waves = ((n + rows - 1) / rows + sms - 1) / sms;
+                const double few = W >= 24 ? 1.0 : (W >= 18 ? 1.02 : (W >= 12 ? 1.06 : (W >= 8 ? 1.1 : 1.4)));
+                const double split = GJ == 1 ? 1.0 : (GJ == 2 ? 0.97 : 1.06);
+                const double cost = (double)waves * (rows + 8) * (1.0 + 0.25 / R) * few * split * (R > 4 ? 1.06 : 1.0);
+                if (best < 0.0 || cost < best) {
+                    best = cost;
                     bR = R;
                     bW = W;
                     bGJ = GJ;

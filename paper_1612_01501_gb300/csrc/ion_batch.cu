@@ -145,7 +145,6 @@ __global__ void __launch_bounds__(256) batch_step_kernel(const BatchArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ float red_s[32], red_c[32];
-    __shared__ float U_sh;
     __shared__ float ic_s[256];
     pdl_enter();
 
@@ -166,27 +165,28 @@ __global__ void __launch_bounds__(256) batch_step_kernel(const BatchArgs a) {
         }
         __syncthreads();
         if (threadIdx.x == 0) issue_tile(sm, net_v, T.n_pad, 0, bar);
-        const float m_shift = net_v[0];
+        const float C = net_v[0] * GJ_SCALE;
         float ui[R];
         const int local0 = T.row0 - T.seg;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int li = local0 + warp * R + r;
-            ui[r] = (warp * R + r < T.rows) ? (net_v[li] - m_shift) * GJ_SCALE : 0.0f;
+            ui[r] = (warp * R + r < T.rows) ? gj_u(net_v[li], C) : 0.0f;
         }
         uint32_t uses[2] = {0u, 0u};
         float tot[R], Us, Uc;
-        if (!gj_pass<R, 1>(sm, net_v, T.n, T.n_pad, bar, uses, m_shift, ui, 0, lane, a.kahan, tot, Us, Uc)) {
+        if (!gj_pass<R, 1>(sm, net_v, T.n, T.n_pad, bar, uses, C, ui, 0, lane, a.kahan, tot, Us, Uc)) {
             if (threadIdx.x == 0) {
                 atomicOr(c.status, (uint32_t)ST_TIMEOUT);
                 (void)mbar_wait_bounded(&bar[0], uses[0] & 1u);
             }
             return;
         }
-        const float U = gj_reduce<R, 1>(sm, tot, Us, Uc, warp, 0, lane, red_s, red_c, &U_sh);
+        gj_reduce<R, 1>(sm, tot, Us, Uc, warp, 0, lane, red_s, red_c);
+        const float U = gj_sum_u(red_s, red_c);
         if ((int)threadIdx.x < T.rows) {
             const int rr = threadIdx.x;
-            ic_s[rr] = row_current<1>(sm, rr, (net_v[local0 + rr] - m_shift) * GJ_SCALE, T.n, U, T.g);
+            ic_s[rr] = row_current<1>(sm, rr, gj_u(net_v[local0 + rr], C), T.n, U, T.g);
         }
     } else if (T.mode & TILE_STAGE_V) {
         // the network's V_dend (n_pad <= TJ floats) in shared memory, 16-bit local columns
@@ -338,7 +338,6 @@ __global__ void __launch_bounds__(256, 4) batch_persist_kernel(const BatchPersis
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ float red_s[32], red_c[32];
-    __shared__ float U_sh;
     __shared__ float ic_s[256];
     __shared__ int ok_sh;
     float *vb = reinterpret_cast<float *>(smem_raw);   // the piece's network's V_dend(t)
@@ -393,22 +392,23 @@ __global__ void __launch_bounds__(256, 4) batch_persist_kernel(const BatchPersis
             }
             if (P.kind == TILE_DENSE) {
                 const DenseSmem sm{vb, P.n_pad, 1, part};
-                const float m_shift = vb[0];
+                const float C = vb[0] * GJ_SCALE;
                 for (int sub = 0; sub < P.rows; sub += 8 * R) {
                     const int local0 = P.row0 - P.seg + sub;
                     const int srows = min(8 * R, P.rows - sub);
                     float ui[R];
 #pragma unroll
                     for (int r = 0; r < R; ++r)
-                        ui[r] = (warp * R + r < srows) ? (vb[local0 + warp * R + r] - m_shift) * GJ_SCALE : 0.0f;
+                        ui[r] = (warp * R + r < srows) ? gj_u(vb[local0 + warp * R + r], C) : 0.0f;
                     uint32_t uses[2] = {0u, 0u};
                     float tot[R], Us, Uc;
-                    (void)gj_pass<R, 1>(sm, nullptr, P.n, P.n_pad, nullptr, uses, m_shift, ui, 0, lane, a.kahan, tot,
+                    (void)gj_pass<R, 1>(sm, nullptr, P.n, P.n_pad, nullptr, uses, C, ui, 0, lane, a.kahan, tot,
                                         Us, Uc);
-                    const float U = gj_reduce<R, 1>(sm, tot, Us, Uc, warp, 0, lane, red_s, red_c, &U_sh);
+                    gj_reduce<R, 1>(sm, tot, Us, Uc, warp, 0, lane, red_s, red_c);
+                    const float U = gj_sum_u(red_s, red_c);
                     if ((int)threadIdx.x < srows)
                         ic_s[sub + threadIdx.x] = row_current<1>(sm, threadIdx.x,
-                                                                 (vb[local0 + threadIdx.x] - m_shift) * GJ_SCALE,
+                                                                 gj_u(vb[local0 + threadIdx.x], C),
                                                                  P.n, U, P.g);
                     __syncthreads();   // part[] is rewritten by the next row block
                 }

@@ -15,7 +15,7 @@
 // N > TJ.  A CTA has GR x GJ warps: GR row groups of R rows and GJ interleaved column
 // splits.  Each lane holds u_i of its R rows and walks its columns four at a time: one
 // 16-byte shared load of raw V_dend, centred, scaled and negated in registers
-// (x_j = -(V_j - m) s: two packed f32x2 operations per four columns), then 4 x R pairs
+// (x_j = C - s V_j: two packed f32x2 operations per four columns, gj_u), then 4 x R pairs
 // through packed f32x2 arithmetic (per two pairs: one FADD2, one FMUL2, two ex2, one
 // FFMA2).  Lane sums are folded into Kahan-compensated accumulators every 64 columns, then
 // summed pairwise across lanes (a fixed butterfly) and across column splits, so results
@@ -50,7 +50,6 @@ __global__ void __launch_bounds__(DenseBounds<R>::threads) dense_step_kernel(con
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ float red_s[32], red_c[32];
-    __shared__ float U_sh;
 
     const StepCommon &c = a.c;
     const int n = c.n;
@@ -65,30 +64,35 @@ __global__ void __launch_bounds__(DenseBounds<R>::threads) dense_step_kernel(con
         mbar_init(&bar[1], 1);
         fence_mbar_init();
     }
-    pdl_enter();
-
-    const int64_t t = step_index(c);
-    const float *vcur = a.vd_in != nullptr ? a.vd_in : vd_cur(c);
-    float *vnext = a.fuse ? vd_next(c) : nullptr;
     const int row_base = blockIdx.x * rows_cta;
     float *cs = sm.part + W * R;              // staged Cell words of the CTA's rows
-    float *ic_s = cs + NCW * rows_cta;        // their gap currents
+    // the row this thread updates (a CTA has fewer rows than threads), and its pulse: read
+    // before the wait on the previous step
+    const int mine = threadIdx.x, row = row_base + mine;
+    const bool has_row = mine < rows_cta && row < n;
+    const PulseAhead pa = pulse_ahead(c.pulses, row, has_row && a.fuse);
     __syncthreads();
+    pdl_enter();
+
+    const float *vcur = a.vd_in != nullptr ? a.vd_in : vd_cur(c);
     if (threadIdx.x == 0)
         for (int k = 0; k < 2 && k < sm.n_tiles; ++k) issue_tile(sm, vcur, c.n_pad, k, bar);
     // the rows' state words travel to shared memory while the pair loop runs
     if (a.fuse) stage_cells(cs, c.S, vcur, row_base, rows_cta, n);
-    const float m_shift = vcur[0];
+    const float C = vcur[0] * GJ_SCALE;
+    const int64_t t = step_index(c);
 
     float ui[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int i = row_base + rg * R + r;
-        ui[r] = (i < n) ? (vcur[i] - m_shift) * GJ_SCALE : 0.0f;
+        ui[r] = (i < n) ? gj_u(vcur[i], C) : 0.0f;
     }
+    float iapp = pulse_current(c.pulses, pa, t);
+    if (c.iapp != nullptr && has_row) iapp += c.iapp[row];
     uint32_t uses[2] = {0u, 0u};
     float tot[R], Us, Uc;
-    if (!gj_pass<R, GJ>(sm, vcur, n, c.n_pad, bar, uses, m_shift, ui, csp, lane, a.kahan, tot, Us, Uc)) {
+    if (!gj_pass<R, GJ>(sm, vcur, n, c.n_pad, bar, uses, C, ui, csp, lane, a.kahan, tot, Us, Uc)) {
         if (threadIdx.x == 0) {
             if (c.status != nullptr) atomicOr(c.status, (uint32_t)ST_TIMEOUT);   // primitives pass none
             // let any copy still in flight land before the CTA's shared memory is released
@@ -101,28 +105,20 @@ __global__ void __launch_bounds__(DenseBounds<R>::threads) dense_step_kernel(con
         cp_async_wait_all();   // no staging copy may still be landing when the CTA exits
         return;
     }
-    const float U = gj_reduce<R, GJ>(sm, tot, Us, Uc, rg, csp, lane, red_s, red_c, &U_sh);
-
-    for (int rr = threadIdx.x; rr < rows_cta; rr += blockDim.x) {
-        const int i = row_base + rr;
-        if (i >= n) break;
-        const float ic = row_current<GJ>(sm, rr, (vcur[i] - m_shift) * GJ_SCALE, n, U, a.g);
-        if (!a.fuse) a.ic_out[i] = ic;
-        else ic_s[rr] = ic;
-    }
-    if (!a.fuse) return;
-    cp_async_wait_all();
-    __syncthreads();
+    gj_reduce<R, GJ>(sm, tot, Us, Uc, rg, csp, lane, red_s, red_c);
+    if ((mine & ~31) >= rows_cta) return;     // warps without a row
+    const float U = gj_sum_u(red_s, red_c);
+    if (!has_row) return;
     // one thread per cell, from the staged words (ten threads per cell, cell_step_role,
     // measured slower here: 0.89 against 0.70 us per step at 8192 cells)
-    for (int rr = threadIdx.x; rr < rows_cta; rr += blockDim.x) {
-        const int i = row_base + rr;
-        if (i >= n) break;
-        float iapp = pulse_current(c.pulses, i, t);
-        if (c.iapp != nullptr) iapp += c.iapp[i];
-        const CellNext o = cell_step(c.P, staged_cell(cs, rows_cta, rr), ic_s[rr], iapp);
-        finish_cell(c, t, vnext, i, o);
+    const float vd = a.fuse ? cs[mine] : vcur[row];
+    const float ic = row_current<GJ>(sm, mine, gj_u(vd, C), n, U, a.g);
+    if (!a.fuse) {
+        a.ic_out[row] = ic;
+        return;
     }
+    const CellNext o = cell_step(c.P, staged_cell(cs, rows_cta, mine), ic, iapp);
+    finish_cell(c, t, vd_next(c), row, o);
 }
 
 // ---- persistent: many steps in one cooperative launch ------------------------------------
@@ -145,7 +141,7 @@ __global__ void __launch_bounds__(PersistBounds<R>::threads) dense_persist_kerne
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ float red_s[32], red_c[32];
-    __shared__ float U_sh, m_sh;
+    __shared__ float m_sh;
     __shared__ int ok_sh;
 
     const StepCommon &c = a.c;
@@ -209,15 +205,15 @@ __global__ void __launch_bounds__(PersistBounds<R>::threads) dense_persist_kerne
         // shift m = V_dend of cell 0 at step t (from L2, or from the tile itself)
         if (threadIdx.x == 0) m_sh = single ? sm.tile0[0] : __ldcg(vcur);
         __syncthreads();
-        const float m_shift = m_sh;
+        const float C = m_sh * GJ_SCALE;
         float ui[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int rr = rg * R + r;
-            ui[r] = (rr < rows_here) ? (cs[rr] - m_shift) * GJ_SCALE : 0.0f;
+            ui[r] = (rr < rows_here) ? gj_u(cs[rr], C) : 0.0f;
         }
         float tot[R], Us, Uc;
-        if (!gj_pass<R, GJ>(sm, single ? nullptr : vcur, n, c.n_pad, bar, uses, m_shift, ui, csp, lane, a.kahan, tot,
+        if (!gj_pass<R, GJ>(sm, single ? nullptr : vcur, n, c.n_pad, bar, uses, C, ui, csp, lane, a.kahan, tot,
                             Us, Uc)) {
             if (threadIdx.x == 0) {
                 atomicOr(c.status, (uint32_t)ST_TIMEOUT);
@@ -226,9 +222,10 @@ __global__ void __launch_bounds__(PersistBounds<R>::threads) dense_persist_kerne
             }
             break;
         }
-        const float U = gj_reduce<R, GJ>(sm, tot, Us, Uc, rg, csp, lane, red_s, red_c, &U_sh);
+        gj_reduce<R, GJ>(sm, tot, Us, Uc, rg, csp, lane, red_s, red_c);
+        const float U = gj_sum_u(red_s, red_c);
         for (int rr = threadIdx.x; rr < rows_here; rr += blockDim.x)
-            ic_s[rr] = row_current<GJ>(sm, rr, (cs[rr] - m_shift) * GJ_SCALE, n, U, a.g);
+            ic_s[rr] = row_current<GJ>(sm, rr, gj_u(cs[rr], C), n, U, a.g);
         __syncthreads();
         if (roles) {   // one round: read the cell, barrier, write its new words
             const int role = threadIdx.x / rows32, rr = threadIdx.x - role * rows32;
@@ -290,9 +287,9 @@ size_t dense_smem_bytes(int n_pad, int R, int W) {
     const size_t tiles = (n_tiles > 1 ? 2 * TJ : n_pad) * sizeof(float);
     return tiles + (size_t)W * R * sizeof(float);   // part[rows_cta][GJ] = (W / GJ) * R * GJ floats
 }
-// the per-step kernel also stages its rows' Cell words and keeps their currents
+// the per-step kernel also stages its rows' Cell words
 static size_t dense_step_smem_bytes(int n_pad, int R, int W, int GJ) {
-    return dense_smem_bytes(n_pad, R, W) + (size_t)(NCW + 1) * (W / GJ) * R * sizeof(float);
+    return dense_smem_bytes(n_pad, R, W) + (size_t)NCW * (W / GJ) * R * sizeof(float);
 }
 
 // ---- launch-shape dispatch: R rows per warp, W warps = (W / GJ) row groups x GJ splits ----

@@ -12,6 +12,12 @@ namespace ion {
 
 constexpr float PAD_U = 1.0e6f;   // |u| of padded columns: 2^{-PAD_U^2} is exactly 0 (matrix kernel)
 
+// u = s V - C of a row, C = fl(s m) with m the step's shift (V_dend of cell 0): one fused
+// operation, the columns' negated x = C - s V the same bits with the other sign.  C is rounded,
+// but the same C enters every u, so differences and N u_i - sum u_j are free of it; each u is
+// rounded once, relative to |V - m|, as by (V - m) s.
+__device__ __forceinline__ float gj_u(float v, float C) { return fmaf(v, GJ_SCALE, -C); }
+
 struct DenseSmem {
     float *tile0;     // buffer b at tile0 + b * buf_len
     int buf_len;
@@ -39,15 +45,15 @@ __device__ __forceinline__ void issue_tile(const DenseSmem &sm, const float *src
 // column against the lane's R rows, summed into acc[r].  CHECK: the block may run past n4
 // (the last block of a tile), so each column is tested; a full block runs without tests.
 template <int R, int GJ, int BLK, bool CHECK>
-__device__ __forceinline__ void gj_block(const float4 *t4, int m0, int n4, float2 negm2, float2 negs2,
+__device__ __forceinline__ void gj_block(const float4 *t4, int m0, int n4, float2 c2, float2 negs2,
                                          const float2 (&u2)[R], float2 (&acc)[R]) {
 #pragma unroll 4
     for (int mm = 0; mm < BLK; ++mm) {
         const int m = m0 + mm * 32 * GJ;
         if (CHECK && m >= n4) break;
         const float4 v = t4[m];
-        const float2 va = __fmul2_rn(__fadd2_rn(make_float2(v.x, v.y), negm2), negs2);
-        const float2 vb = __fmul2_rn(__fadd2_rn(make_float2(v.z, v.w), negm2), negs2);
+        const float2 va = __ffma2_rn(make_float2(v.x, v.y), negs2, c2);
+        const float2 vb = __ffma2_rn(make_float2(v.z, v.w), negs2, c2);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const float2 da = __fadd2_rn(u2[r], va);
@@ -66,7 +72,7 @@ __device__ __forceinline__ void gj_block(const float4 *t4, int m0, int n4, float
 // flight (issue_tile) and the remaining ones are issued here; if NULL the single tile
 // already holds V_dend (single-CTA persistent mode).  The tiles hold raw V_dend: each lane
 // centres, scales and negates the four columns of a 16-byte load as it reads them,
-// x_j = -(V_j - m) s, so there is no pass over the tile between its arrival and the pair
+// x_j = C - s V_j (gj_u), so there is no pass over the tile between its arrival and the pair
 // loop.  Columns past the last real cell are skipped.  After a tile's pairs, every warp
 // adds up its even share of the tile's real x_j (the linear part's sum_j u_j is not
 // needed before the reduction, and an even share keeps the warps balanced).  On return
@@ -75,7 +81,7 @@ __device__ __forceinline__ void gj_block(const float4 *t4, int m0, int n4, float
 // Returns false (in every thread) if a bulk copy did not land in time.
 template <int R, int GJ>
 __device__ __forceinline__ bool gj_pass(const DenseSmem &sm, const float *src, int n, int n_pad, uint64_t *bar,
-                                        uint32_t (&bar_uses)[2], float m_shift, const float (&ui)[R], int cs,
+                                        uint32_t (&bar_uses)[2], float C, const float (&ui)[R], int cs,
                                         int lane, int kahan, float (&tot)[R], float &Us, float &Uc) {
     float ks[R], kc[R];
     float2 u2[R];
@@ -85,7 +91,7 @@ __device__ __forceinline__ bool gj_pass(const DenseSmem &sm, const float *src, i
         u2[r] = make_float2(ui[r], ui[r]);
     }
     float ns = 0.0f, nc = 0.0f;   // compensated sum of x = -u over this thread's share of columns
-    const float2 negm2 = make_float2(-m_shift, -m_shift);
+    const float2 c2 = make_float2(C, C);
     const float2 negs2 = make_float2(-GJ_SCALE, -GJ_SCALE);
     constexpr int BLK = 16;       // float4 loads per lane between Kahan folds
     for (int kt = 0; kt < sm.n_tiles; ++kt) {
@@ -110,8 +116,8 @@ __device__ __forceinline__ bool gj_pass(const DenseSmem &sm, const float *src, i
             float2 acc[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) acc[r] = make_float2(0.0f, 0.0f);
-            if (m0 + (BLK - 1) * 32 * GJ < n4w) gj_block<R, GJ, BLK, false>(t4, m0, n4w, negm2, negs2, u2, acc);
-            else gj_block<R, GJ, BLK, true>(t4, m0, n4w, negm2, negs2, u2, acc);
+            if (m0 + (BLK - 1) * 32 * GJ < n4w) gj_block<R, GJ, BLK, false>(t4, m0, n4w, c2, negs2, u2, acc);
+            else gj_block<R, GJ, BLK, true>(t4, m0, n4w, c2, negs2, u2, acc);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const float blk = acc[r].x + acc[r].y;
@@ -122,8 +128,8 @@ __device__ __forceinline__ bool gj_pass(const DenseSmem &sm, const float *src, i
         // this thread's share of the tile's real x_j, the same transform as above
         for (int j4 = threadIdx.x; j4 < n4; j4 += blockDim.x) {
             const float4 v = t4[j4];
-            const float2 va = __fmul2_rn(__fadd2_rn(make_float2(v.x, v.y), negm2), negs2);
-            const float2 vb = __fmul2_rn(__fadd2_rn(make_float2(v.z, v.w), negm2), negs2);
+            const float2 va = __ffma2_rn(make_float2(v.x, v.y), negs2, c2);
+            const float2 vb = __ffma2_rn(make_float2(v.z, v.w), negs2, c2);
             const int rem = real - 4 * j4;   // real columns in this float4 (>= 1)
             float x = va.x;
             if (rem > 1) x += va.y;
@@ -145,11 +151,13 @@ __device__ __forceinline__ bool gj_pass(const DenseSmem &sm, const float *src, i
     return true;
 }
 
-// Reduce the lane sums into part[row][split] and the block's sum_j u_j (returned).
+// Reduce the lane sums into part[row][split] and the threads' shares of sum_j u_j into one
+// compensated pair per warp; complete (with all earlier shared-memory writes and, through
+// cp_async_wait_all, staging copies of every thread) at the barrier it ends with.
 template <int R, int GJ>
-__device__ __forceinline__ float gj_reduce(const DenseSmem &sm, const float (&tot)[R], float Us, float Uc, int rg,
-                                           int cs, int lane, float *red_s, float *red_c, float *U_sh) {
-    const int warp = threadIdx.x >> 5, W = blockDim.x >> 5;
+__device__ __forceinline__ void gj_reduce(const DenseSmem &sm, const float (&tot)[R], float Us, float Uc, int rg,
+                                          int cs, int lane, float *red_s, float *red_c) {
+    const int warp = threadIdx.x >> 5;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         float v = tot[r];
@@ -166,15 +174,17 @@ __device__ __forceinline__ float gj_reduce(const DenseSmem &sm, const float (&to
         red_s[warp] = Us;
         red_c[warp] = Uc;
     }
+    cp_async_wait_all();
     __syncthreads();
-    if (warp == 0) {   // the warps' compensated partial sums, combined by a fixed butterfly
-        float v = lane < W ? red_s[lane] - red_c[lane] : 0.0f;
+}
+// The block's sum_j u_j, after gj_reduce: every warp that needs it adds up the warps'
+// compensated partial sums by the same fixed butterfly (no second barrier).  Whole warps only.
+__device__ __forceinline__ float gj_sum_u(const float *red_s, const float *red_c) {
+    const int lane = threadIdx.x & 31, W = blockDim.x >> 5;
+    float v = lane < W ? red_s[lane] - red_c[lane] : 0.0f;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) *U_sh = v;
-    }
-    __syncthreads();
-    return *U_sh;
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
 }
 
 // Gap current of local row rr (after gj_reduce).
