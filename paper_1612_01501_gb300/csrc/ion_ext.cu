@@ -73,8 +73,9 @@ static ion_status persist_run(ion_sim *s, int64_t n_steps, const float *iapp) {
         a.timeout_ns = s->barrier_timeout_ns;
         a.debug_delay_ns = s->debug_delay_ns;
         a.bar_base = s->barrier_base;
-        cudaError_t e = reset_barrier(s);
-        if (e == cudaSuccess) e = persist_dense(a, s->persist_R, s->persist_W, s->persist_GJ, nullptr, true, s->st);
+        const bool small = s->n <= DENSE_SMALL;   // one CTA: no grid barrier
+        cudaError_t e = small ? launch_dense_small(a, s->st) : reset_barrier(s);
+        if (e == cudaSuccess && !small) e = persist_dense(a, s->persist_R, s->persist_W, s->persist_GJ, nullptr, true, s->st);
         s->launches++;
         if (e == cudaSuccess) e = launch_advance(s->d_t, chunk, s->st);
         s->launches++;
@@ -84,25 +85,19 @@ static ion_status persist_run(ion_sim *s, int64_t n_steps, const float *iapp) {
     return ION_OK;
 }
 
-// Shape of a persistent launch: one CTA of ceil(n / 8) warps (8 rows each, one column
-// split) when n <= 144, so small networks keep V_dend in shared memory; else the
+// Shape of a persistent launch: one CTA of its own kernel for small networks; else the
 // per-step shape, if the persistent kernel allows that many threads and all its CTAs
 // can be resident at once.
 static bool choose_persist_shape(ion_sim *s) {
+    if (s->n <= DENSE_SMALL) {
+        s->persist_R = s->persist_W = s->persist_GJ = 1;   // not used
+        return true;
+    }
     PersistArgs probe{};
     probe.c.n = s->n;
     probe.c.n_pad = s->n_pad;
-    int R, W, GJ;
-    if (s->n <= 144) {
-        R = 8;
-        W = (s->n + 7) / 8;
-        GJ = 1;
-    } else {
-        R = s->dense_R;
-        W = s->dense_W;
-        GJ = s->dense_GJ;
-        if (W * 32 > persist_max_threads(R)) return false;
-    }
+    const int R = s->dense_R, W = s->dense_W, GJ = s->dense_GJ;
+    if (W * 32 > persist_max_threads(R)) return false;
     int grid = 0;
     if (persist_dense(probe, R, W, GJ, &grid, false, s->st) != cudaSuccess || grid <= 0) return false;
     s->persist_R = R;
@@ -131,7 +126,7 @@ ion_status ion_sim_setup_extras(ion_sim *s, const ion_params *p) {
             // several CTAs: the half-work kernel, if its shape and grid fit
             const int rows = (s->persist_W / s->persist_GJ) * s->persist_R;
             const int grid = (s->n + rows - 1) / rows;
-            if (grid >= 2 && s->persist_R <= 4 && s->persist_W <= 28 && (s->flags & ION_FLAG_HALF_WORK)) {
+            if (s->n > DENSE_SMALL && grid >= 2 && s->persist_R <= 4 && s->persist_W <= 28 && (s->flags & ION_FLAG_HALF_WORK)) {
                 HalfArgs probe{};
                 probe.rows = rows;
                 int fits = 0;

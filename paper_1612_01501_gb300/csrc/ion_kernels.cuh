@@ -343,6 +343,8 @@ cudaError_t launch_default_state(const ModelF &P, float V0, float ca0, float gca
 cudaError_t prepare_dense_step(int rows_per_warp, int warps, int col_splits, int n_pad);
 cudaError_t persist_dense(const PersistArgs &a, int rows_per_warp, int warps, int col_splits, int *grid_out,
                           bool launch, cudaStream_t st);
+constexpr int DENSE_SMALL = 192;   // cells up to which a persistent launch is one CTA (ion_dense_small.cu)
+cudaError_t launch_dense_small(const PersistArgs &a, cudaStream_t st);
 cudaError_t launch_dense_half(const HalfArgs &a, int rows_per_warp, int warps, int col_splits, int grid,
                               bool launch, int *ok_out, cudaStream_t st);
 int half_colsum_stride(int grid, int rows_per_cta);

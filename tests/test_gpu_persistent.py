@@ -140,3 +140,26 @@ def test_grid_barrier_counter_wraps_past_2_to_32(cuda, O, half):
     a, _ = _run(cfg["n"], cfg["g"], S0, 200, flags, chunks=2)
     b, _ = _run(cfg["n"], cfg["g"], S0, 200, flags, chunks=2, debug_barrier_base=(1 << 32) - 300)
     np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1, 2, 5, 31, 33, 64, 99, 130, 191, 192, 193])
+def test_one_cta_network_matches_step_launches(cuda, O, n):
+    """The one-CTA kernel (up to 192 cells; 193 takes the grid-barrier kernel) against the
+    per-step launches over 120 steps with pulses, odd and even step counts per call, all
+    fields: the currents differ by the order of at most 192 terms (below 1e-6 of them, at most
+    0.02 uA/cm^2 a step, so 1e-9 mV each), a voltage by a few FP32 units of 60 mV (4e-6)."""
+    g = inputs.junction_weight(0.04, n)
+    cfg = dict(n=n, jitter=inputs.vdend_jitter(n, 9))
+    S0 = initial_state(O, cfg)
+    pul = inputs.pulse_windows(np.arange(0, n, 3), [(0.5, 3.0), (2.0, 4.0)], 5.0)
+    out = []
+    for flags in (ion.FLAG_KAHAN, ion.FLAG_KAHAN | ion.FLAG_PERSISTENT):
+        with ion.Simulation(n, ion.DENSE_UNIFORM, g=g, init_state=S0, flags=flags) as sim:
+            sim.set_input(pul)
+            for k in (1, 2, 50, 67):
+                sim.step(k)
+            out.append(sim.state())
+    scale = np.maximum(np.abs(out[0]), 1e-3)
+    assert np.abs(out[0][:3] - out[1][:3]).max() <= 1e-4
+    assert (np.abs(out[0] - out[1])[3:18] / scale[3:18]).max() <= 1e-4
+    assert np.abs(out[0][18] - out[1][18]).max() <= 1e-4
