@@ -245,9 +245,10 @@ ion_status ion_default_state(const ion_model *model, int32_t n, float *out);
 ion_status ion_create(const ion_net *net, const ion_conn *conn, const ion_params *params,
                       const float *init_state, ion_sim **out);
 
-/* Several independent networks advanced together: one launch per time step covers all
- * of them (a list of tiles, each one network's rows), and ion_step replays CUDA graphs of
- * graph_steps launches.  Cells are numbered consecutively across networks (network b's
+/* Several independent networks advanced together: one to three launches per time step cover
+ * all of them (lists of tiles, each one network's rows; the launches of different lists run
+ * side by side, on streams of the handle that are forked from and joined to its stream within
+ * ion_step), and ion_step replays CUDA graphs of graph_steps steps.  Cells are numbered consecutively across networks (network b's
  * cell i is global cell offset_b + i, offset_b = n_0 + ... + n_{b-1}); init_state, the
  * state read and written, pulse cells and trace samples all use this numbering.
  * Dense networks may have at most 8192 cells; CSR arrays must be host memory.

@@ -923,17 +923,27 @@ static cudaError_t enqueue_one_step(ion_sim *s, int k_off, const float *iapp) {
     return e;
 }
 
+// Enqueue k consecutive steps from offset 0 of the device step counter (iapp_base: their dense
+// evoked input), between the extension's fork and join if it has them.
+static cudaError_t enqueue_run(ion_sim *s, int k, const float *iapp_base) {
+    cudaError_t e = s->fork_hook ? s->fork_hook(s) : cudaSuccess;
+    for (int j = 0; j < k && e == cudaSuccess; ++j)
+        e = enqueue_one_step(s, j, iapp_base ? iapp_base + (int64_t)j * s->n : nullptr);
+    if (s->join_hook) {
+        const cudaError_t e1 = s->join_hook(s);
+        if (e == cudaSuccess) e = e1;
+    }
+    return e;
+}
+
 // Enqueue k steps directly (no graph) followed by the device counter advance.
 static cudaError_t enqueue_steps_direct(ion_sim *s, int64_t k, const float *iapp_base) {
     int64_t done = 0;
     while (done < k) {
         const int64_t chunk = std::min<int64_t>(k - done, 1 << 20);
-        for (int64_t j = 0; j < chunk; ++j) {
-            const float *iapp = iapp_base ? iapp_base + (done + j) * (int64_t)s->n : nullptr;
-            cudaError_t e = enqueue_one_step(s, (int)j, iapp);
-            if (e != cudaSuccess) return e;
-        }
-        cudaError_t e = launch_advance(s->d_t, chunk, s->st);
+        cudaError_t e = enqueue_run(s, (int)chunk, iapp_base ? iapp_base + done * (int64_t)s->n : nullptr);
+        if (e != cudaSuccess) return e;
+        e = launch_advance(s->d_t, chunk, s->st);
         s->launches++;
         if (e != cudaSuccess) return e;
         s->t_enq += chunk;
@@ -947,8 +957,7 @@ static ion_status build_graph_once(ion_sim *s) {
     cudaGraph_t g = nullptr;
     const int64_t launches0 = s->launches;
     ION_CK(s, cudaStreamBeginCapture(s->st, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaSuccess;
-    for (int j = 0; j < K && e == cudaSuccess; ++j) e = enqueue_one_step(s, j, nullptr);
+    cudaError_t e = enqueue_run(s, K, nullptr);
     if (e == cudaSuccess) e = launch_advance(s->d_t, K, s->st);
     cudaError_t e2 = cudaStreamEndCapture(s->st, &g);
     s->launches = launches0;

@@ -1,16 +1,22 @@
-// ion_batch.cu -- many independent networks advanced by one launch per time step.
+// ion_batch.cu -- many independent networks advanced together, a few launches per time step.
 //
 // Parameter sweeps run many small networks of uneven sizes and densities.  Each network
 // b gets a segment of the state arrays starting at seg_b (a multiple of 256 cells, the
-// tail padded like a single network's V_dend), so dense networks can stage their V_dend
-// with one 16-byte aligned bulk copy and CSR networks use global column indices into the
-// same arrays.  The work of a step is a list of tiles (network, first row, rows): a
-// dense tile is 8 warps x R rows of one network against all of that network's columns
-// (the single-network pair loop, ion_dense_core.cuh), a CSR tile is up to 256 rows with
-// SW lanes per row (ion_csr_core.cuh); every tile then runs the explicit-Euler update
-// of its rows.  Tiles are ordered by decreasing cost so the hardware scheduler packs the
-// long ones first; the launches of K steps are captured into one CUDA graph and
-// replayed.  ion_autotune times the tile shapes and keeps the fastest.
+// tail padded like a single network's V_dend), so networks can stage their V_dend with one
+// 16-byte aligned bulk copy.  The work of a step is a list of tiles (network, first row,
+// rows): a dense tile is blocks of 8 warps x R rows of one network against all of that
+// network's columns (the single-network pair loop, ion_dense_core.cuh), a CSR tile is up to
+// 256 rows, from the network's sliced rows where its V_dend is staged; every tile then runs
+// the explicit-Euler update of its rows.  The networks are dealt to up to three chains of
+// launches that run side by side (dense and CSR networks have kernels of their own), and
+// within a chain tiles are ordered by decreasing cost so the hardware scheduler packs the
+// long ones first; the launches of K steps are captured into one CUDA graph and replayed.
+// ion_autotune times the tile shapes and keeps the fastest.
+//
+// What bounds it: instruction issue (the 96-network sweep of 32-4096 cells: 70 % issued).
+// That sweep, us per step: 20.3 (the 48 dense networks alone 17.5, the 48 CSR ones 8.8); one
+// launch per step with fixed tiles, 16-bit rows with heads and tails, state and pulses read
+// after the sums took 30.4.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -42,6 +48,7 @@ struct BatchTile {
     int32_t sw;      // CSR: lanes per row
     float g;         // dense: pair weight; CSR with TILE_UNIFORM_W: every edge weight
     int32_t mode;    // CSR: TileMode bits
+    int32_t slice0;  // CSR with TILE_STAGE_V: the network's first slice
 };
 
 struct BatchArgs {
@@ -51,16 +58,109 @@ struct BatchArgs {
     const int32_t *col;
     const uint16_t *col16;    // network-local columns (TILE_C16 networks)
     const float *w;
+    const uint4 *scols;       // sliced columns (and weights) of the staged CSR networks
+    const float4 *sw;
+    const int32_t *soff;      // first round of each slice, and the end
     int32_t kahan;
+    int32_t rows_max;         // rows of the largest tile (<= 256: one thread updates each)
+    int32_t vbuf;             // floats of the V_dend buffer
 };
 
-// V_dend of a network-local column from shared memory (the network's staged copy)
-struct VjShared {
-    const float *vs;
-    __device__ __forceinline__ float operator()(uint32_t j) const { return vs[j]; }
+// ---- sliced rows of a staged CSR network -----------------------------------------------------
+// As in ion_csr_sliced.cu, without the sort and the bank order: a slice is 32 / SW consecutive
+// rows of one network, SW lanes per row, its columns stored round by round (8 edges of every
+// lane, 512 contiguous bytes), padded with the row's own column (dV = 0: adds exactly 0).  A
+// row's sum depends on its edges and SW alone, not on the tile or piece it is computed in, so
+// the per-step and the persistent kernel give the same bits.
+template <bool HAS_W>
+struct SliceAhead {
+    static constexpr int D = HAS_W ? 2 : 4;   // rounds in flight per lane
+    uint4 q[D];
+    float4 wa[HAS_W ? D : 1], wb[HAS_W ? D : 1];
+    int e0, n;                                // first round, rounds
+    __device__ __forceinline__ void load(int j, int round, const uint4 *cols, const float4 *w) {
+        const int lane = threadIdx.x & 31;
+        q[j] = __ldg(cols + (int64_t)round * 32 + lane);
+        if (HAS_W) {
+            wa[j] = __ldg(w + (int64_t)round * 64 + lane);
+            wb[j] = __ldg(w + (int64_t)round * 64 + 32 + lane);
+        }
+    }
+    // the header and first rounds of a slice
+    __device__ __forceinline__ void begin(int slice, const int32_t *off, const uint4 *cols, const float4 *w) {
+        e0 = __ldg(off + slice);
+        n = __ldg(off + slice + 1) - e0;
+#pragma unroll
+        for (int j = 0; j < D; ++j)
+            if (j < n) load(j, e0 + j, cols, w);
+    }
 };
+// Currents of rows [r0, r0 + rows) of a network (local rows) into ic_s; `ah` holds this warp's
+// first slice already (slice_begin below).
+template <bool HAS_W>
+__device__ __forceinline__ void slice_rows(SliceAhead<HAS_W> &ah, int slice0, int lsw, int n, int r0, int rows,
+                                           const int32_t *off, const uint4 *cols, const float4 *w, const float *vs,
+                                           float g, float *ic_s) {
+    constexpr int D = SliceAhead<HAS_W>::D;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int per = 32 >> lsw, s0 = r0 / per, ns = (r0 + rows - 1) / per - s0 + 1;
+    const VjSliced vj{vs};
+    for (int s = warp; s < ns; s += 8) {
+        if (s != warp) ah.begin(slice0 + s0 + s, off, cols, w);
+        const int i = (s0 + s) * per + (lane >> lsw);
+        const float vi = vs[min(i, n - 1)];
+        float ks = 0.0f, kc = 0.0f;           // compensated over groups of D rounds
+        for (int k = 0; k < ah.n; k += D) {
+            float blk = 0.0f;
+#pragma unroll
+            for (int j = 0; j < D; ++j) {
+                if (k + j < ah.n) blk += csr_group16<HAS_W>(ah.q[j], ah.wa[HAS_W ? j : 0], ah.wb[HAS_W ? j : 0], vi, vj);
+                if (k + D + j < ah.n) ah.load(j, ah.e0 + k + D + j, cols, w);
+            }
+            kahan_add(ks, kc, blk);
+        }
+        float acc = ks - kc;
+        for (int o = (1 << lsw) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((lane & ((1 << lsw) - 1)) == 0 && i >= r0 && i < r0 + rows)
+            ic_s[i - r0] = (HAS_W ? acc : acc * g) * (1.0f / GJ_SCALE);
+    }
+}
+// This warp's first slice of rows [r0, ...) of a network
+template <bool HAS_W>
+__device__ __forceinline__ void slice_begin(SliceAhead<HAS_W> &ah, int slice0, int lsw, int r0, int rows,
+                                            const int32_t *off, const uint4 *cols, const float4 *w) {
+    const int per = 32 >> lsw, warp = threadIdx.x >> 5, s0 = r0 / per, ns = (r0 + rows - 1) / per - s0 + 1;
+    if (warp < ns) ah.begin(slice0 + s0 + warp, off, cols, w);
+}
 
-// CSR rows of a TILE_C16 tile: 16-bit local columns, V_dend from `vj` (staged or global)
+// The sliced columns (and weights) from the networks' 16-bit rows: a warp per slice.
+struct SliceDesc {
+    int32_t row, rows;   // first row (padded index), rows (<= 32 / SW)
+    int32_t seg, lsw;
+};
+__global__ void __launch_bounds__(128) batch_slice_fill_kernel(const SliceDesc *desc, int n_slices, const int32_t *off,
+                                                               const int32_t *row_ptr, const uint16_t *col16,
+                                                               const float *w, uint16_t *cols, float *wout) {
+    const int s = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (s >= n_slices) return;
+    const SliceDesc d = desc[s];
+    const int rr = lane >> d.lsw, sw = 1 << d.lsw, li = lane & (sw - 1);
+    const bool has = rr < d.rows;
+    const int i = d.row + (has ? rr : 0);
+    const int b = row_ptr[i], e = has ? row_ptr[i + 1] : b;
+    const int64_t r0 = off[s];
+    const int rounds = off[s + 1] - (int)r0;
+    const uint16_t self = (uint16_t)(i - d.seg);
+    for (int k = 0; k < rounds; ++k)
+        for (int t = 0; t < 8; ++t) {
+            const int x = b + (k * sw + li) * 8 + t;
+            const bool real = x < e;
+            cols[((r0 + k) * 32 + lane) * 8 + t] = real ? col16[x] : self;
+            if (wout) wout[((r0 + k) * 64 + (t >> 2) * 32 + lane) * 4 + (t & 3)] = real ? w[x] : 0.0f;
+        }
+}
+
+// CSR rows of a TILE_C16 tile: 16-bit local columns, V_dend from `vj` (global memory)
 template <int SW, bool HAS_W, class VJ>
 __device__ __forceinline__ void batch_csr_rows16(const BatchArgs &a, const BatchTile &T, const float *vcur, VJ vj,
                                                  float *ic_s) {
@@ -139,74 +239,127 @@ __device__ __forceinline__ void batch_csr_rows(const BatchArgs &a, const BatchTi
     }
 }
 
-// 256 threads: 8 warps.  Dense tiles: 8 row groups of R rows, one column split.
+// ---- the per-step kernels ------------------------------------------------------------------
+// What both do around the row currents: the tile's pulses are read before the wait on the
+// previous step (neither they nor the tile list change between steps), its rows' state words
+// travel to shared memory while the sums run, and one thread per row updates its cell.
+struct TileRow {
+    int64_t i;            // this thread's cell
+    bool has;
+    PulseAhead pa;
+};
+__device__ __forceinline__ TileRow tile_row(const BatchArgs &a, const BatchTile &T) {
+    const bool has = (int)threadIdx.x < T.rows;
+    const int64_t i = T.row0 + (int64_t)threadIdx.x;
+    return {i, has, pulse_ahead(a.c.pulses, i, has)};
+}
+__device__ __forceinline__ void tile_stage(const BatchArgs &a, const TileRow &r, const float *vcur, float *cs) {
+    if (r.has)
+#pragma unroll
+        for (int w = 0; w < NCW; ++w)
+            cp_async4(cs + w * a.rows_max + threadIdx.x, (w == 0 ? vcur : a.c.S.f(cell_word_field(w))) + r.i);
+    cp_async_commit();
+}
+__device__ __forceinline__ void tile_update(const BatchArgs &a, const TileRow &r, int64_t t, const float *cs, float ic) {
+    float iapp = pulse_current(a.c.pulses, r.pa, t);
+    if (a.c.iapp != nullptr) iapp += a.c.iapp[r.i];
+    const CellNext o = cell_step(a.c.P, staged_cell(cs, a.rows_max, threadIdx.x), ic, iapp);
+    finish_cell(a.c, t, vd_next(a.c), r.i, o);
+}
+
+// Dense tiles, 8 warps: blocks of 8 row groups of R rows against the network's staged columns.
 template <int R>
-__global__ void __launch_bounds__(256) batch_step_kernel(const BatchArgs a) {
+__global__ void __launch_bounds__(256) batch_dense_kernel(const BatchArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ float red_s[32], red_c[32];
-    __shared__ float ic_s[256];
-    pdl_enter();
-
     const BatchTile T = a.tiles[blockIdx.x];
     const StepCommon &c = a.c;
+    const TileRow row = tile_row(a, T);
+    float *cs = reinterpret_cast<float *>(smem_raw) + a.vbuf + 8 * R;
+    const DenseSmem sm = dense_smem(smem_raw, T.n_pad);   // one tile: n_pad <= 8192
+    if (threadIdx.x == 0) {
+        mbar_init(&bar[0], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    pdl_enter();
+    const float *vcur = vd_cur(c), *net_v = vcur + T.seg;
+    if (threadIdx.x == 0) issue_tile(sm, net_v, T.n_pad, 0, bar);
+    tile_stage(a, row, vcur, cs);
     const int64_t t = step_index(c);
-    const float *vcur = vd_cur(c);
-    float *vnext = vd_next(c);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-    if (T.kind == TILE_DENSE) {
-        const DenseSmem sm = dense_smem(smem_raw, T.n_pad);   // one tile: n_pad <= 8192
-        const float *net_v = vcur + T.seg;
-        if (threadIdx.x == 0) {
-            mbar_init(&bar[0], 1);
-            mbar_init(&bar[1], 1);
-            fence_mbar_init();
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) issue_tile(sm, net_v, T.n_pad, 0, bar);
-        const float C = net_v[0] * GJ_SCALE;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, mine = threadIdx.x;
+    const float C = net_v[0] * GJ_SCALE;
+    const int local0 = T.row0 - T.seg;
+    uint32_t uses[2] = {0u, 0u};
+    float U = 0.0f, ic = 0.0f;
+    for (int sub = 0; sub < T.rows; sub += 8 * R) {
         float ui[R];
-        const int local0 = T.row0 - T.seg;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const int li = local0 + warp * R + r;
-            ui[r] = (warp * R + r < T.rows) ? gj_u(net_v[li], C) : 0.0f;
+            const int rr = sub + warp * R + r;
+            ui[r] = rr < T.rows ? gj_u(net_v[local0 + rr], C) : 0.0f;
         }
-        uint32_t uses[2] = {0u, 0u};
         float tot[R], Us, Uc;
-        if (!gj_pass<R, 1>(sm, net_v, T.n, T.n_pad, bar, uses, C, ui, 0, lane, a.kahan, tot, Us, Uc)) {
+        if (!gj_pass<R, 1>(sm, sub == 0 ? net_v : nullptr, T.n, T.n_pad, bar, uses, C, ui, 0, lane, a.kahan, tot, Us, Uc,
+                           sub == 0)) {
             if (threadIdx.x == 0) {
                 atomicOr(c.status, (uint32_t)ST_TIMEOUT);
                 (void)mbar_wait_bounded(&bar[0], uses[0] & 1u);
             }
+            cp_async_wait_all();
             return;
         }
+        if (sub > 0) __syncthreads();   // the last block's partial sums have been read
         gj_reduce<R, 1>(sm, tot, Us, Uc, warp, 0, lane, red_s, red_c);
-        const float U = gj_sum_u(red_s, red_c);
-        if ((int)threadIdx.x < T.rows) {
-            const int rr = threadIdx.x;
-            ic_s[rr] = row_current<1>(sm, rr, gj_u(net_v[local0 + rr], C), T.n, U, T.g);
-        }
-    } else if (T.mode & TILE_STAGE_V) {
-        // the network's V_dend (n_pad <= TJ floats) in shared memory, 16-bit local columns
-        float *vs = reinterpret_cast<float *>(smem_raw);
-        if (threadIdx.x == 0) {
-            mbar_init(&bar[0], 1);
-            fence_mbar_init();
-            mbar_expect_tx(&bar[0], (uint32_t)T.n_pad * 4u);
-            bulk_g2s(vs, vcur + T.seg, (uint32_t)T.n_pad * 4u, &bar[0]);
-        }
-        __syncthreads();
-        const bool landed = mbar_wait_bounded(&bar[0], 0u);
+        if (sub == 0) U = gj_sum_u(red_s, red_c);
+        const int rr = mine - sub;      // the thread that owns a row of this block takes its current
+        if (row.has && rr >= 0 && rr < 8 * R) ic = row_current<1>(sm, rr, gj_u(cs[mine], C), T.n, U, T.g);
+    }
+    if (row.has) tile_update(a, row, t, cs, ic);
+}
+
+// CSR tiles (and networks without junctions)
+__global__ void __launch_bounds__(256) batch_csr_kernel(const BatchArgs a) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ float ic_s[256];
+    const BatchTile T = a.tiles[blockIdx.x];
+    const StepCommon &c = a.c;
+    const TileRow row = tile_row(a, T);
+    float *vs = reinterpret_cast<float *>(smem_raw), *cs = vs + a.vbuf;
+    const bool staged = (T.mode & TILE_STAGE_V) != 0, uniform = (T.mode & TILE_UNIFORM_W) != 0;
+    const int lsw = 31 - __clz(T.sw), local0 = T.row0 - T.seg;
+    // the first slice of this warp, before the wait too
+    SliceAhead<false> au;
+    SliceAhead<true> aw;
+    if (staged && uniform) slice_begin(au, T.slice0, lsw, local0, T.rows, a.soff, a.scols, a.sw);
+    else if (staged) slice_begin(aw, T.slice0, lsw, local0, T.rows, a.soff, a.scols, a.sw);
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    pdl_enter();
+    const float *vcur = vd_cur(c);
+    if (staged && threadIdx.x == 0) {   // the network's V_dend (n_pad <= TJ floats)
+        mbar_expect_tx(&bar, (uint32_t)T.n_pad * 4u);
+        bulk_g2s(vs, vcur + T.seg, (uint32_t)T.n_pad * 4u, &bar);
+    }
+    tile_stage(a, row, vcur, cs);
+    const int64_t t = step_index(c);
+    if (staged) {
+        const bool landed = threadIdx.x >= 32 || mbar_wait_bounded(&bar, 0u);
         if (__syncthreads_or(!landed)) {
             if (threadIdx.x == 0) {
                 atomicOr(c.status, (uint32_t)ST_TIMEOUT);
-                (void)mbar_wait_bounded(&bar[0], 0u);
+                (void)mbar_wait_bounded(&bar, 0u);
             }
+            cp_async_wait_all();
             return;
         }
-        batch_csr_tile16(a, T, vcur, VjShared{vs}, ic_s);
+        if (uniform) slice_rows(au, T.slice0, lsw, T.n, local0, T.rows, a.soff, a.scols, a.sw, vs, T.g, ic_s);
+        else slice_rows(aw, T.slice0, lsw, T.n, local0, T.rows, a.soff, a.scols, a.sw, vs, T.g, ic_s);
     } else if (T.mode & TILE_C16) {
         batch_csr_tile16(a, T, vcur, VjGlobal{vcur + T.seg}, ic_s);
     } else {
@@ -219,14 +372,9 @@ __global__ void __launch_bounds__(256) batch_step_kernel(const BatchArgs a) {
             default: batch_csr_rows<32>(a, T, vcur, ic_s); break;
         }
     }
+    cp_async_wait_all();
     __syncthreads();
-    if ((int)threadIdx.x >= T.rows) return;
-    const int64_t i = T.row0 + threadIdx.x;
-    const Cell cell = load_cell(c.S, vcur, i);
-    float iapp = pulse_current(c.pulses, i, t);
-    if (c.iapp != nullptr) iapp += c.iapp[i];
-    const CellNext o = cell_step(c.P, cell, ic_s[threadIdx.x], iapp);
-    finish_cell(c, t, vnext, i, o);
+    if (row.has) tile_update(a, row, t, cs, ic_s[threadIdx.x]);
 }
 
 // ---- persistent form: many steps of every network in one cooperative launch -------------
@@ -250,6 +398,7 @@ struct PersistItem {
     int32_t pieces;   // pieces of this network (arrivals per step)
     int32_t sw;       // CSR: lanes per row
     int32_t mode;     // CSR: TileMode bits
+    int32_t slice0;   // CSR with TILE_STAGE_V: the network's first slice
     float g;
 };
 
@@ -260,6 +409,9 @@ struct BatchPersistArgs {
     const int32_t *row_ptr;
     const uint16_t *col16;
     const float *w;
+    const uint4 *scols;        // as in BatchArgs
+    const float4 *sw;
+    const int32_t *soff;
     uint32_t *cnt;             // arrival counter per network (zeroed before the launch)
     uint32_t *abort_flag;      // set by a CTA whose wait gave up (zeroed before the launch)
     uint64_t timeout_ns;
@@ -323,10 +475,6 @@ __device__ __forceinline__ void persist_csr_piece(const BatchPersistArgs &a, con
 #undef ION_CSR_SW
 }
 
-struct VRowSmem {
-    const float *v;
-    __device__ __forceinline__ float operator()(int j) const { return v[j]; }
-};
 struct VRowCG {
     const float *v;
     __device__ __forceinline__ float operator()(int j) const { return __ldcg(v + j); }
@@ -413,7 +561,16 @@ __global__ void __launch_bounds__(256, 4) batch_persist_kernel(const BatchPersis
                     __syncthreads();   // part[] is rewritten by the next row block
                 }
             } else if (P.mode & TILE_STAGE_V) {
-                persist_csr_piece(a, P, VRowSmem{vb}, VjShared{vb}, ic_s);
+                const int lsw = 31 - __clz(P.sw), r0 = P.row0 - P.seg;
+                if (P.mode & TILE_UNIFORM_W) {
+                    SliceAhead<false> ah;
+                    slice_begin(ah, P.slice0, lsw, r0, P.rows, a.soff, a.scols, a.sw);
+                    slice_rows(ah, P.slice0, lsw, P.n, r0, P.rows, a.soff, a.scols, a.sw, vb, P.g, ic_s);
+                } else {
+                    SliceAhead<true> ah;
+                    slice_begin(ah, P.slice0, lsw, r0, P.rows, a.soff, a.scols, a.sw);
+                    slice_rows(ah, P.slice0, lsw, P.n, r0, P.rows, a.soff, a.scols, a.sw, vb, P.g, ic_s);
+                }
             } else {
                 persist_csr_piece(a, P, VRowCG{vcur + P.seg}, VjGlobalCG{vcur + P.seg}, ic_s);
             }
@@ -469,9 +626,12 @@ struct BatchNet {
     float g;          // dense: pair weight; CSR with uniform weights: every edge weight
     int64_t e0, nnz;  // CSR edges in the global arrays
     int sw;
+    int slice0 = 0;         // staged CSR: first slice
     bool uniform = false;   // CSR: every weight bitwise equal (g)
     bool c16 = false;       // CSR: 16-bit network-local columns in col16
 };
+
+constexpr int BATCH_CHAINS = 4;
 
 struct BatchExt {
     std::vector<BatchNet> nets;
@@ -489,10 +649,29 @@ struct BatchExt {
     std::vector<int32_t> h_map;     // user cell -> padded cell
     BatchTile *d_tiles = nullptr;
     int n_tiles = 0;
-    int R = 2;                      // dense rows per warp (rows per dense tile = 8 R)
-    int csr_rows = 128;             // rows per CSR tile
+    // The networks are independent, so their tiles are dealt to a few chains of launches that
+    // run side by side: the latency of one chain's step (launch, V_dend copies, the last
+    // tiles' updates) overlaps another chain's work.  Chain 0 runs on the handle's stream, the
+    // others on side streams forked from it before, and joined after, the steps of a call.
+    struct Chain {
+        bool dense = false;
+        int off = 0, n = 0;             // tiles
+        int vbuf = 256, rows_max = 32;  // shared memory of its launches
+    };
+    std::vector<Chain> chains;
+    cudaStream_t side[BATCH_CHAINS - 1] = {};
+    cudaEvent_t ev_fork = nullptr, ev_join[BATCH_CHAINS - 1] = {};
+    bool forked_now = false;            // the next step is the first after a fork
+    int R = 4;                      // dense rows per warp (rows per dense tile = 8 R)
+    int csr_rows = 256;             // rows per CSR tile (fewer where rows are long)
     int sw_scale = 0;               // 0: lanes per row from the degree; +-1: twice / half that
     int max_dense_pad = 256;
+    // sliced rows of the staged CSR networks, for the lanes per row of sw_scale `slice_scale`
+    std::vector<int32_t> h_rp;      // row_ptr over the padded cells
+    uint16_t *d_scols = nullptr;
+    float *d_sw = nullptr;
+    int32_t *d_soff = nullptr;
+    int slice_scale = -2;           // none built yet
     float *d_tmp = nullptr;         // 19 x n_user staging for state I/O
 };
 
@@ -506,36 +685,173 @@ static int csr_sw_for(double deg, int scale) {
     return sw;
 }
 
+// Lanes per row of a sliced network: rows of about four rounds or more, so that the last round's
+// padding stays small.
+static int slice_sw_for(double deg, int scale) {
+    int sw = 1;
+    while (sw < 32 && 64 * sw <= deg) sw *= 2;
+    if (scale > 0 && sw < 32) sw *= 2;
+    if (scale < 0 && sw > 1) sw /= 2;
+    return sw;
+}
+
+static bool net_staged(const BatchExt *X, const BatchNet &b) {
+    return b.kind == ION_CSR && b.c16 && b.n_pad <= X->max_dense_pad;   // fits the launches' shared memory
+}
+
+// The sliced layout for the current lanes-per-row scale (kept while that does not change).
+static ion_status batch_build_slices(ion_sim *s) {
+    BatchExt *X = ext_of(s);
+    if (X->slice_scale == X->sw_scale) return ION_OK;
+    std::vector<SliceDesc> desc;
+    std::vector<int32_t> off;
+    int64_t tot = 0;
+    bool weights = false;
+    for (BatchNet &b : X->nets) {
+        const double deg = b.n > 0 ? (double)b.nnz / b.n : 0.0;
+        if (b.kind == ION_CSR) b.sw = net_staged(X, b) ? slice_sw_for(deg, X->sw_scale) : csr_sw_for(deg, X->sw_scale);
+        if (!net_staged(X, b)) continue;
+        weights = weights || !b.uniform;
+        b.slice0 = (int)desc.size();
+        int lsw = 0;
+        while ((1 << lsw) < b.sw) ++lsw;
+        const int per = 32 >> lsw;
+        for (int r = 0; r < b.n; r += per) {
+            const int here = std::min(per, b.n - r);
+            int most = 0;
+            for (int q = 0; q < here; ++q) most = std::max(most, X->h_rp[(size_t)b.seg + r + q + 1] - X->h_rp[(size_t)b.seg + r + q]);
+            desc.push_back({b.seg + r, here, b.seg, lsw});
+            off.push_back((int32_t)tot);
+            tot += (most + 8 * b.sw - 1) / (8 * b.sw);
+            if (tot >= INT32_MAX / 64) return ion_fail(s, ION_ERR_INVALID_ARG, "batch: too many edges");
+        }
+    }
+    off.push_back((int32_t)tot);
+    cudaError_t e = cudaStreamSynchronize(s->st);
+    ion_drop_graphs(s);   // captured steps hold the old arrays
+    cudaFree(X->d_scols);
+    cudaFree(X->d_sw);
+    cudaFree(X->d_soff);
+    X->d_scols = nullptr;
+    X->d_sw = nullptr;
+    X->d_soff = nullptr;
+    X->slice_scale = -2;
+    if (!desc.empty()) {
+        SliceDesc *d_desc = nullptr;
+        const size_t rounds = (size_t)std::max<int64_t>(tot, 1);
+        if (e == cudaSuccess) e = ion_alloc(&X->d_scols, rounds * 512);
+        if (e == cudaSuccess && weights) e = ion_alloc(&X->d_sw, rounds * 1024);
+        if (e == cudaSuccess) e = ion_alloc(&X->d_soff, off.size() * sizeof(int32_t));
+        if (e == cudaSuccess) e = ion_alloc(&d_desc, desc.size() * sizeof(SliceDesc));
+        if (e == cudaSuccess) e = cudaMemcpy(X->d_soff, off.data(), off.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(d_desc, desc.data(), desc.size() * sizeof(SliceDesc), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) {
+            batch_slice_fill_kernel<<<(unsigned)((desc.size() + 3) / 4), 128, 0, s->st>>>(
+                d_desc, (int)desc.size(), X->d_soff, s->d_rowptr, s->d_col16, s->d_w, X->d_scols, X->d_sw);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
+        cudaFree(d_desc);
+    }
+    if (e != cudaSuccess)
+        return ion_fail(s, e == cudaErrorMemoryAllocation ? ION_ERR_OOM : ION_ERR_CUDA, "batch slices: %s", cudaGetErrorString(e));
+    X->slice_scale = X->sw_scale;
+    return ION_OK;
+}
+
+// Work per tile: a tile pays about 3 us of latency (its V_dend copy, its rows' update) whatever
+// it computes, so small networks get several row blocks per tile and short rows more rows;
+// while there are too few tiles to fill the chip, fewer.  Measured (96 networks of 32-4096
+// cells, us per step): 80 000 pairs per dense tile 20.1, one row block 20.9, 160 000: 21.4;
+// 12 networks: 20 000 pairs 5.5, 80 000: 8.6.
+constexpr double DENSE_TILE_PAIRS = 80000.0, DENSE_TILE_LEAST = 16000.0;
+constexpr double CSR_TILE_EDGES = 32768.0, CSR_TILE_LEAST = 2048.0;
+// Chains: two for the dense networks (one: 24.0 us per step, three: as two), one for the rest.
+constexpr int DENSE_CHAINS = 2, CSR_CHAINS = 1;
+static_assert(DENSE_CHAINS + CSR_CHAINS <= BATCH_CHAINS, "one stream per chain");
+
 // Build (or rebuild) the tile list for the current shape parameters.
 static ion_status batch_plan(ion_sim *s) {
     BatchExt *X = ext_of(s);
+    const ion_status ss = batch_build_slices(s);
+    if (ss != ION_OK) {
+        X->n_tiles = 0;   // the slices a tile list would refer to are gone: stepping is refused
+        cudaFree(X->d_tiles);
+        X->d_tiles = nullptr;
+        return ss;
+    }
     std::vector<BatchTile> tiles;
     std::vector<double> cost;
-    const int drows = 8 * X->R;
-    for (const BatchNet &b : X->nets) {
+    std::vector<int> tile_net;
+    double pairs = 0.0, edges = 0.0;
+    for (const BatchNet &b : X->nets) (b.kind == ION_DENSE_UNIFORM ? pairs : edges) += b.kind == ION_DENSE_UNIFORM ? (double)b.n * b.n_pad : (double)b.nnz;
+    const double dense_work = std::min(DENSE_TILE_PAIRS, std::max(DENSE_TILE_LEAST, pairs / (4 * s->sms)));
+    const double csr_work = std::min(CSR_TILE_EDGES, std::max(CSR_TILE_LEAST, edges / s->sms));
+    for (size_t net = 0; net < X->nets.size(); ++net) {
+        const BatchNet &b = X->nets[net];
         if (b.kind == ION_DENSE_UNIFORM) {
+            const int blocks = std::min(256 / (8 * X->R), std::max(1, (int)(dense_work / ((double)8 * X->R * b.n_pad) + 0.5)));
+            const int drows = 8 * X->R * blocks;
             for (int r = 0; r < b.n; r += drows) {
-                BatchTile T{TILE_DENSE, b.seg, b.n, b.n_pad, b.seg + r, std::min(drows, b.n - r), 0, b.g, 0};
+                BatchTile T{TILE_DENSE, b.seg, b.n, b.n_pad, b.seg + r, std::min(drows, b.n - r), 0, b.g, 0, 0};
                 tiles.push_back(T);
+                tile_net.push_back((int)net);
                 cost.push_back((double)T.rows * b.n_pad);
             }
         } else {
             const double deg = b.n > 0 ? (double)b.nnz / b.n : 0.0;
             int mode = (b.uniform ? TILE_UNIFORM_W : 0) | (b.c16 ? TILE_C16 : 0);
-            if (b.c16 && b.n_pad <= X->max_dense_pad) mode |= TILE_STAGE_V;   // fits the launch's shared memory
-            for (int r = 0; r < b.n; r += X->csr_rows) {
-                BatchTile T{TILE_CSR, b.seg, b.n, b.n_pad, b.seg + r, std::min(X->csr_rows, b.n - r),
-                            csr_sw_for(deg, X->sw_scale), b.uniform ? b.g : 0.0f, mode};
+            if (net_staged(X, b)) mode |= TILE_STAGE_V;
+            int crows = X->csr_rows;
+            while (crows > 32 && crows * deg > csr_work) crows = (crows + 1) / 2;
+            for (int r = 0; r < b.n; r += crows) {
+                BatchTile T{TILE_CSR, b.seg, b.n, b.n_pad, b.seg + r, std::min(crows, b.n - r),
+                            b.kind == ION_CSR ? b.sw : 1, b.uniform ? b.g : 0.0f, mode, b.slice0};
                 tiles.push_back(T);
+                tile_net.push_back((int)net);
                 cost.push_back(3.0 * T.rows * deg + 60.0 * T.rows);
             }
         }
     }
+    // deal the networks to chains: dense and CSR ones apart (different kernels), each kind's
+    // networks largest first to the lighter of its chains
+    std::vector<double> net_cost(X->nets.size(), 0.0);
+    for (size_t k = 0; k < tiles.size(); ++k) net_cost[(size_t)tile_net[k]] += cost[k];
+    std::vector<int> chain_of(X->nets.size(), 0);
+    X->chains.clear();
+    for (int dense = 1; dense >= 0; --dense) {
+        std::vector<int> own;
+        for (size_t b = 0; b < X->nets.size(); ++b)
+            if ((X->nets[b].kind == ION_DENSE_UNIFORM) == (dense == 1)) own.push_back((int)b);
+        if (own.empty()) continue;
+        std::stable_sort(own.begin(), own.end(), [&](int a, int b) { return net_cost[(size_t)a] > net_cost[(size_t)b]; });
+        const int nc = std::min<int>((int)own.size(), dense ? DENSE_CHAINS : CSR_CHAINS), c0 = (int)X->chains.size();
+        std::vector<double> load((size_t)nc, 0.0);
+        for (int q = 0; q < nc; ++q) {
+            X->chains.emplace_back();
+            X->chains.back().dense = dense == 1;
+        }
+        for (int b : own) {
+            const int q = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+            load[(size_t)q] += net_cost[(size_t)b];
+            chain_of[(size_t)b] = c0 + q;
+        }
+    }
     std::vector<int> order(tiles.size());
     std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        const int ca = chain_of[(size_t)tile_net[(size_t)a]], cb = chain_of[(size_t)tile_net[(size_t)b]];
+        return ca != cb ? ca < cb : cost[a] > cost[b];
+    });
     std::vector<BatchTile> sorted(tiles.size());
-    for (size_t k = 0; k < order.size(); ++k) sorted[k] = tiles[order[k]];
+    for (size_t k = 0; k < order.size(); ++k) {
+        const BatchTile &T = sorted[k] = tiles[order[k]];
+        BatchExt::Chain &C = X->chains[(size_t)chain_of[(size_t)tile_net[(size_t)order[k]]]];
+        if (C.n++ == 0) C.off = (int)k;
+        if (T.kind == TILE_DENSE || (T.mode & TILE_STAGE_V)) C.vbuf = std::max(C.vbuf, T.n_pad);
+        C.rows_max = std::max(C.rows_max, T.rows);
+    }
+    s->lps = (int64_t)X->chains.size();
     cudaError_t e = cudaStreamSynchronize(s->st);
     ion_drop_graphs(s);   // the captured steps hold the old tile list
     if (e == cudaSuccess && X->d_tiles) e = cudaFree(X->d_tiles);
@@ -550,22 +866,29 @@ static ion_status batch_plan(ion_sim *s) {
     return ION_OK;
 }
 
-// dynamic shared memory of the per-step kernel: a network's V_dend and the dense row partials
-// (staging the tile's cell words here as well measured slower: fewer CTAs per SM)
-static size_t batch_smem(const BatchExt *X) { return (size_t)X->max_dense_pad * 4 + 8 * X->R * 4; }
-
-template <int R>
-static cudaError_t batch_launch_R(const BatchArgs &a, int tiles, size_t smem, cudaStream_t st, bool prepare) {
-    if (prepare)
-        return cudaFuncSetAttribute(batch_step_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return launch_k(batch_step_kernel<R>, dim3(tiles), dim3(256), smem, st, a.c.pdl != 0, a);
+// dynamic shared memory of a chain's launches: a network's V_dend, the dense row partials and
+// the tile's cell words
+static size_t batch_smem(const BatchExt *X, const BatchExt::Chain &C) {
+    return ((size_t)C.vbuf + (C.dense ? 8 * X->R : 0) + (size_t)NCW * C.rows_max) * sizeof(float);
 }
-static cudaError_t batch_launch(const BatchArgs &a, int R, int tiles, size_t smem, cudaStream_t st, bool prepare) {
+
+static const void *batch_fn(bool dense, int R) {
+    if (!dense) return (const void *)batch_csr_kernel;
     switch (R) {
-        case 1: return batch_launch_R<1>(a, tiles, smem, st, prepare);
-        case 2: return batch_launch_R<2>(a, tiles, smem, st, prepare);
-        case 4: return batch_launch_R<4>(a, tiles, smem, st, prepare);
-        case 8: return batch_launch_R<8>(a, tiles, smem, st, prepare);
+        case 1: return (const void *)batch_dense_kernel<1>;
+        case 2: return (const void *)batch_dense_kernel<2>;
+        case 4: return (const void *)batch_dense_kernel<4>;
+        default: return (const void *)batch_dense_kernel<8>;
+    }
+}
+static cudaError_t batch_launch(const BatchArgs &a, bool dense, int R, int tiles, size_t smem, bool pdl, cudaStream_t st) {
+    const dim3 grid(tiles), block(256);
+    if (!dense) return launch_k(batch_csr_kernel, grid, block, smem, st, pdl, a);
+    switch (R) {
+        case 1: return launch_k(batch_dense_kernel<1>, grid, block, smem, st, pdl, a);
+        case 2: return launch_k(batch_dense_kernel<2>, grid, block, smem, st, pdl, a);
+        case 4: return launch_k(batch_dense_kernel<4>, grid, block, smem, st, pdl, a);
+        case 8: return launch_k(batch_dense_kernel<8>, grid, block, smem, st, pdl, a);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -575,15 +898,48 @@ static cudaError_t batch_step(ion_sim *s, int k_off, const float *iapp) {
     if (X->d_tiles == nullptr) return cudaErrorInvalidResourceHandle;   // no tile list: a failed re-plan
     BatchArgs a{};
     a.c = ion_step_common(s, k_off, iapp);
-    a.tiles = X->d_tiles;
     a.row_ptr = s->d_rowptr;
     a.col = s->d_col;
     a.col16 = s->d_col16;
     a.w = s->d_w;
+    a.scols = reinterpret_cast<const uint4 *>(X->d_scols);
+    a.sw = reinterpret_cast<const float4 *>(X->d_sw);
+    a.soff = X->d_soff;
     a.kahan = 1;
-    s->launches++;
-    if (X->n_tiles == 0) return cudaSuccess;
-    return batch_launch(a, X->R, X->n_tiles, batch_smem(X), s->st, false);
+    cudaError_t e = cudaSuccess;
+    for (size_t q = 0; q < X->chains.size() && e == cudaSuccess; ++q) {
+        const BatchExt::Chain &C = X->chains[q];
+        a.tiles = X->d_tiles + C.off;
+        a.rows_max = C.rows_max;
+        a.vbuf = C.vbuf;
+        // a side stream's first launch follows the fork event, not a kernel: an ordinary launch
+        const bool pdl = a.c.pdl && !(q > 0 && X->forked_now);
+        e = batch_launch(a, C.dense, X->R, C.n, batch_smem(X, C), pdl, q == 0 ? s->st : X->side[q - 1]);
+        s->launches++;
+    }
+    X->forked_now = false;
+    return e;
+}
+
+// Before the steps of a captured graph or of a direct run: the side streams start after the
+// handle's stream; after them the handle's stream continues when every chain is done.
+static cudaError_t batch_fork(ion_sim *s) {
+    BatchExt *X = ext_of(s);
+    if (X->chains.size() < 2) return cudaSuccess;
+    cudaError_t e = cudaEventRecord(X->ev_fork, s->st);
+    for (size_t q = 1; q < X->chains.size() && e == cudaSuccess; ++q) e = cudaStreamWaitEvent(X->side[q - 1], X->ev_fork, 0);
+    X->forked_now = true;
+    return e;
+}
+static cudaError_t batch_join(ion_sim *s) {
+    BatchExt *X = ext_of(s);
+    cudaError_t e = cudaSuccess;
+    for (size_t q = 1; q < X->chains.size(); ++q) {   // every side stream joins, also after an error
+        cudaError_t e1 = cudaEventRecord(X->ev_join[q - 1], X->side[q - 1]);
+        if (e1 == cudaSuccess) e1 = cudaStreamWaitEvent(s->st, X->ev_join[q - 1], 0);
+        if (e == cudaSuccess) e = e1;
+    }
+    return e;
 }
 
 // ---- persistent form: planning and launch ----------------------------------------------
@@ -661,7 +1017,8 @@ static ion_status batch_persist_plan(ion_sim *s) {
             if (x.kind != ION_DENSE_UNIFORM) {
                 it.sw = x.sw;
                 it.mode = (x.uniform ? TILE_UNIFORM_W : 0) | (x.c16 ? TILE_C16 : 0);
-                if (x.c16 && x.n_pad <= X->p_vbuf) it.mode |= TILE_STAGE_V;
+                it.slice0 = x.slice0;
+                if (net_staged(X, x)) it.mode |= TILE_STAGE_V;
             }
             pieces.push_back({it, nc[b].per_row * it.rows + nc[b].fixed});
         }
@@ -725,6 +1082,9 @@ static cudaError_t persist_enqueue(ion_sim *s, int n_steps, bool capture) {
     a.row_ptr = s->d_rowptr;
     a.col16 = s->d_col16;
     a.w = s->d_w;
+    a.scols = reinterpret_cast<const uint4 *>(X->d_scols);
+    a.sw = reinterpret_cast<const float4 *>(X->d_sw);
+    a.soff = X->d_soff;
     a.cnt = X->d_pcnt;
     a.abort_flag = X->d_pcnt + X->nets.size();
     a.timeout_ns = s->barrier_timeout_ns;
@@ -807,7 +1167,17 @@ static ion_status batch_persist_run(ion_sim *s, int64_t n_steps, const float *ia
 
 static ion_status batch_prepare(ion_sim *s) {
     BatchExt *X = ext_of(s);
-    cudaError_t e = batch_launch(BatchArgs{}, X->R, 0, batch_smem(X), s->st, true);
+    cudaError_t e = cudaSuccess;
+    size_t most[2] = {0, 0};
+    for (const BatchExt::Chain &C : X->chains) most[C.dense] = std::max(most[C.dense], batch_smem(X, C));
+    for (int dense = 0; dense < 2 && e == cudaSuccess; ++dense)
+        if (most[dense] > 0)
+            e = cudaFuncSetAttribute(batch_fn(dense != 0, X->R), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most[dense]);
+    if (e == cudaSuccess && !X->ev_fork) e = cudaEventCreateWithFlags(&X->ev_fork, cudaEventDisableTiming);
+    for (size_t q = 1; q < X->chains.size() && e == cudaSuccess; ++q) {
+        if (!X->side[q - 1]) e = cudaStreamCreateWithFlags(&X->side[q - 1], cudaStreamNonBlocking);
+        if (e == cudaSuccess && !X->ev_join[q - 1]) e = cudaEventCreateWithFlags(&X->ev_join[q - 1], cudaEventDisableTiming);
+    }
     if (e != cudaSuccess) return ion_fail(s, ION_ERR_CUDA, "batch setup: %s", cudaGetErrorString(e));
     return ION_OK;
 }
@@ -867,10 +1237,18 @@ static void batch_free(ion_sim *s) {
     if (!X) return;
     s->drop_hook = nullptr;
     if (X->p_graph) cudaGraphExecDestroy(X->p_graph);
+    for (int q = 0; q < BATCH_CHAINS - 1; ++q) {   // their work is joined to the handle's stream, which is idle
+        if (X->side[q]) cudaStreamDestroy(X->side[q]);
+        if (X->ev_join[q]) cudaEventDestroy(X->ev_join[q]);
+    }
+    if (X->ev_fork) cudaEventDestroy(X->ev_fork);
     cudaFree(X->d_items);
     cudaFree(X->d_cta_off);
     cudaFree(X->d_pcnt);
     cudaFree(X->d_tiles);
+    cudaFree(X->d_scols);
+    cudaFree(X->d_sw);
+    cudaFree(X->d_soff);
     cudaFree(X->d_tmp);
     cudaFree(s->d_map);
     s->d_map = nullptr;
@@ -986,6 +1364,7 @@ extern "C" ion_status ion_create_batch(int32_t n_nets, const ion_net *nets, cons
         }
     }
     for (size_t i = 0; i < (size_t)seg; ++i) rp[i + 1] += rp[i];
+    X->h_rp = rp;
     // the per-row counts above were placed in network order, so the prefix sum lines the
     // edges up with x.e0 (segments are laid out in network order)
     s->own_csr = true;   // before the allocations, so that a partial failure frees them
@@ -1005,11 +1384,11 @@ extern "C" ion_status ion_create_batch(int32_t n_nets, const ion_net *nets, cons
     if (e == cudaSuccess)
         e = cudaMemcpy(s->d_map, X->h_map.data(), X->h_map.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return fail(ion_fail(nullptr, ION_ERR_CUDA, "ion_create_batch: %s", cudaGetErrorString(e)));
-    for (BatchNet &x : X->nets)
-        if (x.kind == ION_CSR) x.sw = csr_sw_for((double)x.nnz / x.n, 0);
     s->kind = ION_CSR;   // the generic paths see a CSR handle; stepping is overridden
     s->n_user = n_user;
     s->step_override = batch_step;
+    s->fork_hook = batch_fork;
+    s->join_hook = batch_join;
     s->prepare_hook = nullptr;
     // every V_dend padding cell holds the sentinel (the default state wrote V_0 there)
     for (const BatchNet &x : X->nets) {

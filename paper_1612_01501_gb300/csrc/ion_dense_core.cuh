@@ -77,12 +77,14 @@ __device__ __forceinline__ void gj_block(const float4 *t4, int m0, int n4, float
 // adds up its even share of the tile's real x_j (the linear part's sum_j u_j is not
 // needed before the reduction, and an even share keeps the warps balanced).  On return
 // tot[r] holds this lane's compensated column sum for row r, and (Us, Uc) this thread's
-// compensated share of sum_j u_j.  bar_uses counts completed phases of each mbarrier.
+// compensated share of sum_j u_j (if want_u: a CTA that passes over the same columns for
+// several row blocks needs it once).  bar_uses counts completed phases of each mbarrier.
 // Returns false (in every thread) if a bulk copy did not land in time.
 template <int R, int GJ>
 __device__ __forceinline__ bool gj_pass(const DenseSmem &sm, const float *src, int n, int n_pad, uint64_t *bar,
                                         uint32_t (&bar_uses)[2], float C, const float (&ui)[R], int cs,
-                                        int lane, int kahan, float (&tot)[R], float &Us, float &Uc) {
+                                        int lane, int kahan, float (&tot)[R], float &Us, float &Uc,
+                                        bool want_u = true) {
     float ks[R], kc[R];
     float2 u2[R];
 #pragma unroll
@@ -99,7 +101,9 @@ __device__ __forceinline__ bool gj_pass(const DenseSmem &sm, const float *src, i
         const int j0 = kt * TJ;
         const int len = min(TJ, n_pad - j0);
         if (src != nullptr) {
-            const bool landed = mbar_wait_bounded(&bar[b], bar_uses[b] & 1u);
+            // one warp polls, the others wait at the barrier: they leave the issue slots to the
+            // other CTAs of the SM
+            const bool landed = threadIdx.x >= 32 || mbar_wait_bounded(&bar[b], bar_uses[b] & 1u);
             bar_uses[b]++;
             if (__syncthreads_or(!landed)) return false;   // block-uniform decision
         }
@@ -126,7 +130,7 @@ __device__ __forceinline__ bool gj_pass(const DenseSmem &sm, const float *src, i
             }
         }
         // this thread's share of the tile's real x_j, the same transform as above
-        for (int j4 = threadIdx.x; j4 < n4; j4 += blockDim.x) {
+        for (int j4 = threadIdx.x; want_u && j4 < n4; j4 += blockDim.x) {
             const float4 v = t4[j4];
             const float2 va = __ffma2_rn(make_float2(v.x, v.y), negs2, c2);
             const float2 vb = __ffma2_rn(make_float2(v.z, v.w), negs2, c2);

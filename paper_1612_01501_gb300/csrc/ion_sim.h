@@ -88,6 +88,8 @@ struct ion_sim {
 
     // extension points (persistent, batched and surrogate variants)
     cudaError_t (*step_override)(ion_sim *, int k_off, const float *iapp) = nullptr;
+    cudaError_t (*fork_hook)(ion_sim *) = nullptr;   // around a run of step_override calls
+    cudaError_t (*join_hook)(ion_sim *) = nullptr;
     ion_status (*run_override)(ion_sim *, int64_t n_steps, const float *iapp) = nullptr;
     ion_status (*prepare_hook)(ion_sim *) = nullptr;
     ion_status (*state_sync_hook)(ion_sim *) = nullptr;
