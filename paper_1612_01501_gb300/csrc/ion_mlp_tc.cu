@@ -6,10 +6,14 @@
 // evaluates the MLP for their three compartments (V_dend, V_soma, V_axon, each with the
 // cell's [Ca]) as three 128-row tiles: row t of every tile is cell t of the CTA, so thread
 // t ends up holding all three compartments' rates and runs that cell's explicit-Euler
-// update itself.  The tiles go through the two layers one after the other (a version
-// that pushed all three through each layer together, two tensor-core waits per step
-// instead of six, measured slower: it needs twice the TMEM and shared memory per CTA, so
-// half as many CTAs share an SM):
+// update itself.  The tiles are pipelined through two operand buffers: while the tensor core
+// works on one compartment the threads run another's layer 1, epilogue or update, so that
+// of the six completions only the first is waited for with nothing to do.  (The floor is the
+// 192 tanh.bf16x2 of a cell: 5.0 us per step at 65 536 cells.  One tile after the other, the
+// update at the end, this launch took 14.4 us of a step there; pipelined 13.4; with the TMEM
+// allocation and its permit's release before the weights' copy 11.2: the next CTA of an SM
+// does not start while one holds the permit.  All three tiles through a layer together needs
+// a third operand buffer, and then only three CTAs share an SM.)
 //   layer 1 (2 -> 64) in FP32 on the CUDA cores, tanh on packed bf16 pairs, written to
 //     shared memory as the three BF16 A operands of layer 2;
 //   layer 2 (64 x 64): four tcgen05.mma.kind::f16 (M = 128, N = 64, K = 16 each, BF16 in,
@@ -40,8 +44,7 @@ constexpr int ROWS = 128;        // M of every MMA: rows (cells) per CTA
 constexpr int KH = 64;           // hidden width (K of layers 2 and 3)
 constexpr int N2 = 64, N3 = 32;  // layer 2 outputs; layer 3 outputs (24) padded to a multiple of 16
 constexpr int NOUT = ION_MLP_OUT;
-constexpr int NT = 1;                 // tiles through a layer at once (see above)
-constexpr uint32_t TMEM_COLS = 128;   // layer 2: tile c in [64 c, 64 c + 64); layer 3: [32 c, 32 c + 32)
+constexpr uint32_t TMEM_COLS = 128;   // buffer b: layer 2 in columns [64 b, 64 b + 64), layer 3 in the first 32 of them
 constexpr float LOG2E = 1.4426950408889634f;
 
 __host__ __device__ constexpr int core_off(int row, int kchunk) {
@@ -56,11 +59,11 @@ struct Weights {
     float in_shift[2], in_scale[2], out_shift[N3], out_scale[N3];
 };
 struct Smem {
-    __nv_bfloat16 a[NT][ROWS * KH];   // A of layer 2, then of layer 3, per tile
+    __nv_bfloat16 a[2][ROWS * KH];    // A of layer 2, then of layer 3, per buffer
     Weights W;
-    uint64_t bar;
+    uint64_t bar[2];                  // completions of a buffer's MMAs
+    uint64_t wbar;                    // the weights' copy
     uint32_t tmem;
-    int ok;
 };
 static_assert(sizeof(Weights) % 16 == 0, "weights are copied 16 bytes at a time");
 static_assert(offsetof(Smem, W) % 16 == 0, "16-byte aligned operands");
@@ -126,24 +129,26 @@ __device__ __forceinline__ uint32_t tanh_bf16x2(uint32_t x) {
     return y;
 }
 
-// Issue one layer for `tiles` tiles (four K = 16 steps each; tile c's accumulator at TMEM
-// column d_tmem + c * d_stride) from thread 0 and wait for it in every thread.  Returns
-// false (in every thread) if the completion did not arrive in time.
-__device__ __forceinline__ bool tc_layer(Smem &sm, int tiles, const __nv_bfloat16 *B, uint32_t d_tmem,
-                                         uint32_t d_stride, uint32_t idesc, uint32_t &phase) {
+// Hand buffer b to the tensor core (all threads): its generic writes are ordered before the
+// asynchronous reads, then thread 0 issues the layer's four K = 16 steps and the commit.
+__device__ __forceinline__ void tc_issue(Smem &sm, int b, const __nv_bfloat16 *B, uint32_t idesc) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
     if (threadIdx.x == 0) {
         tc_fence_after();
-        for (int c = 0; c < tiles; ++c)
 #pragma unroll
-            for (int kk = 0; kk < KH / 16; ++kk)
-                tc_mma(d_tmem + c * d_stride, smem_desc(sm.a[c] + kk * 16 * 8, 128, 1024),
-                       smem_desc(B + kk * 16 * 8, 128, 1024), idesc, kk > 0 ? 1u : 0u);
-        tc_commit(&sm.bar);
+        for (int kk = 0; kk < KH / 16; ++kk)
+            tc_mma(sm.tmem + b * N2, smem_desc(sm.a[b] + kk * 16 * 8, 128, 1024), smem_desc(B + kk * 16 * 8, 128, 1024),
+                   idesc, kk > 0 ? 1u : 0u);
+        tc_commit(&sm.bar[b]);
     }
-    const bool done = mbar_wait_bounded(&sm.bar, phase & 1u);
-    phase++;
+}
+// Wait (bounded) for the layer last issued on buffer b; false if it did not complete in time.
+__device__ __forceinline__ bool tc_wait(Smem &sm, int b, uint32_t phase) {
+    const bool done = mbar_wait_bounded(&sm.bar[b], phase);
     tc_fence_after();
-    return !__syncthreads_or(!done);
+    return done;
 }
 
 // Layer 1 of one row of tile c: z = W1 x + b1 (FP32), tanh on bf16 pairs, into A (core-matrix layout).
@@ -185,18 +190,19 @@ __device__ __forceinline__ void layer2_epilogue(Smem &sm, int c, uint32_t lane_a
     }
 }
 
-// CTA prologue: weights into shared memory, mbarrier, TMEM columns (warp 0).
+// CTA prologue: TMEM columns (warp 0), weights into shared memory by one bulk copy, mbarriers.
+// The weights are waited for where they are first read (tc_weights).
 __device__ __forceinline__ void tc_setup(Smem &sm, const Weights *Wg) {
-    const int4 *s = reinterpret_cast<const int4 *>(Wg);
-    int4 *d = reinterpret_cast<int4 *>(&sm.W);
-    for (int i = threadIdx.x; i < (int)(sizeof(Weights) / 16); i += blockDim.x) d[i] = s[i];
-    if (threadIdx.x == 0) {
-        mbar_init(&sm.bar, 1);
-        fence_mbar_init();
-    }
     if (threadIdx.x < 32) {
         tmem_alloc(&sm.tmem, TMEM_COLS);
         tmem_relinquish();
+    } else if (threadIdx.x == 32) {
+        mbar_init(&sm.bar[0], 1);
+        mbar_init(&sm.bar[1], 1);
+        mbar_init(&sm.wbar, 1);
+        fence_mbar_init();
+        mbar_expect_tx(&sm.wbar, (uint32_t)sizeof(Weights));
+        bulk_g2s(&sm.W, Wg, (uint32_t)sizeof(Weights), &sm.wbar);
     }
     tc_fence_before();
     __syncthreads();
@@ -208,38 +214,29 @@ __device__ __forceinline__ void tc_teardown(Smem &sm) {
     if (threadIdx.x < 32) tmem_dealloc(sm.tmem, TMEM_COLS);
 }
 
-// Both MMA layers for `tiles` 128-row tiles with inputs (x0[c], x1) of this thread's row;
-// y[c] receives the 24 outputs of tile c in physical units.  Returns false if a completion
-// timed out (status bit set).
-__device__ __forceinline__ bool mlp_tiles(Smem &sm, int tiles, const float (&x0)[NT], float x1, uint32_t &phase,
-                                          float (&y)[NT][NOUT], uint32_t *status) {
-    const int row = threadIdx.x;
-    const uint32_t lane_addr = sm.tmem + ((uint32_t)(32 * (threadIdx.x >> 5)) << 16);
-    for (int c = 0; c < tiles; ++c) layer1_row(sm, c, row, x0[c], x1);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> tensor-core reads
-    tc_fence_before();
-    __syncthreads();
-    bool ok = tc_layer(sm, tiles, sm.W.w2, sm.tmem, N2, idesc_bf16(ROWS, N2), phase);
-    if (ok) {
-        for (int c = 0; c < tiles; ++c) layer2_epilogue(sm, c, lane_addr + c * N2, row);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_fence_before();
-        __syncthreads();
-        ok = tc_layer(sm, tiles, sm.W.w3, sm.tmem, N3, idesc_bf16(ROWS, N3), phase);
-    }
-    if (!ok) {
-        if (threadIdx.x == 0 && status != nullptr) atomicOr(status, (uint32_t)ST_TIMEOUT);
-        if (threadIdx.x == 0) (void)mbar_wait_bounded(&sm.bar, (phase - 1u) & 1u);   // the late MMAs, once more
-        return false;
-    }
-    for (int c = 0; c < tiles; ++c) {
-        float v[32];
-        tc_ld32(lane_addr + c * N3, v);
-        tc_wait_ld();
+// The lane of TMEM this thread reads back, in buffer b
+__device__ __forceinline__ uint32_t tc_lane(const Smem &sm, int b) {
+    return sm.tmem + b * N2 + ((uint32_t)(32 * (threadIdx.x >> 5)) << 16);
+}
+// The 24 outputs of this thread's row of buffer b in physical units (layer 3 done)
+__device__ __forceinline__ void tc_outputs(Smem &sm, int b, float (&y)[NOUT]) {
+    float v[32];
+    tc_ld32(tc_lane(sm, b), v);
+    tc_wait_ld();
 #pragma unroll
-        for (int o = 0; o < NOUT; ++o) y[c][o] = fmaf(v[o] + sm.W.b3[o], sm.W.out_scale[o], sm.W.out_shift[o]);
+    for (int o = 0; o < NOUT; ++o) y[o] = fmaf(v[o] + sm.W.b3[o], sm.W.out_scale[o], sm.W.out_shift[o]);
+}
+// After the last wait (all threads): reports a completion that did not come in time and waits
+// once more (bounded) for both buffers' MMAs, so that the TMEM they write can be freed.
+__device__ __forceinline__ bool tc_finish(Smem &sm, bool ok, uint32_t *status, uint32_t phase0, uint32_t phase1) {
+    if (!__syncthreads_or(!ok)) return true;
+    if (threadIdx.x == 0) {
+        if (status != nullptr) atomicOr(status, (uint32_t)ST_TIMEOUT);
+        (void)mbar_wait_bounded(&sm.bar[0], phase0);
+        (void)mbar_wait_bounded(&sm.bar[1], phase1);
+        (void)mbar_wait_bounded(&sm.wbar, 0u);
     }
-    return true;
+    return false;
 }
 
 __device__ __forceinline__ float learned_xinf(const float (&y)[NOUT], int gate) {
@@ -257,55 +254,94 @@ struct SurrTcArgs {
     const float *ic;    // gap currents of this step (NULL: none)
 };
 
-// The cell update with learned rates: 128 cells per CTA, three tensor-core tiles.
+// The cell update with learned rates: 128 cells per CTA, three tensor-core tiles (dendrite and
+// axon through buffer 0, soma through buffer 1).
 __global__ void __launch_bounds__(128) surrogate_tc_kernel(const SurrTcArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     tc::Smem &sm = *reinterpret_cast<tc::Smem *>(smem_raw);
-    tc::tc_setup(sm, a.W);   // weights and TMEM are not step data: before the dependency wait
-    pdl_enter();
     const StepCommon &c = a.c;
     const int64_t i = (int64_t)blockIdx.x * tc::ROWS + threadIdx.x;
     const bool valid = i < c.n;
-    const int64_t tstep = step_index(c);
+    tc::tc_setup(sm, a.W);   // weights, TMEM and pulses are not step data: before the dependency wait
+    const PulseAhead pa = pulse_ahead(c.pulses, i, valid);
+    pdl_enter();
+    const int64_t t = step_index(c);
     const float *vcur = vd_cur(c);
     float *vnext = vd_next(c);
     Cell cell{};
+    cell.vd = cell.vs = cell.va = -60.0f;
+    cell.ca = 1.0f;
     if (valid) cell = load_cell(c.S, vcur, i);
-    const float ca = valid ? cell.ca : 1.0f;
-    const float x1 = (logf(ca) - sm.W.in_shift[1]) * sm.W.in_scale[1];
-    CellRates gr;
-    uint32_t phase = 0;
-    bool ok = true;
-#pragma unroll 1
-    for (int comp = 0; comp < 3 && ok; ++comp) {
-        const float V = !valid ? -60.0f : (comp == 0 ? cell.vd : (comp == 1 ? cell.vs : cell.va));
-        const float x0[tc::NT] = {(V - sm.W.in_shift[0]) * sm.W.in_scale[0]};
-        float y[tc::NT][tc::NOUT];
-        ok = tc::mlp_tiles(sm, 1, x0, x1, phase, y, c.status);
-        if (comp == 0) {
-            gr.r = tc::learned_rate(y[0], G_R);
-            gr.s = tc::learned_rate(y[0], G_S);
-            gr.q = tc::learned_rate(y[0], G_Q);
-        } else if (comp == 1) {
-            gr.k = tc::learned_rate(y[0], G_K);
-            gr.l = tc::learned_rate(y[0], G_L);
-            gr.ms = Rate{tc::learned_xinf(y[0], G_MS), 0.0f};
-            gr.hs = tc::learned_rate(y[0], G_HS);
-            gr.ns = tc::learned_rate(y[0], G_NS);
-            gr.xs = tc::learned_rate(y[0], G_XS);
-        } else {
-            gr.ma = Rate{tc::learned_xinf(y[0], G_MA), 0.0f};
-            gr.ha = tc::learned_rate(y[0], G_HA);
-            gr.xa = tc::learned_rate(y[0], G_XA);
-        }
+    const float ic = valid && a.ic != nullptr ? a.ic[i] : 0.0f;
+    float iapp = pulse_current(c.pulses, pa, t);
+    if (c.iapp != nullptr && valid) iapp += c.iapp[i];
+    bool ok = mbar_wait_bounded(&sm.wbar, 0u);   // the weights
+    const int row = threadIdx.x;
+    const float dt = c.P.dt, x1 = (logf(cell.ca) - sm.W.in_shift[1]) * sm.W.in_scale[1];
+    auto x0 = [&](float V) { return (V - sm.W.in_shift[0]) * sm.W.in_scale[0]; };
+    constexpr uint32_t L2 = tc::idesc_bf16(tc::ROWS, tc::N2), L3 = tc::idesc_bf16(tc::ROWS, tc::N3);
+    float y[tc::NOUT];
+    tc::layer1_row(sm, 0, row, x0(cell.vd), x1);
+    tc::tc_issue(sm, 0, sm.W.w2, L2);
+    tc::layer1_row(sm, 1, row, x0(cell.vs), x1);
+    tc::tc_issue(sm, 1, sm.W.w2, L2);
+    ok = tc::tc_wait(sm, 0, 0u) && ok;
+    tc::layer2_epilogue(sm, 0, tc::tc_lane(sm, 0), row);
+    tc::tc_issue(sm, 0, sm.W.w3, L3);
+    ok = tc::tc_wait(sm, 1, 0u) && ok;
+    tc::layer2_epilogue(sm, 1, tc::tc_lane(sm, 1), row);
+    tc::tc_issue(sm, 1, sm.W.w3, L3);
+    // dendrite: its outputs, then the axon's layer 1 into the buffer they leave
+    ok = tc::tc_wait(sm, 0, 1u) && ok;
+    tc::tc_outputs(sm, 0, y);
+    tc::layer1_row(sm, 0, row, x0(cell.va), x1);
+    tc::tc_issue(sm, 0, sm.W.w2, L2);
+    bool finite = true;
+    if (valid) {
+        const DendNext d = dend_step(c.P, cell, ic, iapp);
+        vnext[i] = d.vd;
+        c.S.f(F_CA)[i] = d.ca;
+        c.S.f(F_ICAH)[i] = d.icah;
+        c.S.f(F_IC)[i] = ic;
+        c.S.f(F_R)[i] = relax(cell.r, tc::learned_rate(y, G_R), dt);
+        c.S.f(F_S)[i] = relax(cell.s, tc::learned_rate(y, G_S), dt);
+        c.S.f(F_Q)[i] = relax(cell.q, tc::learned_rate(y, G_Q), dt);
+        finite = isfinite(d.vd) && isfinite(d.ca);
     }
+    // soma
+    ok = tc::tc_wait(sm, 1, 1u) && ok;
+    tc::tc_outputs(sm, 1, y);
+    if (valid) {
+        const float ms = tc::learned_xinf(y, G_MS), vs = soma_step(c.P, cell, ms);
+        c.S.f(F_VSOMA)[i] = vs;
+        c.S.f(F_MS)[i] = ms;
+        c.S.f(F_K)[i] = relax(cell.k, tc::learned_rate(y, G_K), dt);
+        c.S.f(F_L)[i] = relax(cell.l, tc::learned_rate(y, G_L), dt);
+        c.S.f(F_HS)[i] = relax(cell.hs, tc::learned_rate(y, G_HS), dt);
+        c.S.f(F_NS)[i] = relax(cell.ns, tc::learned_rate(y, G_NS), dt);
+        c.S.f(F_XS)[i] = relax(cell.xs, tc::learned_rate(y, G_XS), dt);
+        finite = finite && isfinite(vs);
+    }
+    // axon
+    ok = tc::tc_wait(sm, 0, 0u) && ok;
+    tc::layer2_epilogue(sm, 0, tc::tc_lane(sm, 0), row);
+    tc::tc_issue(sm, 0, sm.W.w3, L3);
+    ok = tc::tc_wait(sm, 0, 1u) && ok;
+    tc::tc_outputs(sm, 0, y);
+    ok = tc::tc_finish(sm, ok, c.status, 1u, 1u);
     tc::tc_teardown(sm);
     if (!ok || !valid) return;
-    const float ic = a.ic != nullptr ? a.ic[i] : 0.0f;
-    float iapp = pulse_current(c.pulses, i, tstep);
-    if (c.iapp != nullptr) iapp += c.iapp[i];
-    const CellNext o = cell_step_rates(c.P, cell, ic, iapp, gr);
-    finish_cell(c, tstep, vnext, i, o);
+    const float ma = tc::learned_xinf(y, G_MA), va = axon_step(c.P, cell, ma);
+    c.S.f(F_VAXON)[i] = va;
+    c.S.f(F_MA)[i] = ma;
+    c.S.f(F_HA)[i] = relax(cell.ha, tc::learned_rate(y, G_HA), dt);
+    c.S.f(F_XA)[i] = relax(cell.xa, tc::learned_rate(y, G_XA), dt);
+    if (!finite || !isfinite(va)) atomicOr(c.status, (uint32_t)ST_NONFINITE);
+    if (c.par >= 0 && (int)(t & 1) != c.par) atomicOr(c.status, (uint32_t)ST_SLOT);
+    if (c.trace != nullptr && ((t + 1) % c.trace_stride) == 0) {
+        const int64_t sample = (t + 1) / c.trace_stride - 1;
+        c.trace[(sample % c.trace_cap) * (int64_t)c.n + i] = va;
+    }
 }
 
 // Batched evaluation: out[k * 24 + o] for n (V, [Ca]) pairs, 128 per CTA.
@@ -316,15 +352,27 @@ __global__ void __launch_bounds__(128) mlp_eval_tc_kernel(const tc::Weights *Wg,
     tc::tc_setup(sm, Wg);
     const int64_t k = (int64_t)blockIdx.x * tc::ROWS + threadIdx.x;
     const bool valid = k < n;
-    float x0[tc::NT] = {valid ? (V[k] - sm.W.in_shift[0]) * sm.W.in_scale[0] : 0.0f};
+    bool ok = mbar_wait_bounded(&sm.wbar, 0u);   // the weights
+    const float x0 = valid ? (V[k] - sm.W.in_shift[0]) * sm.W.in_scale[0] : 0.0f;
     const float x1 = valid ? (logf(ca[k]) - sm.W.in_shift[1]) * sm.W.in_scale[1] : 0.0f;
-    uint32_t phase = 0;
-    float y[tc::NT][tc::NOUT];
-    const bool ok = tc::mlp_tiles(sm, 1, x0, x1, phase, y, status);
-    tc::tc_teardown(sm);
-    if (!ok || !valid) return;
+    float y[tc::NOUT];
+    tc::layer1_row(sm, 0, threadIdx.x, x0, x1);
+    tc::tc_issue(sm, 0, sm.W.w2, tc::idesc_bf16(tc::ROWS, tc::N2));
+    ok = tc::tc_wait(sm, 0, 0u) && ok;
+    tc::layer2_epilogue(sm, 0, tc::tc_lane(sm, 0), threadIdx.x);
+    tc::tc_issue(sm, 0, sm.W.w3, tc::idesc_bf16(tc::ROWS, tc::N3));
+    ok = tc::tc_wait(sm, 0, 1u) && ok;
+    tc::tc_outputs(sm, 0, y);
+    if (!__syncthreads_or(!ok)) {
+        if (valid)
 #pragma unroll
-    for (int o = 0; o < tc::NOUT; ++o) out[k * tc::NOUT + o] = y[0][o];
+            for (int o = 0; o < tc::NOUT; ++o) out[k * tc::NOUT + o] = y[o];
+    } else if (threadIdx.x == 0) {
+        atomicOr(status, (uint32_t)ST_TIMEOUT);
+        (void)mbar_wait_bounded(&sm.bar[0], 1u);
+        (void)mbar_wait_bounded(&sm.wbar, 0u);
+    }
+    tc::tc_teardown(sm);
 }
 
 // Pack a host-layout surrogate (ion_surrogate_weights, FP32, row-major [out][in]) into the
