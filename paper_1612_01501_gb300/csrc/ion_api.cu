@@ -470,6 +470,8 @@ void ion_sim_free_device(ion_sim *s) {
     cudaFree(s->d_pamp);
     cudaFree(s->d_iapp);
     cudaFree(s->d_trace);
+    if (s->h_stage) cudaFreeHost(s->h_stage);
+    s->h_stage = nullptr;
     cudaFree(s->d_ic);
     cudaFree(s->d_cellp);
     s->d_cellp = nullptr;
@@ -936,6 +938,10 @@ static cudaError_t enqueue_run(ion_sim *s, int k, const float *iapp_base) {
     return e;
 }
 
+// The counter's advance follows a step kernel (not, with an extension's join, an event): it may
+// be scheduled while that drains.
+static bool advance_pdl(const ion_sim *s) { return !(s->flags & ION_FLAG_NO_PDL) && !s->pdl_off && !s->join_hook; }
+
 // Enqueue k steps directly (no graph) followed by the device counter advance.
 static cudaError_t enqueue_steps_direct(ion_sim *s, int64_t k, const float *iapp_base) {
     int64_t done = 0;
@@ -943,7 +949,7 @@ static cudaError_t enqueue_steps_direct(ion_sim *s, int64_t k, const float *iapp
         const int64_t chunk = std::min<int64_t>(k - done, 1 << 20);
         cudaError_t e = enqueue_run(s, (int)chunk, iapp_base ? iapp_base + done * (int64_t)s->n : nullptr);
         if (e != cudaSuccess) return e;
-        e = launch_advance(s->d_t, chunk, s->st);
+        e = launch_advance(s->d_t, chunk, s->st, advance_pdl(s));
         s->launches++;
         if (e != cudaSuccess) return e;
         s->t_enq += chunk;
@@ -958,7 +964,7 @@ static ion_status build_graph_once(ion_sim *s) {
     const int64_t launches0 = s->launches;
     ION_CK(s, cudaStreamBeginCapture(s->st, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = enqueue_run(s, K, nullptr);
-    if (e == cudaSuccess) e = launch_advance(s->d_t, K, s->st);
+    if (e == cudaSuccess) e = launch_advance(s->d_t, K, s->st, advance_pdl(s));
     cudaError_t e2 = cudaStreamEndCapture(s->st, &g);
     s->launches = launches0;
     if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -999,6 +1005,12 @@ extern "C" ion_status ion_step(ion_sim *s, int64_t n_steps, const ion_input *inp
         const int64_t cnt = n_steps * (int64_t)s->n;
         if (input->mem == ION_DEVICE) {
             iapp = input->dense;
+        } else if (s->h_stage && !s->input_busy && cnt <= ion_sim::STAGE) {
+            // a closed loop's input: the step kernels read it from pinned memory, early in the
+            // step; free again at the next synchronisation
+            std::memcpy(s->stage_input(), input->dense, (size_t)cnt * sizeof(float));
+            s->input_busy = true;
+            iapp = s->stage_input();
         } else {
             if (cnt > s->iapp_cap) {
                 ION_CK(s, cudaStreamSynchronize(s->st));
@@ -1057,17 +1069,37 @@ extern "C" ion_status ion_step(ion_sim *s, int64_t n_steps, const ion_input *inp
 }
 
 // ---- synchronisation and state I/O ----------------------------------------------------
-extern "C" ion_status ion_sync(ion_sim *s) {
-    if (!s) return ion_fail(nullptr, ION_ERR_INVALID_ARG, "ion_sync: NULL handle");
-    ION_CK(s, cudaStreamSynchronize(s->st));
-    uint32_t st = 0;
-    ION_CK(s, cudaMemcpy(&st, s->d_status, sizeof st, cudaMemcpyDeviceToHost));
-    s->sticky |= st;
+static ion_status sticky_status(ion_sim *s) {
     if (s->sticky & ST_TIMEOUT) return ion_fail(s, ION_ERR_TIMEOUT, "a bounded device wait timed out");
     if (s->sticky & ST_NONFINITE) return ion_fail(s, ION_ERR_NONFINITE, "non-finite voltage or [Ca] in the state");
     if (s->sticky & ST_SLOT)
         return ion_fail(s, ION_ERR_CUDA, "the device step counter and the host's step count disagree");
     return ION_OK;
+}
+
+extern "C" ion_status ion_sync(ion_sim *s) {
+    if (!s) return ion_fail(nullptr, ION_ERR_INVALID_ARG, "ion_sync: NULL handle");
+    ION_CK(s, cudaStreamSynchronize(s->st));
+    s->input_busy = false;
+    uint32_t st = 0;
+    ION_CK(s, cudaMemcpy(&st, s->d_status, sizeof st, cudaMemcpyDeviceToHost));
+    s->sticky |= st;
+    return sticky_status(s);
+}
+
+// A small read through the pinned buffer: one launch, one synchronisation.
+static ion_status read_staged(ion_sim *s, int32_t field, float *out, int64_t count) {
+    ION_CK(s, launch_state_put(ion_field_ptr(s, ION_V_DEND), s->d_state, s->stride, s->n, field, s->d_status, s->h_stage,
+                               ion_sim::STAGE, !(s->flags & ION_FLAG_NO_PDL) && !s->pdl_off, s->st));
+    ION_CK(s, cudaStreamSynchronize(s->st));
+    s->input_busy = false;
+    uint32_t st;
+    std::memcpy(&st, s->h_stage + ion_sim::STAGE, sizeof st);
+    s->sticky |= st;
+    const ion_status code = sticky_status(s);
+    if (code != ION_OK && code != ION_ERR_NONFINITE && code != ION_ERR_TIMEOUT) return code;
+    std::memcpy(out, s->h_stage, (size_t)count * sizeof(float));
+    return code;
 }
 
 float *ion_field_ptr(ion_sim *s, int32_t field) {
@@ -1095,6 +1127,17 @@ extern "C" ion_status ion_read_state(ion_sim *s, int32_t field, float *out, int6
     if (s->state_sync_hook) {
         ion_status st = s->state_sync_hook(s);
         if (st != ION_OK) return st;
+    }
+    // The pinned buffer costs about 300 us to make and give back, 15 us less per read: it is made
+    // at a handle's fourth small read.
+    if (!s->d_map && count <= ion_sim::STAGE) {
+        if (!s->h_stage && ++s->small_reads == 4 &&
+            cudaHostAlloc(reinterpret_cast<void **>(&s->h_stage), (2 * ion_sim::STAGE + 1) * sizeof(float),
+                          cudaHostAllocMapped) != cudaSuccess) {
+            s->h_stage = nullptr;
+            (void)cudaGetLastError();
+        }
+        if (s->h_stage) return read_staged(s, field, out, count);
     }
     const ion_status st = ion_sync(s);
     if (st != ION_OK && st != ION_ERR_NONFINITE && st != ION_ERR_TIMEOUT) return st;

@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(256) batch_dense_kernel(const BatchArgs a) {
             ui[r] = rr < T.rows ? gj_u(net_v[local0 + rr], C) : 0.0f;
         }
         float tot[R], Us, Uc;
-        if (!gj_pass<R, 1>(sm, sub == 0 ? net_v : nullptr, T.n, T.n_pad, bar, uses, C, ui, 0, lane, a.kahan, tot, Us, Uc,
+        if (!gj_pass<R, 1, true>(sm, sub == 0 ? net_v : nullptr, T.n, T.n_pad, bar, uses, C, ui, 0, lane, a.kahan, tot, Us, Uc,
                            sub == 0)) {
             if (threadIdx.x == 0) {
                 atomicOr(c.status, (uint32_t)ST_TIMEOUT);

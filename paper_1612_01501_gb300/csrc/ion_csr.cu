@@ -703,11 +703,33 @@ cudaError_t launch_default_state(const ModelF &P, float V0, float ca0, float gca
 }
 
 // ---- small helpers ------------------------------------------------------------------
-__global__ void advance_kernel(int64_t *t_dev, int64_t k) { *t_dev += k; }
+__global__ void advance_kernel(int64_t *t_dev, int64_t k) {
+    pdl_enter();
+    *t_dev += k;
+}
 
-cudaError_t launch_advance(int64_t *t_dev, int64_t k, cudaStream_t st) {
-    advance_kernel<<<1, 1, 0, st>>>(t_dev, k);
-    return cudaGetLastError();
+cudaError_t launch_advance(int64_t *t_dev, int64_t k, cudaStream_t st, bool pdl) {
+    return launch_k(advance_kernel, dim3(1), dim3(1), 0, st, pdl, t_dev, k);
+}
+
+// One field (or, field < 0, all of them) of n cells and the status word into a pinned host
+// buffer: one launch instead of two copies, each with a synchronisation of its own.
+__global__ void state_put_kernel(const float *vd, const float *base, int64_t stride, int n, int field,
+                                 const uint32_t *status, float *dst, int64_t status_at) {
+    pdl_enter();
+    const int total = field < 0 ? NF * n : n;
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < total) {
+        const int f = field < 0 ? q / n : field, i = field < 0 ? q - f * n : q;
+        dst[q] = f == 0 ? vd[i] : base[f * stride + i];
+    }
+    if (q == 0) reinterpret_cast<uint32_t *>(dst)[status_at] = *status;
+}
+cudaError_t launch_state_put(const float *vd, const float *base, int64_t stride, int n, int field, const uint32_t *status,
+                             float *dst, int64_t status_at, bool pdl, cudaStream_t st) {
+    const int total = field < 0 ? NF * n : n;
+    return launch_k(state_put_kernel, dim3((total + 255) / 256), dim3(256), 0, st, pdl, vd, base, stride, n, field, status,
+                    dst, status_at);
 }
 
 __global__ void fill_kernel(float *p, float v, int64_t n) {

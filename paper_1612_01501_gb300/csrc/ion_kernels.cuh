@@ -335,7 +335,9 @@ cudaError_t launch_csr_chunk_bounds(const int32_t *row_ptr, const int32_t *col, 
                                     int32_t *mid, cudaStream_t st);
 size_t csr_chunk_smem_bytes(int n_pad, int rows);
 cudaError_t launch_cell_step(const CellArgs &a, cudaStream_t st);
-cudaError_t launch_advance(int64_t *t_dev, int64_t k, cudaStream_t st);
+cudaError_t launch_advance(int64_t *t_dev, int64_t k, cudaStream_t st, bool pdl = false);
+cudaError_t launch_state_put(const float *vd, const float *base, int64_t stride, int n, int field, const uint32_t *status,
+                             float *dst, int64_t status_at, bool pdl, cudaStream_t st);
 cudaError_t launch_fill(float *p, float v, int64_t n, cudaStream_t st);
 cudaError_t launch_rates(float V, float ca, float *xinf_tau /*24 floats, device*/, cudaStream_t st);
 cudaError_t launch_default_state(const ModelF &P, float V0, float ca0, float gcal, int32_t n, int64_t stride,

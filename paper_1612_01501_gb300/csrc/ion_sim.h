@@ -40,6 +40,14 @@ struct ion_sim {
     int32_t n_pulses = 0;
     float *d_iapp = nullptr;
     int64_t iapp_cap = 0;
+    // a handle whose state is read again and again in small pieces (a closed loop) gets a pinned
+    // buffer that kernels read and write in place: STAGE floats of state out with the status
+    // word behind them, then STAGE floats of evoked input
+    static constexpr int64_t STAGE = 16384;
+    float *h_stage = nullptr;
+    int small_reads = 0;
+    bool input_busy = false;        // steps that read the staged input may still be in flight
+    float *stage_input() const { return h_stage + STAGE + 1; }
     // trace
     float *d_trace = nullptr;
     int32_t trace_stride = 0, trace_cap = 0;
