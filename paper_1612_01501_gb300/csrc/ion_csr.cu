@@ -644,9 +644,15 @@ cudaError_t launch_csr_col16(const int32_t *col, int64_t nnz, int64_t n_alloc, u
 // pulses).  The CTAs walk the cells in opposite directions on even and odd steps: the cells a
 // step ends with are still in L2 when the next begins with them, so up to L2's worth of the
 // state is neither read from nor written back to HBM.  2^21 cells with
-// pulses on a fifth: 46.8 us per step (0.92 of the measured copy rate in the bytes above), 53.6
-// in one direction only, 61.8 before with the pulse table read after the state
-__global__ void __launch_bounds__(256) cell_step_kernel(const CellArgs a) {
+// pulses on a fifth: 45.7 us per step (0.95 of the measured copy rate in the bytes above); 46.9
+// with CTAs of 256 threads, 53.6 in one direction only, 61.8 before with the pulse table read
+// after the state.
+//
+// CTAs of 128 threads at 51 registers: ten per SM, 1280 cells in flight, and a step's last CTAs
+// leave less of the chip idle than larger ones do (2^20 cells 21.1 -> 20.4 us, 16 384 cells
+// 1.93 -> 1.69).  Twelve per SM spill (2^21 cells 46.2 us), nine keep too little in flight (47.7).
+constexpr int CELL_THREADS = 128;
+__global__ void __launch_bounds__(CELL_THREADS, 10) cell_step_kernel(const CellArgs a) {
     const StepCommon &c = a.c;
     const int64_t b = c.par == 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
     const int64_t i = b * blockDim.x + threadIdx.x;
@@ -666,8 +672,8 @@ __global__ void __launch_bounds__(256) cell_step_kernel(const CellArgs a) {
 }
 
 cudaError_t launch_cell_step(const CellArgs &a, cudaStream_t st) {
-    const int64_t grid = ((int64_t)a.c.n + 255) / 256;
-    return launch_k(cell_step_kernel, dim3((unsigned)grid), dim3(256), 0, st, a.c.pdl != 0, a);
+    const int64_t grid = ((int64_t)a.c.n + CELL_THREADS - 1) / CELL_THREADS;
+    return launch_k(cell_step_kernel, dim3((unsigned)grid), dim3(CELL_THREADS), 0, st, a.c.pdl != 0, a);
 }
 
 // ---- rate functions and default state (host-visible copies of the device model) ----
