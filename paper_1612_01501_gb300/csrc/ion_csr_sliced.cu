@@ -386,22 +386,27 @@ ion_status ion_build_sliced(ion_sim *s, int lanes) {
     if (e != cudaSuccess) return done(e);
     std::vector<int32_t> off((size_t)(slices + pad) + 1);
     std::vector<uint16_t> rowid((size_t)(slices + pad) * per, (uint16_t)L.rows);
-    std::vector<std::pair<int32_t, int32_t>> len;   // (-edges, row)
+    std::vector<int32_t> order((size_t)L.rows), first;   // rows by falling edge count (a counting sort)
     int64_t tot = 0;
     for (int ch = 0; ch < C; ++ch)
         for (int b = 0; b < grid; ++b) {
             const int r0 = b * L.rows, here = std::min(L.rows, n - r0);
-            len.resize((size_t)here);
-            for (int r = 0; r < here; ++r)
-                len[(size_t)r] = {bound[(size_t)ch * n + r0 + r] - bound[(size_t)(ch + 1) * n + r0 + r], r};
-            std::sort(len.begin(), len.end());
+            auto edges = [&](int r) {
+                return bound[(size_t)(ch + 1) * n + r0 + r] - bound[(size_t)ch * n + r0 + r];
+            };
+            int32_t most = 0;
+            for (int r = 0; r < here; ++r) most = std::max(most, edges(r));
+            first.assign((size_t)most + 2, 0);
+            for (int r = 0; r < here; ++r) first[(size_t)(most - edges(r)) + 1]++;
+            for (int32_t k = 0; k <= most; ++k) first[(size_t)k + 1] += first[(size_t)k];
+            for (int r = 0; r < here; ++r) order[(size_t)first[(size_t)(most - edges(r))]++] = r;
             for (int q = 0; q < L.nsl; ++q) {
                 const int64_t base = ((int64_t)ch * grid + b) * L.nsl + q;
                 off[(size_t)base] = (int32_t)tot;
-                if (q * per < here) tot += (-len[(size_t)q * per].first + 8 * sw - 1) / (8 * sw);
+                if (q * per < here) tot += (edges(order[(size_t)q * per]) + 8 * sw - 1) / (8 * sw);
                 if (tot >= INT32_MAX / 64) return done(cudaSuccess);   // keep the unsliced layout
                 for (int r = 0; r < per && q * per + r < here; ++r)
-                    rowid[(size_t)base * per + r] = (uint16_t)len[(size_t)q * per + r].second;
+                    rowid[(size_t)base * per + r] = (uint16_t)order[(size_t)q * per + r];
             }
         }
     std::fill(off.begin() + slices, off.end(), (int32_t)tot);
