@@ -128,8 +128,8 @@ __global__ void __launch_bounds__(DenseBounds<R>::threads) dense_step_kernel(con
 // of the CTA's threads (each thread reads its cell, then a CTA barrier, then writes), else
 // one thread per cell.  V_dend(t+1) of the rows goes to the other global V_dend buffer and
 // the CTAs meet at a bounded grid barrier (a release flag, grid_barrier_flag) before
-// staging it for the next step.  With a single CTA and a single tile (small networks)
-// V_dend never leaves shared memory: the tile is updated in place.
+// staging it for the next step.  Networks of one CTA (up to DENSE_SMALL cells) have a kernel
+// of their own (ion_dense_small.cu), so this one always runs two CTAs or more.
 // Launch bounds of the persistent variant: 896 threads when R <= 4, else 576.
 template <int R>
 struct PersistBounds {
@@ -156,7 +156,6 @@ __global__ void __launch_bounds__(PersistBounds<R>::threads) dense_persist_kerne
     float *xs = cs + NCW * rows_cta;          // their m_s, m_a, I_CaH, I_c
     float *ic_s = xs + 4 * rows_cta;          // their gap currents
     const RoleOutSmem out{cs, xs, rows_cta};
-    const bool single = gridDim.x == 1 && sm.n_tiles == 1;
     const int row_base = blockIdx.x * rows_cta;
     const int rows_here = max(0, min(rows_cta, n - row_base));
     const int64_t t0 = *c.t_dev;
@@ -181,15 +180,6 @@ __global__ void __launch_bounds__(PersistBounds<R>::threads) dense_persist_kerne
     }
     __syncthreads();
     uint32_t uses[2] = {0u, 0u};
-    if (single && threadIdx.x == 0) issue_tile(sm, vd_slot(c.S, t0), c.n_pad, 0, bar);
-    if (single) {   // wait for the one initial copy; afterwards the tile is updated in place
-        const bool landed = mbar_wait_bounded(&bar[0], 0u);
-        uses[0] = 1;
-        if (__syncthreads_or(!landed)) {
-            if (threadIdx.x == 0) atomicOr(c.status, (uint32_t)ST_TIMEOUT);
-            return;
-        }
-    }
     if (a.debug_delay_ns > 0 && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
         const uint64_t d0 = globaltimer_ns();
         while (globaltimer_ns() - d0 < (uint64_t)a.debug_delay_ns) __nanosleep(1000);
@@ -200,10 +190,10 @@ __global__ void __launch_bounds__(PersistBounds<R>::threads) dense_persist_kerne
         const int64_t t = t0 + k;
         const float *vcur = vd_slot(c.S, t);
         float *vnext = vd_slot(c.S, t + 1);
-        if (!single && threadIdx.x == 0)
+        if (threadIdx.x == 0)
             for (int q = 0; q < 2 && q < sm.n_tiles; ++q) issue_tile(sm, vcur, c.n_pad, q, bar);
-        // shift m = V_dend of cell 0 at step t (from L2, or from the tile itself)
-        if (threadIdx.x == 0) m_sh = single ? sm.tile0[0] : __ldcg(vcur);
+        // shift m = V_dend of cell 0 at step t (from L2)
+        if (threadIdx.x == 0) m_sh = __ldcg(vcur);
         __syncthreads();
         const float C = m_sh * GJ_SCALE;
         float ui[R];
@@ -213,8 +203,7 @@ __global__ void __launch_bounds__(PersistBounds<R>::threads) dense_persist_kerne
             ui[r] = (rr < rows_here) ? gj_u(cs[rr], C) : 0.0f;
         }
         float tot[R], Us, Uc;
-        if (!gj_pass<R, GJ>(sm, single ? nullptr : vcur, n, c.n_pad, bar, uses, C, ui, csp, lane, a.kahan, tot,
-                            Us, Uc)) {
+        if (!gj_pass<R, GJ>(sm, vcur, n, c.n_pad, bar, uses, C, ui, csp, lane, a.kahan, tot, Us, Uc)) {
             if (threadIdx.x == 0) {
                 atomicOr(c.status, (uint32_t)ST_TIMEOUT);
                 atomicExch(a.abort_flag, 1u);
@@ -259,14 +248,9 @@ __global__ void __launch_bounds__(PersistBounds<R>::threads) dense_persist_kerne
             }
         }
         done = k + 1;
-        if (single) {
-            __syncthreads();                          // all pair loops are done with the tile
-            for (int rr = threadIdx.x; rr < rows_here; rr += blockDim.x) sm.tile0[rr] = cs[rr];
-            __syncthreads();
-        } else if (!grid_barrier_flag(a.bar_count, a.bar_flag, a.abort_flag, a.bar_base + (uint32_t)(k + 1) * gridDim.x,
-                                      a.timeout_ns, c.status, &ok_sh)) {
+        if (!grid_barrier_flag(a.bar_count, a.bar_flag, a.abort_flag, a.bar_base + (uint32_t)(k + 1) * gridDim.x,
+                               a.timeout_ns, c.status, &ok_sh))
             break;
-        }
     }
     // write the state back (after an aborted run: the CTA's last completed step)
     __syncthreads();

@@ -70,7 +70,7 @@ __device__ __forceinline__ void gj_block(const float4 *t4, int m0, int n4, float
 
 // One pass over all columns.  If `src` is non-NULL the first two tiles must already be in
 // flight (issue_tile) and the remaining ones are issued here; if NULL the single tile
-// already holds V_dend (single-CTA persistent mode).  The tiles hold raw V_dend: each lane
+// already holds V_dend (the batch kernels).  The tiles hold raw V_dend: each lane
 // centres, scales and negates the four columns of a 16-byte load as it reads them,
 // x_j = C - s V_j (gj_u), so there is no pass over the tile between its arrival and the pair
 // loop.  Columns past the last real cell are skipped.  After a tile's pairs, every warp
