@@ -452,83 +452,110 @@ cudaError_t launch_csr_chunk_bounds(const int32_t *row_ptr, const int32_t *col, 
     return cudaGetLastError();
 }
 
+constexpr int CELL_THREADS = 128;   // CTA of the kernels that only update cells (cell_step_kernel has the figures)
+
 // ---- simplified gap junctions (SGJ use case, Sec. 2.3.2) ---------------------------------
 // Each connection contributes w (V_i - V_j) (the small-dV limit of the RGJ term).
 // Dense: Ic_i = g sum_j (V_i - V_j) = g (N (V_i - m) - sum_j (V_j - m)), m = V_dend of cell 0
 // (shifted so nearly equal voltages do not cancel).  Larger networks take two launches
-// per step: P CTAs write Kahan partial sums of V_j - m over fixed strided ranges, then
-// every CTA of the update sums the P partials in index order and updates its cells
-// (deterministic).
-__global__ void __launch_bounds__(256) sgj_partial_kernel(const StepCommon c, float *part) {
-    __shared__ float red[8];
-    pdl_enter();
-    const int64_t t = step_index(c);
-    const float *vcur = vd_cur(c);
-    const float m = vcur[0];
-    float s = 0.0f, cc = 0.0f;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < c.n; j += (int64_t)gridDim.x * blockDim.x)
-        kahan_add(s, cc, vcur[j] - m);
-    float v = s - cc;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float tot = 0.0f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-        part[blockIdx.x] = tot;
-    }
+// per step: P CTAs write compensated partial sums of V_j - m over fixed strided ranges, then
+// every warp of the update sums the P partials in a fixed order and updates its cells
+// (deterministic).  Networks of at most SGJ_ONE_LAUNCH cells take one: every CTA sums V_j - m
+// over all cells itself, in the same order in every CTA.
+//
+// A step is bound by latency up to some 10^5 cells, by memory beyond.  So the sums run in four
+// chains per thread over 16-byte loads, the partials are added by all lanes (one thread adding
+// 256 of them held every CTA of the update for 2 us), the cells' words and pulses are on their
+// way before the sum is known, and the update walks the cells in opposite directions on even
+// and odd steps (cell_step_kernel).
+// Per step before / now: 200 cells 2.6 / 2.0 us, 8192 5.1 / 2.9, 16 384 7.1 / 3.7 (one launch),
+// 16 385 5.3 / 3.8, 100 003 7.4 / 5.5, 600 011 24.8 / 16.1, 1 211 904 57.4 / 30.1.
+__device__ __forceinline__ void two_sum_add(float &s, float &e, float so, float eo) {   // (s + e) += so + eo
+    const float t = s + so, b = t - s;
+    e = (e + eo) + ((s - (t - b)) + (so - b));
+    s = t;
 }
-// part == NULL (networks of at most SGJ_ONE_LAUNCH cells): every CTA sums V_j - m over all
-// cells itself, in one fixed order (the same in every CTA), so one launch does the step.
-__global__ void __launch_bounds__(256) sgj_dense_update_kernel(const StepCommon c, const float *part, int n_part,
-                                                               float g) {
-    __shared__ float U_sh;
+// sum of V_j - m over j = 4 first .. 4 first + 3, then every 4 stride on, of all threads of a
+// CTA of 256 (each gets it)
+__device__ __forceinline__ float sgj_block_sum(const float *v, int n, float m, int64_t first, int64_t stride) {
     __shared__ float red[8];
+    float s[4] = {}, cc[4] = {};
+#pragma unroll 4
+    for (int64_t j = 4 * first; j < n; j += 4 * stride) {   // the padding reaches a multiple of 256
+        const float4 x = *reinterpret_cast<const float4 *>(v + j);
+        kahan_add(s[0], cc[0], x.x - m);
+        kahan_add(s[1], cc[1], j + 1 < n ? x.y - m : 0.0f);
+        kahan_add(s[2], cc[2], j + 2 < n ? x.z - m : 0.0f);
+        kahan_add(s[3], cc[3], j + 3 < n ? x.w - m : 0.0f);
+    }
+    float S = s[0], E = -cc[0];
+#pragma unroll
+    for (int q = 1; q < 4; ++q) two_sum_add(S, E, s[q], -cc[q]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+        two_sum_add(S, E, __shfl_xor_sync(0xffffffffu, S, off), __shfl_xor_sync(0xffffffffu, E, off));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = S + E;
+    __syncthreads();
+    float tot = 0.0f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) tot += red[w];
+    return tot;
+}
+__global__ void __launch_bounds__(256) sgj_partial_kernel(const StepCommon c, float *part) {
     pdl_enter();
+    (void)step_index(c);
+    const float *vcur = vd_cur(c);
+    const float tot = sgj_block_sum(vcur, c.n, vcur[0], (int64_t)blockIdx.x * 256 + threadIdx.x, (int64_t)gridDim.x * 256);
+    if (threadIdx.x == 0) part[blockIdx.x] = tot;
+}
+// ONE: the whole step (part NULL).  Else the launch after sgj_partial_kernel, which lets this
+// one start only after it has itself waited for the previous step: the state is complete here,
+// and only the partial sums have to be waited for.
+template <bool ONE>
+__global__ void __launch_bounds__(ONE ? 256 : CELL_THREADS, ONE ? 1 : 10)
+    sgj_dense_update_kernel(const StepCommon c, const float *part, int n_part, float g) {
+    const int64_t b = !ONE && c.par == 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const int64_t i = b * blockDim.x + threadIdx.x;
+    const bool mine = i < c.n;
+    const PulseAhead pa = pulse_ahead(c.pulses, i, mine);
+    if (ONE) pdl_enter();
     const int64_t t = step_index(c);
     const float *vcur = vd_cur(c);
-    float *vnext = vd_next(c);
-    if (part == nullptr) {
-        const float m0 = vcur[0];
-        float s = 0.0f, cc = 0.0f;
-        for (int64_t j = threadIdx.x; j < c.n; j += blockDim.x) kahan_add(s, cc, vcur[j] - m0);
-        float v = s - cc;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float tot = 0.0f;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-            U_sh = tot;
-        }
-    } else if (threadIdx.x == 0) {
-        float s = 0.0f, cc = 0.0f;
-        for (int q = 0; q < n_part; ++q) kahan_add(s, cc, part[q]);
-        U_sh = s - cc;
-    }
-    __syncthreads();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= c.n) return;
     const float m = vcur[0];
-    const float ic = g * fmaf((float)c.n, vcur[i] - m, -U_sh);
-    const Cell cell = load_cell(c.S, vcur, i);
-    float iapp = pulse_current(c.pulses, i, t);
-    if (c.iapp != nullptr) iapp += c.iapp[i];
+    Cell cell{};
+    float iapp = 0.0f;
+    if (mine) {
+        cell = load_cell(c.S, vcur, i);
+        iapp = pulse_current(c.pulses, pa, t);
+        if (c.iapp != nullptr) iapp += c.iapp[i];
+    }
+    float U;
+    if (ONE) {
+        U = sgj_block_sum(vcur, c.n, m, threadIdx.x, 256);
+    } else {
+        pdl_enter();
+        float s = 0.0f, cc = 0.0f;
+        for (int q = threadIdx.x & 31; q < n_part; q += 32) kahan_add(s, cc, part[q]);
+        float e = -cc;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+            two_sum_add(s, e, __shfl_xor_sync(0xffffffffu, s, off), __shfl_xor_sync(0xffffffffu, e, off));
+        U = s + e;
+    }
+    if (!mine) return;
+    const float ic = g * fmaf((float)c.n, cell.vd - m, -U);
     const CellNext o = cell_step(c.P, cell, ic, iapp);
-    finish_cell(c, t, vnext, i, o);
+    finish_cell(c, t, vd_next(c), i, o);
 }
 cudaError_t launch_sgj_dense_step(const StepCommon &c, float g, float *part, cudaStream_t st) {
-    if (c.n <= SGJ_ONE_LAUNCH) {
-        return launch_k(sgj_dense_update_kernel, dim3((c.n + 255) / 256), dim3(256), 0, st, c.pdl != 0, c,
+    if (c.n <= SGJ_ONE_LAUNCH)
+        return launch_k(sgj_dense_update_kernel<true>, dim3((c.n + 255) / 256), dim3(256), 0, st, c.pdl != 0, c,
                         (const float *)nullptr, 0, g);
-    }
     const int n_part = sgj_partials(c.n);
     cudaError_t e = launch_k(sgj_partial_kernel, dim3(n_part), dim3(256), 0, st, c.pdl != 0, c, part);
     if (e != cudaSuccess) return e;
-    return launch_k(sgj_dense_update_kernel, dim3((c.n + 255) / 256), dim3(256), 0, st, c.pdl != 0, c,
-                    (const float *)part, n_part, g);
+    return launch_k(sgj_dense_update_kernel<false>, dim3((c.n + CELL_THREADS - 1) / CELL_THREADS), dim3(CELL_THREADS), 0,
+                    st, c.pdl != 0, c, (const float *)part, n_part, g);
 }
 int sgj_partials(int n) { return std::min(256, std::max(1, (n + 4095) / 4096)); }
 
@@ -648,10 +675,9 @@ cudaError_t launch_csr_col16(const int32_t *col, int64_t nnz, int64_t n_alloc, u
 // with CTAs of 256 threads, 53.6 in one direction only, 61.8 before with the pulse table read
 // after the state.
 //
-// CTAs of 128 threads at 51 registers: ten per SM, 1280 cells in flight, and a step's last CTAs
+// CTAs of 128 threads at 48 registers: ten per SM, 1280 cells in flight, and a step's last CTAs
 // leave less of the chip idle than larger ones do (2^20 cells 21.1 -> 20.4 us, 16 384 cells
 // 1.93 -> 1.69).  Twelve per SM spill (2^21 cells 46.2 us), nine keep too little in flight (47.7).
-constexpr int CELL_THREADS = 128;
 __global__ void __launch_bounds__(CELL_THREADS, 10) cell_step_kernel(const CellArgs a) {
     const StepCommon &c = a.c;
     const int64_t b = c.par == 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
