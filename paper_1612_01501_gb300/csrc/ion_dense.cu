@@ -27,8 +27,8 @@
 // pair loop ran; it writes V_dend(t+1) to the other V_dend buffer.
 //
 // Per-step launches are programmatically dependent (launch_k, pdl_enter): the kernel may
-// be scheduled while the previous step drains, initialises its mbarriers, then waits for
-// that step's completion before its first global access.  The V_dend slot comes from the
+// be scheduled while the previous step drains, initialises its mbarriers, reads its rows'
+// pulses (constant data), then waits for that step's completion before it reads any state.  The V_dend slot comes from the
 // host-passed parity, so the tile copy is issued without waiting on the step counter.
 #include <cuda_runtime.h>
 

@@ -17,8 +17,10 @@
 // The rows are walked in opposite directions on even and odd steps: what the last step left in
 // L2 (part of its last rows) is read first, before it is evicted.
 //
-// At 8192 cells: 42.1 us per step (0.95 of the measured copy rate); eight rows per CTA of 8 warps (1024 CTAs, each staging
-// and transforming all of V_dend first, evict-first loads, one direction) 65.8.
+// At 8192 cells: 41.7 us per step (0.95 of the measured copy rate); eight rows per CTA of 8
+// warps (1024 CTAs, each staging and transforming all of V_dend first, evict-first loads, one
+// direction) 65.8.  Keeping a fixed share of the rows in L2 by cache hints (20 to 40 % loaded
+// evict-last, the rest evict-first) measured 42.8 to 45.7: the plain loads stay.
 #include <cuda_runtime.h>
 
 #include <algorithm>
