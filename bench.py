@@ -60,23 +60,25 @@ K3_SWEEP = (1 << 16, 1 << 18, 1 << 20, 1 << 22)
 # None where no capture matches the line's kernel and shape
 # (bytes per launch, source, launch shape the capture used: autotuner fields that must match)
 TRAFFIC = {   # an entry is removed when its kernel changes, until it is captured again
-    ("c2", "dense_step_kernel"): (532224, "profiles/dense_step_kernel_c2_8192.md",
+    ("c2", "dense_step_kernel"): (530688, "profiles/dense_step_kernel_c2_8192.md",
                                   dict(dense_rows_per_warp=4, dense_warps=28, dense_col_splits=2)),
-    ("k3", "cell_step_kernel"): (275259392 + 241500416, "profiles/cell_step_kernel_k3_4194304.md", {}),
-    ("c3_k10", "csr_step_kernel"): (7211520, "profiles/csr_step_kernel_c3_k10.md",
-                                    dict(csr_lanes_per_row=1, csr_rows_per_cta=128)),
-    # captured at 32 lanes per row: the DRAM bytes are those of the padded layout (each
-    # index byte and state word read once), the same for any lane count
+    ("k3", "cell_step_kernel"): (285282816 + 242117120, "profiles/cell_step_kernel_k3_4194304.md", {}),
+    ("c3_k10", "csr_direct_step_kernel"): (7364096, "profiles/csr_direct_step_kernel_c3_k10.md",
+                                           dict(csr_lanes_per_row=4, csr_rows_per_cta=128)),
+    # the DRAM bytes of a cold launch are those of the layout (each index byte and state word
+    # read once), the same for any lane count
+    ("c3_k100", "csr_sliced_step_kernel"): (21719808, "profiles/csr_sliced_step_kernel_c3_k100.md", dict(csr_staging=2)),
+    ("c3_k1000", "csr_sliced_step_kernel"): (139095296 + 2982656, "profiles/csr_sliced_step_kernel_c3_k1000.md",
+                                             dict(csr_staging=2)),
+    # the chunked kernel on the compact layout (networks kept in the bank order; the default
+    # staged network runs the sliced kernel)
     ("c3_k1000", "csr_chunk_step_kernel"): (135862784 + 2681600, "profiles/csr_chunk_step_kernel_c3_k1000.md",
                                             dict(csr_staging=2)),
-    # captured with 8-row dense tiles: the DRAM bytes (state, CSR indices; V_dend tiles
-    # come from L2) are read once per step whatever the tile shape
-    ("c3_k100", "csr_chunk_step_kernel"): (18866432, "profiles/csr_chunk_step_kernel_c3_k100.md", dict(csr_staging=2)),
-    ("c2_sgj", "sgj_dense_update_kernel"): (517376, "profiles/sgj_dense_update_kernel_c2_sgj_8192.md", {}),
-    ("c4", "batch_step_kernel"): (44903168 + 71936, "profiles/batch_step_kernel_c4.md", {}),
-    ("c5", "surrogate_tc_kernel"): (4612352, "profiles/surrogate_tc_kernel_c5.md", {}),
-    # captured at one row per warp: every weight is streamed once whatever the rows per warp
-    ("c2_matrix", "matrix_step_kernel"): (272269312 + 5144320, "profiles/matrix_step_kernel_c2_matrix_8192.md", {}),
+    # one of the step's two dense launches
+    ("c4", "batch_dense_kernel"): (3876352, "profiles/batch_kernels_c4.md", {}),
+    ("c5", "surrogate_tc_kernel"): (4796416, "profiles/surrogate_tc_kernel_c5.md", {}),
+    # captured at four rows in flight: every weight is streamed once whatever their number
+    ("c2_matrix", "matrix_step_kernel"): (268974848 + 3223040, "profiles/matrix_step_kernel_c2_matrix_8192.md", {}),
 }
 
 
@@ -747,7 +749,8 @@ def main():
         peak = ion.ion_probe_peak(0, 4096, stream)
         achieved = work / per_step_s
         roof = {"bound": "alu", "unit": "ex2/s", "achieved": achieved, "peak": peak, "frac": achieved / peak,
-                "traffic": None, "kernel": "batch_persist_kernel" if best == "persistent" else "batch_step_kernel",
+                "traffic": None, "kernel": "batch_persist_kernel" if best == "persistent" else "batch_dense_kernel",
+                "kernels": "batch_dense_kernel and batch_csr_kernel launches in side-by-side chains",
                 "peak_source": "measured SFU ex2 rate (ion_probe_peak) in the same process",
                 "us_per_timestep": per_step_s * 1e6}
         extra = {"pair_evals_per_s": sum(b["n"] ** 2 for b in cfg["nets"] if b["kind"] == "dense") / per_step_s,
@@ -784,7 +787,7 @@ def main():
         peak = ion.ion_probe_peak(0, 4096, stream)
         achieved = ex2_step / per_step_s
         roof = {"bound": "alu", "unit": "ex2/s", "achieved": achieved, "peak": peak, "frac": achieved / peak,
-                "traffic": None, "kernel": {"persistent": "dense_persist_kernel",
+                "traffic": None, "kernel": {"persistent": "dense_small_kernel" if n <= 192 else "dense_persist_kernel",
                            "persistent_half": "dense_half_kernel"}.get(best, "dense_step_kernel"),
                 "peak_source": "measured SFU ex2 rate (ion_probe_peak) in the same process",
                 "ffma_peak_per_s": ion.ion_probe_peak(1, 4096, stream), "us_per_timestep": per_step_s * 1e6,
