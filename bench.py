@@ -74,6 +74,7 @@ TRAFFIC = {   # an entry is removed when its kernel changes, until it is capture
     # staged network runs the sliced kernel)
     ("c3_k1000", "csr_chunk_step_kernel"): (135862784 + 2681600, "profiles/csr_chunk_step_kernel_c3_k1000.md",
                                             dict(csr_staging=2)),
+    ("c2_sgj", "sgj_dense_update_kernel"): (515584, "profiles/sgj_dense_update_kernel_c2_sgj_8192.md", {}),
     # one of the step's two dense launches
     ("c4", "batch_dense_kernel"): (3876352, "profiles/batch_kernels_c4.md", {}),
     ("c5", "surrogate_tc_kernel"): (4796416, "profiles/surrogate_tc_kernel_c5.md", {}),
