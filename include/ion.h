@@ -117,9 +117,12 @@ enum ion_flag {
     ION_FLAG_NO_PDL = 1u << 9      /* launch the per-step kernels as ordinary stream-ordered
                                       launches.  By default each is launched with programmatic
                                       stream serialization: its CTAs may be scheduled while the
-                                      previous step's kernel drains, and wait on the device
-                                      (griddepcontrol.wait) for its completion before touching
-                                      memory.  Results are identical either way.             */
+                                      previous step's kernel drains.  Before they wait on the
+                                      device (griddepcontrol.wait) for its completion they read
+                                      only what the handle owns and no step writes (its copy of
+                                      the connectivity, pulses, launch tables); state, evoked
+                                      input and borrowed arrays are read after the wait.
+                                      Results are identical either way.                      */
 };
 
 typedef struct {
@@ -134,8 +137,10 @@ typedef struct {
  * row_ptr[0] = 0, non-decreasing, row_ptr[n] = nnz), col_idx[nnz] in [0, n), strictly
  * ascending within a row, no self loops, pattern symmetric; weight[nnz] (may be NULL:
  * every weight is g_c).  mem says where the three arrays live; ION_DEVICE arrays are
- * borrowed and must outlive the handle.  The symmetry check is done for host arrays
- * only (device arrays are trusted). */
+ * borrowed and must outlive the handle; row_ptr, col_idx and weight are read by every step,
+ * so values rewritten by work on the handle's stream hold from the next ion_step on (with
+ * the pattern's size and order unchanged).  The symmetry check is done for host arrays only
+ * (device arrays are trusted). */
 typedef struct {
     float g_c;
     const int32_t *row_ptr;

@@ -126,7 +126,9 @@ cudaError_t prepare_csr_step() {
 // Where it runs (short rows, small networks) a step is a few dependent memory latencies long,
 // so everything that does not change between steps (the row's bounds, its first SHORT_E columns
 // and weights per lane, its pulse) is read before the wait on the previous step; after it the
-// V_dend gathers and the rows' state words (cp.async) go out together.  256 threads, SW lanes
+// V_dend gathers and the rows' state words (cp.async) go out together.  Arrays borrowed from the
+// caller (a.borrowed) are read after the wait: the caller may rewrite them on the handle's
+// stream between two calls, and only the wait orders this kernel after such a write.  256 threads, SW lanes
 // per row, four gathers in flight per lane; then one thread per row runs the update.  C16:
 // 16-bit columns.  LIN: linear junctions, w (V_i - V_j).
 // 65 536 cells, k = 10: 5.6 us per step (4 lanes, 128 rows per CTA); the kernel that read
@@ -166,11 +168,12 @@ __global__ void __launch_bounds__(256) csr_direct_step_kernel(const CsrArgs a, i
         if (LIN) return HAS_W ? wt * (vi - vj) : vi - vj;
         return gj_edge(vi, vj, wt);
     };
-    head(sub);
+    if (!a.borrowed) head(sub);
     const int mine = threadIdx.x;
     const bool has_row = mine < rows && row0 + mine < n;
     const PulseAhead pa = pulse_ahead(c.pulses, row0 + mine, has_row && a.fuse);
     pdl_enter();
+    if (a.borrowed) head(sub);
     const int64_t t = step_index(c);
     const float *vcur = vd_cur(c);
     if (a.fuse && has_row) {

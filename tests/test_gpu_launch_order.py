@@ -1,0 +1,50 @@
+"""What a programmatically launched step may read before it waits for the launch before it:
+only what the handle owns and no step writes.  Values that other work on the handle's stream
+writes right before a call (borrowed weights, evoked input) must be the ones the call uses."""
+import numpy as np
+import pytest
+
+from paper_1612_01501_gb300 import inputs
+from paper_1612_01501_gb300 import ion
+
+from test_gpu_parity import torch_cuda  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,k,sgj", [(2000, 10, False), (20000, 24, False), (2000, 40, True)])
+def test_borrowed_weights_rewritten_between_steps(torch_cuda, n, k, sgj):
+    """The weights are the last words of a 256 MB tensor that a kernel rescales right before
+    every step, with no synchronisation between: the programmatic launches give the bits of
+    ordinary ones, and those of a handle that owns a copy of the weights of that step."""
+    torch = torch_cuda
+    rp, col = inputs.random_symmetric_csr(n, k, 71)
+    nnz = len(col)
+    S0 = ion.ion_default_state(n)
+    S0[0] = (S0[0] + inputs.vdend_jitter(n, 71)).astype(np.float32)
+    base = ion.FLAG_KAHAN | (ion.FLAG_SGJ if sgj else 0)
+    scale = np.float32(1.25)
+    stream = torch.cuda.Stream()
+    d_rp, d_col = torch.from_numpy(rp).cuda(), torch.from_numpy(col).cuda()
+    out = []
+    for extra in (0, ion.FLAG_NO_PDL):
+        big = torch.full((64 << 20,), 0.002, dtype=torch.float32, device="cuda")
+        w = big[-nnz:]
+        torch.cuda.synchronize()
+        with ion.Simulation(n, ion.CSR, row_ptr=d_rp, col=d_col, w=w, init_state=S0, flags=base | extra,
+                            stream=stream.cuda_stream) as sim:
+            with torch.cuda.stream(stream):
+                for _ in range(6):
+                    big.mul_(float(scale))
+                    sim.step(1)
+            out.append(sim.state())
+    assert np.array_equal(out[0], out[1])
+    # the oracle of the bits: each step on its own handle with that step's weights, as given
+    wt, S = np.full(nnz, 0.002, np.float32), S0
+    for t in range(6):
+        wt = (wt * scale).astype(np.float32)
+        with ion.Simulation(n, ion.CSR, row_ptr=rp, col=col, w=wt, init_state=S,
+                            flags=base | ion.FLAG_CSR_AS_GIVEN, tune=dict(csr_staging=1)) as sim:
+            sim.step(1)
+            S = sim.state()
+    assert np.array_equal(out[0], S)
