@@ -468,8 +468,8 @@ constexpr int CELL_THREADS = 128;   // CTA of the kernels that only update cells
 //
 // A step is bound by latency up to some 10^5 cells, by memory beyond.  So the sums run in four
 // chains per thread over 16-byte loads, the partials are added by all lanes (one thread adding
-// 256 of them held every CTA of the update for 2 us), the cells' words and pulses are on their
-// way before the sum is known, and the update walks the cells in opposite directions on even
+// 256 of them held every CTA of the update for 2 us), the cells' words are on their way before
+// the sum is known, the pulses before the wait, and the update walks the cells in opposite directions on even
 // and odd steps (cell_step_kernel).
 // Per step before / now: 200 cells 2.6 / 2.0 us, 8192 5.1 / 2.9, 16 384 7.1 / 3.7 (one launch),
 // 16 385 5.3 / 3.8, 100 003 7.4 / 5.5, 600 011 24.8 / 16.1, 1 211 904 57.4 / 30.1.
@@ -511,9 +511,9 @@ __global__ void __launch_bounds__(256) sgj_partial_kernel(const StepCommon c, fl
     const float tot = sgj_block_sum(vcur, c.n, vcur[0], (int64_t)blockIdx.x * 256 + threadIdx.x, (int64_t)gridDim.x * 256);
     if (threadIdx.x == 0) part[blockIdx.x] = tot;
 }
-// ONE: the whole step (part NULL).  Else the launch after sgj_partial_kernel, which lets this
-// one start only after it has itself waited for the previous step: the state is complete here,
-// and only the partial sums have to be waited for.
+// ONE: the whole step (part NULL).  Else the launch after sgj_partial_kernel: the state is that
+// of a launch before the one it waits for, but only the wait makes memory visible to a launch,
+// so nothing but the pulses is read before it.
 template <bool ONE>
 __global__ void __launch_bounds__(ONE ? 256 : CELL_THREADS, ONE ? 1 : 10)
     sgj_dense_update_kernel(const StepCommon c, const float *part, int n_part, float g) {
@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(ONE ? 256 : CELL_THREADS, ONE ? 1 : 10)
     const int64_t i = b * blockDim.x + threadIdx.x;
     const bool mine = i < c.n;
     const PulseAhead pa = pulse_ahead(c.pulses, i, mine);
-    if (ONE) pdl_enter();
+    pdl_enter();
     const int64_t t = step_index(c);
     const float *vcur = vd_cur(c);
     const float m = vcur[0];
@@ -536,7 +536,6 @@ __global__ void __launch_bounds__(ONE ? 256 : CELL_THREADS, ONE ? 1 : 10)
     if (ONE) {
         U = sgj_block_sum(vcur, c.n, m, threadIdx.x, 256);
     } else {
-        pdl_enter();
         float s = 0.0f, cc = 0.0f;
         for (int q = threadIdx.x & 31; q < n_part; q += 32) kahan_add(s, cc, part[q]);
         float e = -cc;

@@ -48,3 +48,48 @@ def test_borrowed_weights_rewritten_between_steps(torch_cuda, n, k, sgj):
             sim.step(1)
             S = sim.state()
     assert np.array_equal(out[0], S)
+
+
+# short rows on the direct kernel; linear dense networks of two launches per step (more than
+# 16 384 cells)
+@pytest.mark.parametrize("case,n", [("csr_k10", 20001), ("sgj_dense", 20000), ("sgj_dense", 300007)])
+def test_pulses_trace_and_input_match_ordinary_launches(torch_cuda, case, n):
+    """Everything that is read early or kept by the step index -- pulses, the trace, a device
+    input rewritten right before the call -- over graph replays and direct launches, bit for
+    bit what ordinary launches give."""
+    torch = torch_cuda
+    S0 = ion.ion_default_state(n)
+    S0[0] = (S0[0] + inputs.vdend_jitter(n, 23)).astype(np.float32)
+    if case == "csr_k10":
+        rp, col = inputs.random_symmetric_csr(n, 10, 23)
+        kw = dict(row_ptr=rp, col=col, w=np.full(len(col), inputs.junction_weight(0.04, 10), np.float32))
+        kind, base = ion.CSR, ion.FLAG_KAHAN
+    else:
+        kw = dict(g=float(np.float32(inputs.junction_weight(0.04, n))))
+        kind, base = ion.DENSE_UNIFORM, ion.FLAG_KAHAN | ion.FLAG_SGJ
+    rng = np.random.default_rng(n)
+    cells = np.sort(rng.integers(0, n, n // 3)).astype(np.int32)          # several pulses on some cells
+    beg = rng.integers(0, 90, len(cells)).astype(np.int64)
+    pul = (cells, beg, beg + rng.integers(1, 40, len(cells)), rng.uniform(1, 6, len(cells)).astype(np.float32))
+    stream = torch.cuda.Stream()
+    out = []
+    for extra in (0, ion.FLAG_NO_PDL):
+        drive = torch.zeros((5, n), dtype=torch.float32, device="cuda")
+        big = torch.zeros(64 << 20, dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        with ion.Simulation(n, kind, init_state=S0, flags=base | extra, stream=stream.cuda_stream, **kw) as sim:
+            sim.set_input(pul)
+            ion.ion_set_trace(sim.h, 1, 140)
+            sim.step(100)
+            sim.step(7)
+            with torch.cuda.stream(stream):
+                for q in range(4):
+                    big.add_(1.0)
+                    drive.copy_(big[:5 * n].view(5, n))
+                    sim.step(5, dense=drive)
+            sim.step(3)
+            sim.sync()
+            out.append((sim.state(), ion.ion_read_trace(sim.h, n, 130)))
+    assert np.isfinite(out[0][0]).all()
+    assert np.array_equal(out[0][0], out[1][0])
+    assert np.array_equal(out[0][1], out[1][1])
