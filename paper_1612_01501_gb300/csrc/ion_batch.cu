@@ -872,13 +872,13 @@ static size_t batch_smem(const BatchExt *X, const BatchExt::Chain &C) {
     return ((size_t)C.vbuf + (C.dense ? 8 * X->R : 0) + (size_t)NCW * C.rows_max) * sizeof(float);
 }
 
-static const void *batch_fn(bool dense, int R) {
-    if (!dense) return (const void *)batch_csr_kernel;
+static cudaError_t batch_allow_smem(bool dense, int R, size_t need) {
+    if (!dense) return allow_smem(batch_csr_kernel, need);
     switch (R) {
-        case 1: return (const void *)batch_dense_kernel<1>;
-        case 2: return (const void *)batch_dense_kernel<2>;
-        case 4: return (const void *)batch_dense_kernel<4>;
-        default: return (const void *)batch_dense_kernel<8>;
+        case 1: return allow_smem(batch_dense_kernel<1>, need);
+        case 2: return allow_smem(batch_dense_kernel<2>, need);
+        case 4: return allow_smem(batch_dense_kernel<4>, need);
+        default: return allow_smem(batch_dense_kernel<8>, need);
     }
 }
 static cudaError_t batch_launch(const BatchArgs &a, bool dense, int R, int tiles, size_t smem, bool pdl, cudaStream_t st) {
@@ -945,7 +945,7 @@ static cudaError_t batch_join(ion_sim *s) {
 // ---- persistent form: planning and launch ----------------------------------------------
 template <int R>
 static cudaError_t persist_kernel_attr(size_t smem, int *per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(batch_persist_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(batch_persist_kernel<R>, smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, batch_persist_kernel<R>, 256, smem);
     return e;
 }
@@ -1165,14 +1165,12 @@ static ion_status batch_persist_run(ion_sim *s, int64_t n_steps, const float *ia
     return ION_OK;
 }
 
+// What the launches of the current tile list (batch_plan) need before they can be captured.
 static ion_status batch_prepare(ion_sim *s) {
     BatchExt *X = ext_of(s);
     cudaError_t e = cudaSuccess;
-    size_t most[2] = {0, 0};
-    for (const BatchExt::Chain &C : X->chains) most[C.dense] = std::max(most[C.dense], batch_smem(X, C));
-    for (int dense = 0; dense < 2 && e == cudaSuccess; ++dense)
-        if (most[dense] > 0)
-            e = cudaFuncSetAttribute(batch_fn(dense != 0, X->R), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most[dense]);
+    for (size_t q = 0; q < X->chains.size() && e == cudaSuccess; ++q)
+        e = batch_allow_smem(X->chains[q].dense, X->R, batch_smem(X, X->chains[q]));
     if (e == cudaSuccess && !X->ev_fork) e = cudaEventCreateWithFlags(&X->ev_fork, cudaEventDisableTiming);
     for (size_t q = 1; q < X->chains.size() && e == cudaSuccess; ++q) {
         if (!X->side[q - 1]) e = cudaStreamCreateWithFlags(&X->side[q - 1], cudaStreamNonBlocking);
@@ -1679,8 +1677,8 @@ static ion_status autotune_persist_batch(ion_sim *s, int32_t steps, ion_tune *ch
     }
     X->R = bR;
     if (st == ION_OK) st = batch_persist_plan(s);
-    if (st == ION_OK) st = batch_prepare(s);   // the per-step kernel (dense inputs) uses R too
-    if (st == ION_OK) st = batch_plan(s);
+    if (st == ION_OK) st = batch_plan(s);      // the per-step kernels (dense inputs) use R too
+    if (st == ION_OK) st = batch_prepare(s);
     cudaFree(save);
     if (st != ION_OK) return st;
     if (chosen) {

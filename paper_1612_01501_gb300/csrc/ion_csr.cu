@@ -380,8 +380,7 @@ static cudaError_t chunk_T(const CsrArgs &a, int rows, const int32_t *mid, int n
                            cudaStream_t st) {
     const size_t smem = csr_chunk_smem_bytes(a.c.n_pad, rows);
     if (prepare)
-        return cudaFuncSetAttribute(csr_chunk_step_kernel<SW, VEC, HAS_W, C16, LIN>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return allow_smem(csr_chunk_step_kernel<SW, VEC, HAS_W, C16, LIN>, smem);
     const int grid = (a.c.n + rows - 1) / rows;
     return launch_k(csr_chunk_step_kernel<SW, VEC, HAS_W, C16, LIN>, dim3(grid), dim3(1024), smem, st,
                     a.c.pdl != 0, a, rows, mid, n_chunks);

@@ -312,7 +312,7 @@ struct StepOp {
         const int rows_cta = (L.W / GJ) * R;
         const size_t smem = dense_step_smem_bytes(L.a->c.n_pad, R, L.W, GJ);
         if (L.prepare_only)
-            return cudaFuncSetAttribute(dense_step_kernel<R, GJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            return allow_smem(dense_step_kernel<R, GJ>, smem);
         const int grid = (L.a->c.n + rows_cta - 1) / rows_cta;
         return launch_k(dense_step_kernel<R, GJ>, dim3(grid), dim3(L.W * 32), smem, L.st, L.a->c.pdl != 0, *L.a);
     }
@@ -335,8 +335,7 @@ struct PersistOp {
         // the tiles and partials, then the rows' state copy (15 + 4 words) and currents
         const size_t smem = dense_smem_bytes(L.a->c.n_pad, R, L.W) + (size_t)(NCW + 5) * rows_cta * sizeof(float);
         if (!L.launch) {   // prepare, and report whether every CTA can be resident at once
-            cudaError_t e = cudaFuncSetAttribute(dense_persist_kernel<R, GJ>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = allow_smem(dense_persist_kernel<R, GJ>, smem);
             if (e != cudaSuccess) return e;
             int per_sm = 0, dev = 0, sms = 0;
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dense_persist_kernel<R, GJ>, L.W * 32, smem);

@@ -313,8 +313,7 @@ static cudaError_t half_RG(const HalfArgs &a0, int W, int G, bool launch, int *o
     }
     const size_t smem = half_smem_bytes(G, a.rows, GR, a.chunk);
     if (!launch) {
-        cudaError_t e = cudaFuncSetAttribute(dense_half_kernel<R, GJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+        cudaError_t e = allow_smem(dense_half_kernel<R, GJ>, smem);
         if (e != cudaSuccess) return e;
         int per_sm = 0, dev = 0, sms = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dense_half_kernel<R, GJ>, W * 32, smem);

@@ -60,6 +60,19 @@ inline cudaError_t launch_k(void (*k)(P...), dim3 grid, dim3 block, size_t smem,
     return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
+// Let a kernel take up to `need` bytes of dynamic shared memory.  The limit belongs to the
+// function, not to a handle: it is always set to all that its static part leaves of a CTA's
+// 227 KB, so that no handle's setup lowers it for another handle.
+template <class F>
+inline cudaError_t allow_smem(F *fn, size_t need) {
+    cudaFuncAttributes fa{};
+    const cudaError_t e = cudaFuncGetAttributes(&fa, (const void *)fn);
+    if (e != cudaSuccess) return e;
+    const size_t limit = 227 * 1024 - fa.sharedSizeBytes;
+    if (need > limit) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
+}
+
 // V_dend slot holding step t: slot 0 is field F_VDEND, slot 1 is field 19.
 __device__ __forceinline__ float *vd_slot(const StateView &S, int64_t t) {
     return S.base + ((t & 1) ? 19 : 0) * S.stride;
