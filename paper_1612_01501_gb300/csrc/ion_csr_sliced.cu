@@ -8,7 +8,10 @@
 // SW lanes per row.  A slice's columns are stored round by round: a round is 8 edges of every
 // lane, 32 x 16 bytes read by one coalesced load, so a warp walks one stream without row
 // bounds, heads, tails or a remainder loop; the sort keeps the padding of a slice's shorter
-// rows small.  Columns are 16-bit offsets into the staged buffer; padding entries point at the
+// rows small (sorted sliced ELLPACK, Kreutzer et al. 2014).  A row far longer than the mean
+// gets more lanes, up to the whole warp: a warp walking it with SW lanes would hold every
+// other warp at the chunk's barrier (65 536 cells, k = 100, 8 rows of 3000 edges: 37.5 us per
+// step with the mean row's lanes, 10.3 now, 10.0 without such rows).  Columns are 16-bit offsets into the staged buffer; padding entries point at the
 // row's own V_dend behind the buffers (dV = 0: they add exactly 0).
 //
 // Bank order: one gather reads entry t of all 32 lanes, from 32 random banks about 3.5
@@ -30,6 +33,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -43,9 +47,16 @@ namespace ion {
 constexpr int SL_THREADS = 1024, SL_WARPS = SL_THREADS / 32;
 constexpr size_t SL_SMEM = 227 * 1024 - 1024;   // dynamic shared memory of a CTA
 
+// An entry of L.rowid: a row of the CTA (L.rows: none) and its slice's lanes per row (log2).
+constexpr int ROW_BITS = 10;
+static_assert(SL_THREADS <= 1 << ROW_BITS, "rows and the none mark fit the row bits");
+__host__ __device__ constexpr uint16_t row_entry(int row, int lsw) { return (uint16_t)(row | lsw << ROW_BITS); }
+__host__ __device__ constexpr int entry_row(uint16_t v) { return v & ((1 << ROW_BITS) - 1); }
+__host__ __device__ constexpr int entry_lsw(uint16_t v) { return v >> ROW_BITS; }
+
 struct SliceItem {
     int32_t e0, e1;  // first round and end (as loaded: nothing waits on them before they are used)
-    uint16_t rr;     // this lane's row within the CTA (L.rows: none)
+    uint16_t row;    // this lane's entry of L.rowid
     __device__ __forceinline__ int n() const { return e1 - e0; }
 };
 
@@ -73,7 +84,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) csr_sliced_step_kernel(const Cs
         SliceItem it;
         it.e0 = __ldg(L.off + next_base);
         it.e1 = __ldg(L.off + next_base + 1);
-        it.rr = __ldg(L.rowid + ((next_base << (5 - L.lsw)) + (lane >> L.lsw)));
+        it.row = __ldg(L.rowid + ((next_base << (5 - L.lsw)) + (lane >> L.lsw)));
         next_base += ++next_p == passes ? (int)gridDim.x * L.nsl - (passes - 1) * SL_WARPS : SL_WARPS;
         if (next_p == passes) next_p = 0;
         return it;
@@ -157,7 +168,8 @@ __global__ void __launch_bounds__(SL_THREADS, 1) csr_sliced_step_kernel(const Cs
         const VjSliced vj{vs + b * L.chunk};
         for (int p = 0; p < passes; ++p) {
             const SliceItem nn = next_item();   // the slice after next: its header arrives meanwhile
-            const float vi = own[cur.rr];
+            const int rr = entry_row(cur.row), sw = 1 << entry_lsw(cur.row);
+            const float vi = own[rr];
             float ks = 0.0f, kc = 0.0f;   // compensated over groups of D rounds
             const uint4 *pc = stream(cur);
             const float4 *wc = wstream(cur);
@@ -176,8 +188,8 @@ __global__ void __launch_bounds__(SL_THREADS, 1) csr_sliced_step_kernel(const Cs
                 if (last) break;
             }
             float acc = ks - kc;
-            for (int off = (1 << L.lsw) >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-            if ((lane & ((1 << L.lsw) - 1)) == 0) ic_s[cur.rr] += acc;
+            for (int off = sw >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            if ((lane & (sw - 1)) == 0) ic_s[rr] += acc;
             cur = nxt;
             nxt = nn;
         }
@@ -255,8 +267,8 @@ __global__ void __launch_bounds__(128) sliced_fill_kernel(const int32_t *bound, 
     const int64_t base = (int64_t)blockIdx.x * 4 + warp;
     if (base >= slices) return;
     const int ch = (int)(base / ((int64_t)grid * L.nsl)), cta = (int)(base / L.nsl % grid);
-    const int rr = L.rowid[(base << (5 - L.lsw)) + (lane >> L.lsw)];
-    const int sw = 1 << L.lsw, li = lane & (sw - 1);
+    const uint16_t row = L.rowid[(base << (5 - L.lsw)) + (lane >> L.lsw)];
+    const int rr = entry_row(row), sw = 1 << entry_lsw(row), li = lane & (sw - 1);
     const int64_t r0 = L.off[base];
     const int T = 8 * (int)(L.off[base + 1] - r0);   // entries of every lane
     auto at = [&](int t) { return ((r0 + (t >> 3)) * 32 + lane) * 8 + (t & 7); };
@@ -347,7 +359,16 @@ SliceLayout ion_plan_sliced(int32_t n, int32_t n_pad, int64_t nnz, int sms, int 
         while (L.lsw < 5 && (L.rows << (L.lsw + 1)) <= SL_THREADS && (8 << (L.lsw + 1)) <= seg) L.lsw++;
     const int per = 32 >> L.lsw;
     L.nsl = (L.rows + per * SL_WARPS - 1) / (per * SL_WARPS) * SL_WARPS;   // whole passes of the 32 warps
+    // twice the mean rounds, at least four: no row of a random graph is near it
+    L.most_rounds = std::max(4, 2 * (int)std::ceil(seg / (8 << L.lsw)));
     return L;
+}
+
+// Lanes (log2) of a row with `edges` edges in a chunk
+static int row_lsw(const SliceLayout &L, int32_t edges) {
+    int lsw = L.lsw;
+    while (lsw < 5 && edges > (8 << lsw) * L.most_rounds) ++lsw;
+    return lsw;
 }
 
 void ion_free_sliced(ion_sim *s) {
@@ -363,10 +384,7 @@ void ion_free_sliced(ion_sim *s) {
 ion_status ion_build_sliced(ion_sim *s, int lanes) {
     ion_free_sliced(s);
     SliceLayout L = ion_plan_sliced(s->n, s->n_pad, s->nnz, s->sms, lanes);
-    const int n = s->n, C = L.n_chunks, grid = (n + L.rows - 1) / L.rows, per = 32 >> L.lsw, sw = 1 << L.lsw;
-    const int64_t slices = (int64_t)C * grid * L.nsl;
-    const int64_t pad = 2 * (int64_t)grid * L.nsl;   // empty slices behind the last, for the look-ahead
-    if ((slices + pad) * 32 >= INT32_MAX) return ION_OK;
+    const int n = s->n, C = L.n_chunks, grid = (n + L.rows - 1) / L.rows, per0 = 32 >> L.lsw;
     int32_t *d_bound = nullptr;
     uint16_t *d_order = nullptr;
     auto done = [&](cudaError_t e) {
@@ -384,29 +402,46 @@ ion_status ion_build_sliced(ion_sim *s, int lanes) {
     e = cudaMemcpyAsync(bound.data(), d_bound, bound.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, s->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
     if (e != cudaSuccess) return done(e);
+    auto edges_at = [&](int ch, int i) { return bound[(size_t)(ch + 1) * n + i] - bound[(size_t)ch * n + i]; };
+    // slices per (chunk, CTA): rows of different lanes are in slices of their own
+    for (int ch = 0; ch < C; ++ch)
+        for (int b = 0; b < grid; ++b) {
+            int rows_of[6] = {}, need = 0;
+            for (int i = b * L.rows; i < std::min(n, (b + 1) * L.rows); ++i) rows_of[row_lsw(L, edges_at(ch, i))]++;
+            for (int l = 0; l <= 5; ++l) need += (rows_of[l] + (32 >> l) - 1) / (32 >> l);
+            L.nsl = std::max(L.nsl, (need + SL_WARPS - 1) / SL_WARPS * SL_WARPS);
+        }
+    const int64_t slices = (int64_t)C * grid * L.nsl;
+    const int64_t pad = 2 * (int64_t)grid * L.nsl;   // empty slices behind the last, for the look-ahead
+    if ((slices + pad) * 32 >= INT32_MAX) return done(cudaSuccess);   // keep the unsliced layout
     std::vector<int32_t> off((size_t)(slices + pad) + 1);
-    std::vector<uint16_t> rowid((size_t)(slices + pad) * per, (uint16_t)L.rows);
+    std::vector<uint16_t> rowid((size_t)(slices + pad) * per0, row_entry(L.rows, L.lsw));
     std::vector<int32_t> order((size_t)L.rows), first;   // rows by falling edge count (a counting sort)
     int64_t tot = 0;
     for (int ch = 0; ch < C; ++ch)
         for (int b = 0; b < grid; ++b) {
             const int r0 = b * L.rows, here = std::min(L.rows, n - r0);
-            auto edges = [&](int r) {
-                return bound[(size_t)(ch + 1) * n + r0 + r] - bound[(size_t)ch * n + r0 + r];
-            };
+            auto edges = [&](int r) { return edges_at(ch, r0 + r); };
             int32_t most = 0;
             for (int r = 0; r < here; ++r) most = std::max(most, edges(r));
             first.assign((size_t)most + 2, 0);
             for (int r = 0; r < here; ++r) first[(size_t)(most - edges(r)) + 1]++;
             for (int32_t k = 0; k <= most; ++k) first[(size_t)k + 1] += first[(size_t)k];
             for (int r = 0; r < here; ++r) order[(size_t)first[(size_t)(most - edges(r))]++] = r;
-            for (int q = 0; q < L.nsl; ++q) {
+            for (int q = 0, at = 0; q < L.nsl; ++q) {   // at: the next row of the sorted order
                 const int64_t base = ((int64_t)ch * grid + b) * L.nsl + q;
                 off[(size_t)base] = (int32_t)tot;
-                if (q * per < here) tot += (edges(order[(size_t)q * per]) + 8 * sw - 1) / (8 * sw);
+                if (at >= here) continue;
+                const int32_t longest = edges(order[(size_t)at]);
+                const int lsw = row_lsw(L, longest), rep = 1 << (lsw - L.lsw);   // entries of a row
+                tot += (longest + (8 << lsw) - 1) / (8 << lsw);
                 if (tot >= INT32_MAX / 64) return done(cudaSuccess);   // keep the unsliced layout
-                for (int r = 0; r < per && q * per + r < here; ++r)
-                    rowid[(size_t)base * per + r] = (uint16_t)order[(size_t)q * per + r];
+                for (int x = 0; x < per0; ++x) {
+                    const int r = at + x / rep;
+                    const bool mine = r < here && row_lsw(L, edges(order[(size_t)r])) == lsw;
+                    rowid[(size_t)base * per0 + x] = row_entry(mine ? order[(size_t)r] : L.rows, lsw);
+                }
+                for (int x = 0; x < 32 >> lsw && at < here && row_lsw(L, edges(order[(size_t)at])) == lsw; ++x) ++at;
             }
         }
     std::fill(off.begin() + slices, off.end(), (int32_t)tot);

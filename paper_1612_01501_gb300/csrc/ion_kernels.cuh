@@ -282,9 +282,11 @@ struct SliceLayout {
     const uint4 *cols;       // NULL: no such layout; per round 32 lanes x 8 columns
     const float4 *w;         // NULL, or per round 2 x 32 lanes x 4 weights
     const int32_t *off;      // first round of each slice, slices in (chunk, CTA, slice) order, and the end
-    const uint16_t *rowid;   // 32 / SW rows of each slice (within the CTA; 0xFFFF: none)
+    const uint16_t *rowid;   // 32 / SW entries of each slice: a row of the CTA (rows: none) and the slice's
+                             // own lanes per row (row_entry; a row with more lanes has several entries)
     int32_t rows;            // rows per CTA (a multiple of 4)
-    int32_t lsw;             // log2 of the lanes per row
+    int32_t lsw;             // log2 of the lanes per row (long rows have more)
+    int32_t most_rounds;     // longest a row may be, in rounds, before it gets more lanes
     int32_t nsl;             // slices per (chunk, CTA)
     int32_t n_chunks, chunk; // V_dend chunks and floats per chunk
     int32_t nbuf;            // chunk buffers in shared memory
