@@ -341,6 +341,7 @@ void ion_csr_fill(const ion_sim *s, CsrArgs &a, bool staged) {
     a.g = s->g;
     a.col16 = csr_use16(s, staged) ? s->d_col16 : nullptr;
     a.borrowed = s->own_csr ? 0 : 1;
+    a.long_rounds = std::max(4, (int)std::ceil((double)s->nnz / s->n / s->csr_SW));   // four times the mean
 }
 
 ion_status ion_setup_csr_staging(ion_sim *s, int mode) {
