@@ -166,9 +166,12 @@ __global__ void __launch_bounds__(256) csr_direct_step_kernel(const CsrArgs a, i
         }
         columns();
     };
-    auto edge = [&](float vi, float vj, float wt) {
-        if (LIN) return HAS_W ? wt * (vi - vj) : vi - vj;
-        return gj_edge(vi, vj, wt);
+    // an edge's term added to a sum, the last product fused into it (one rounding, as gj_edge2)
+    auto add = [&](float s, float vi, float vj, float wt) {
+        const float d = vi - vj;
+        if (LIN) return HAS_W ? fmaf(wt, d, s) : s + d;
+        const float du = d * GJ_SCALE, f = fmaf(0.8f, ex2_approx(-du * du), 0.2f);
+        return fmaf(HAS_W ? wt * f : f, du, s);
     };
     if (!a.borrowed) head(sub);
     const int mine = threadIdx.x;
@@ -194,9 +197,11 @@ __global__ void __launch_bounds__(256) csr_direct_step_kernel(const CsrArgs a, i
 #pragma unroll
             for (int k = 0; k < SHORT_E; ++k)
                 if (e + k * SW < e1) v[k] = __ldg(vcur + j[k]);
+            float part[2] = {0.0f, 0.0f};   // two short chains
 #pragma unroll
             for (int k = 0; k < SHORT_E; ++k)
-                if (e + k * SW < e1) acc += edge(vi, v[k], HAS_W ? w[k] : 1.0f);
+                if (e + k * SW < e1) part[k >> 1] = add(part[k >> 1], vi, v[k], HAS_W ? w[k] : 1.0f);
+            acc += part[0] + part[1];
             e += SHORT_E * SW;
             columns();
         }
@@ -219,9 +224,11 @@ __global__ void __launch_bounds__(256) csr_direct_step_kernel(const CsrArgs a, i
 #pragma unroll
                     for (int k = 0; k < SHORT_E; ++k)
                         if (q + k * 32 < end) v[k] = __ldg(vcur + jl[k]);
+                    float part[2] = {0.0f, 0.0f};
 #pragma unroll
                     for (int k = 0; k < SHORT_E; ++k)
-                        if (q + k * 32 < end) sum += edge(vl, v[k], wl[k]);
+                        if (q + k * 32 < end) part[k >> 1] = add(part[k >> 1], vl, v[k], wl[k]);
+                    sum += part[0] + part[1];
                 }
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
