@@ -296,10 +296,14 @@ void ion_choose_csr_shape(double mean_deg, int *SW, int *rows) {
 // The direct kernel: about four edges per lane (what it reads ahead of the step), and as many
 // rows per CTA as keep every CTA of the grid resident at once (up to 3.5 per SM), since a
 // second wave pays the whole chain of latencies again: 65 536 cells, k = 10: 5.6 us per step
-// with 128 rows per CTA, 6.5 with 64, 6.9 with 256; k = 24: 8.7 / 9.0.
+// with 128 rows per CTA, 6.5 with 64, 6.9 with 256; k = 24: 8.7 / 9.0.  Rows of 56 or more edges
+// take no more lanes than the chip holds threads for (a warp on one row after another pays every
+// row's chain): 30 000 cells, k = 100: 11.2 us with 32 lanes, 9.8 with 8; k = 200: 15.9 / 14.5;
+// 65 536 cells, k = 100, 32-bit linear: 30.2 with 32, 28.2 with 4.
 void ion_choose_direct_shape(int32_t n, double mean_deg, int sms, int *SW, int *rows) {
     int sw = 1;
     while (sw < 32 && 4 * sw < mean_deg) sw *= 2;
+    while (mean_deg >= 56.0 && sw > 4 && (int64_t)n * sw > 2048LL * sms) sw /= 2;
     int r = 256 / sw;
     while (r < 256 && (double)n / r > 3.5 * sms) r *= 2;
     *SW = sw;
@@ -386,13 +390,22 @@ ion_status ion_setup_csr_staging(ion_sim *s, int mode) {
     return ION_OK;
 }
 
+// Does a step without staging run csr_direct_step_kernel (else csr_step_kernel)?  us per step direct /
+// csr_step: 16-bit columns, 65 536 cells: k = 32: 11.3 / 17.6, 48: 15.0 / 18.3, 64: 18.6 / 15.3,
+// 100: 27.2 / 18.1 (weights: 29.5 / 21.4); 30 000 cells, k = 100: 11.2 / 11.6; 9 001, k = 1000:
+// 14.5 / 15.6.  Long rows of 32-bit columns take 16-byte loads of four; linear junctions on 32-bit
+// columns are in the direct kernel only.
+static bool csr_direct(const ion_sim *s, bool col16, bool lin) {
+    if (col16) return s->n <= 40000 || s->nnz < 56 * (int64_t)s->n;
+    return lin || s->nnz < 32 * (int64_t)s->n;
+}
+
 // The CSR step of the handle's layout: sliced, chunked or direct.
 cudaError_t ion_launch_csr(const ion_sim *s, const CsrArgs &a) {
     if (s->csr_staged == 1)
         return s->sl.cols ? launch_csr_sliced_step(a, s->sl, s->st)
                           : launch_csr_chunk_step(a, s->csr_chunk_SW, s->csr_chunk_rows, s->d_mid, s->n_chunks, false, s->st);
-    // 16-bit columns, linear junctions and short rows; long rows of 32-bit columns take 16-byte loads
-    if (a.col16 != nullptr || a.lin || s->nnz < 32 * (int64_t)s->n)
+    if (csr_direct(s, a.col16 != nullptr, a.lin != 0))
         return launch_csr_direct_step(a, s->csr_SW, s->csr_rows, s->st);
     return launch_csr_step(a, s->csr_SW, s->csr_rows, s->st);
 }
@@ -684,7 +697,7 @@ extern "C" ion_status ion_create(const ion_net *net, const ion_conn *conn, const
             if (hs != ION_OK) return fail(hs);
         }
         int SW, rows;
-        if (!s->d_rev && (csr_use16(s, false) || (s->flags & ION_FLAG_SGJ) || s->nnz < 32 * (int64_t)s->n))
+        if (!s->d_rev && csr_direct(s, csr_use16(s, false), (s->flags & ION_FLAG_SGJ) != 0))
             ion_choose_direct_shape(s->n, (double)s->nnz / s->n, sms, &SW, &rows);
         else
             ion_choose_csr_shape((double)s->nnz / s->n, &SW, &rows);

@@ -21,11 +21,13 @@
 namespace ion {
 
 // One CTA of 256 threads owns `rows` consecutive rows (rows <= 256).  Phase 1: groups of
-// SW lanes take the rows round-robin; phase 2: thread t updates row t.  For 32-bit columns in
-// long rows (16-byte loads of four) and the stand-alone primitive; short rows and 16-bit
-// columns run csr_direct_step_kernel.
-template <int SW, bool VEC, bool HAS_W>
+// SW lanes take the rows round-robin; phase 2: thread t updates row t.  For long rows (16-byte
+// loads of four 32-bit or eight 16-bit columns; csr_direct has the rule and its figures) and the
+// stand-alone primitive; the rest runs csr_direct_step_kernel.  LIN: linear junctions, on 16-bit
+// columns only.
+template <int SW, bool VEC, bool HAS_W, bool C16, bool LIN>
 __global__ void __launch_bounds__(256) csr_step_kernel(const CsrArgs a, int rows) {
+    static_assert(!LIN || C16, "linear junctions run on the 16-bit column layout");
     __shared__ float ic_s[256];
     pdl_enter();
     const StepCommon &c = a.c;
@@ -56,8 +58,12 @@ __global__ void __launch_bounds__(256) csr_step_kernel(const CsrArgs a, int rows
         const float vi = vin;
         bounds(it + 1, e0n, e1n, vin);
         float acc = 0.0f;
-        if (e1 > e0)   // rows past the end (and empty rows) have e0 == e1
-            acc = csr_row_sum<SW, VEC, HAS_W>(vcur, a.col, a.w, e0, e1, vi, li);
+        if (e1 > e0) {   // rows past the end (and empty rows) have e0 == e1
+            if (C16)
+                acc = csr_row_sum16<SW, HAS_W, false, LIN>(a.col16, a.w, e0, e1, vi, li, VjGlobal{vcur});
+            else
+                acc = csr_row_sum<SW, VEC, HAS_W>(vcur, a.col, a.w, e0, e1, vi, li);
+        }
 #pragma unroll
         for (int off = SW / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
         if (li == 0 && rr < rows) ic_s[rr] = (HAS_W ? acc : acc * a.g) * (1.0f / GJ_SCALE);
@@ -78,13 +84,20 @@ __global__ void __launch_bounds__(256) csr_step_kernel(const CsrArgs a, int rows
     finish_cell(c, t, vnext, i, o);
 }
 
-template <int SW, bool VEC, bool HAS_W>
+template <int SW, bool VEC, bool HAS_W, bool C16 = false, bool LIN = false>
 static cudaError_t launch_csr_T(const CsrArgs &a, int rows, cudaStream_t st) {
     const int grid = (a.c.n + rows - 1) / rows;
-    return launch_k(csr_step_kernel<SW, VEC, HAS_W>, dim3(grid), dim3(256), 0, st, a.c.pdl != 0, a, rows);
+    return launch_k(csr_step_kernel<SW, VEC, HAS_W, C16, LIN>, dim3(grid), dim3(256), 0, st, a.c.pdl != 0, a, rows);
 }
 template <int SW>
 static cudaError_t launch_csr_SW(const CsrArgs &a, int rows, cudaStream_t st) {
+    if (a.lin) {
+        if (a.col16 == nullptr) return cudaErrorInvalidValue;
+        return a.w != nullptr ? launch_csr_T<SW, true, true, true, true>(a, rows, st)
+                              : launch_csr_T<SW, true, false, true, true>(a, rows, st);
+    }
+    if (a.col16 != nullptr)   // 16-byte aligned indices (and weights, both the handle's own)
+        return a.w != nullptr ? launch_csr_T<SW, true, true, true>(a, rows, st) : launch_csr_T<SW, true, false, true>(a, rows, st);
     const bool vec = ((uintptr_t)a.col % 16 == 0) && (a.w == nullptr || (uintptr_t)a.w % 16 == 0);
     if (a.w != nullptr) return vec ? launch_csr_T<SW, true, true>(a, rows, st) : launch_csr_T<SW, false, true>(a, rows, st);
     return vec ? launch_csr_T<SW, true, false>(a, rows, st) : launch_csr_T<SW, false, false>(a, rows, st);
@@ -107,10 +120,15 @@ cudaError_t launch_csr_step(const CsrArgs &a, int SW, int rows, cudaStream_t st)
 // Prefer L1 over shared memory for the V_dend gathers (the kernel uses 1 KB of shared).
 template <int SW>
 static void carveout_SW() {
-    cudaFuncSetAttribute(csr_step_kernel<SW, true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    cudaFuncSetAttribute(csr_step_kernel<SW, false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    cudaFuncSetAttribute(csr_step_kernel<SW, true, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    cudaFuncSetAttribute(csr_step_kernel<SW, false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    auto prefer_l1 = [](auto *k) { cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 0); };
+    prefer_l1(csr_step_kernel<SW, true, true, false, false>);
+    prefer_l1(csr_step_kernel<SW, false, true, false, false>);
+    prefer_l1(csr_step_kernel<SW, true, false, false, false>);
+    prefer_l1(csr_step_kernel<SW, false, false, false, false>);
+    prefer_l1(csr_step_kernel<SW, true, true, true, false>);
+    prefer_l1(csr_step_kernel<SW, true, false, true, false>);
+    prefer_l1(csr_step_kernel<SW, true, true, true, true>);
+    prefer_l1(csr_step_kernel<SW, true, false, true, true>);
 }
 cudaError_t prepare_csr_step() {
     carveout_SW<1>();

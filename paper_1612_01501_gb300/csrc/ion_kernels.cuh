@@ -274,7 +274,7 @@ struct CsrArgs {
     int32_t fuse;
     float *ic_out;
     const float *vd_in;
-    int32_t lin;          // 1: linear junctions (SGJ use case); not in csr_step_kernel
+    int32_t lin;          // 1: linear junctions (SGJ use case); in csr_step_kernel on 16-bit columns only
     int32_t long_rounds;  // direct kernel: rounds of four edges per lane before the warp takes over a row
     int32_t borrowed;     // 1: row_ptr, col and w are the caller's device arrays
 };

@@ -83,3 +83,17 @@ def test_long_rows_do_not_hold_a_step(torch_cuda, n, k, staging, hubs, length, m
         finally:
             ion.ion_destroy(h)
     assert us[1] <= most * us[0], us
+
+
+# the rule between the two kernels without staging: 16-bit rows of 56 or more edges in networks of
+# more than 40 000 cells take 16-byte loads
+@pytest.mark.parametrize("n,k", [(40000, 60), (40001, 60), (40001, 52), (65536, 64), (65535, 130)])
+@pytest.mark.parametrize("weights,linear", [("uniform", False), ("random", False), ("uniform", True), ("random", True)])
+def test_unstaged_16_bit_rows_one_step(torch_cuda, O, n, k, weights, linear):
+    rp, col = inputs.random_symmetric_csr(n, k, 3)
+    w, tune = _weights(col, weights), dict(csr_staging=1)
+    if linear:
+        err = _sgj_one_step(O, n, O.CSR, rp=rp, col=col, w=w, tune=tune)
+    else:
+        err = _one_step_case(O, "csr", n, O.CSR, rp=rp, col=col, w=w, warm=2, tune=tune)
+    assert err.max() <= STEP_RTOL, err.max(axis=1)
