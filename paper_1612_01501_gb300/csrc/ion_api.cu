@@ -313,10 +313,12 @@ void ion_choose_direct_shape(int32_t n, double mean_deg, int sms, int *SW, int *
 // Shared-memory staging of V_dend for a CSR network (mode 0: choose, 1: off, 2: on).
 // The sliced kernel pays per chunk of V_dend (about 1.7 us: the copy, the slices' bookkeeping),
 // the direct kernel per edge (a 32-byte sector from L2, 4.4 us per million; 1.8 where V_dend
-// fits L1 beside the rest); us per step direct / staged: 2 000 cells, k = 200: 3.1 / 4.2;
-// 10 000: 4.1 / 4.2 (k = 40), 5.1 / 4.3 (64); 20 000: 3.7 / 4.4 (10), 6.4 / 4.6 (40); 40 000:
-// 5.3 / 4.9 (10), 7.7 / 5.0 (24); 65 536: 5.8 / 8.1 (10), 9.1 / 8.3 (24).  Only CSR
-// arrays copied from the host are staged: their columns were checked to be sorted and in
+// fits L1 beside the rest) and, up to about a wave of CTAs, per row; us per step direct / staged:
+// 2 000 cells, k = 200: 3.1 / 4.3; 4 000: 4.0 / 4.3 (100); 10 000: 3.7 / 4.2 (24), 4.5 / 4.3 (40);
+// 20 000: 3.5 / 4.5 (10), 4.6 / 4.6 (24), 6.5 / 4.7 (40); 30 000: 4.1 / 4.6 (10); 40 000: 5.1 /
+// 4.9 (10), 7.4 / 5.1 (24); 50 000: 5.4 / 5.1 (10); 65 536: 5.5 / 8.1 (10), 8.9 / 8.4 (24);
+// 100 000: 10.2 / 10.2 (10), 17.6 / 10.5 (24); 300 000: 19.8 / 42.4 (10), 35.8 / 46.3 (24).  Only
+// CSR arrays copied from the host are staged: their columns were checked to be sorted and in
 // range, which the chunk boundaries rely on.  32-bit columns (CSR_AS_GIVEN) stage rows of 64 or
 // more edges that keep 32 or more per 128 KB chunk, or any CSR too large for L2 (over 96 MB)
 // with rows of 64 or more.
@@ -326,12 +328,14 @@ static bool stage_by_default(const ion_sim *s, double deg, double csr_bytes) {
     if (!s->d_col16 || s->col16_bank) return deg >= 64.0 && deg / chunks >= 32.0;
     const SliceLayout L = ion_plan_sliced(s->n, s->n_pad, s->nnz, s->sms, 0);
     const double waves = std::ceil((double)s->n / L.rows / s->sms);
-    const double staged = 2.5 + 1.7 * L.n_chunks * waves + 2.0e-5 * s->n, direct = 2.2 + (s->n <= 4000 ? 1.8e-6 : 4.4e-6) * (double)s->nnz;
+    const double staged = 2.5 + 1.7 * L.n_chunks * waves + 2.0e-5 * s->n;
+    const double direct = 2.2 + 3.0e-5 * std::min(s->n, 50000) + (s->n <= 4000 ? 1.8e-6 : 4.4e-6) * (double)s->nnz;
     return staged < direct;
 }
 // The 16-bit columns serve the staged kernel (columns relative to a chunk of at most 2^16
-// cells) and the direct kernel when n <= 65 536 and rows are long enough (mean degree >= 32)
-// for its eight-edge groups; shorter rows read 32-bit columns four at a time.
+// cells) and the kernels without staging when n <= 65 536 and the mean degree is at least 32:
+// half the index bytes, and eight columns to a 16-byte load in csr_step_kernel.  Shorter rows
+// keep the 32-bit columns.
 static bool csr_use16(const ion_sim *s, bool staged) {
     if (s->d_col16 == nullptr || s->d_rev != nullptr) return false;   // the half-work passes read 32-bit columns
     return staged || (s->n <= 65536 && s->nnz >= 32 * (int64_t)s->n);

@@ -97,3 +97,13 @@ def test_unstaged_16_bit_rows_one_step(torch_cuda, O, n, k, weights, linear):
     else:
         err = _one_step_case(O, "csr", n, O.CSR, rp=rp, col=col, w=w, warm=2, tune=tune)
     assert err.max() <= STEP_RTOL, err.max(axis=1)
+
+
+# both sides of the line between gathering and staging, each at least as fast there as the other
+# (the figures are beside the rule)
+@pytest.mark.parametrize("n,k,staged", [(2000, 200, 0), (10000, 24, 0), (30000, 10, 0), (40000, 10, 1), (50000, 10, 1),
+                                        (20000, 40, 1), (65536, 10, 0), (65536, 24, 1), (100000, 24, 1), (300000, 10, 0)])
+def test_default_staging(torch_cuda, n, k, staged):
+    rp, col = inputs.random_symmetric_csr(n, k, 3)
+    with ion.Simulation(n, ion.CSR, row_ptr=rp, col=col, w=np.full(len(col), 0.001, np.float32)) as sim:
+        assert ion.ion_csr_layout(sim.h)["staged"] == staged
