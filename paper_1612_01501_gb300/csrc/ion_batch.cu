@@ -133,6 +133,50 @@ __device__ __forceinline__ void slice_begin(SliceAhead<HAS_W> &ah, int slice0, i
     if (warp < ns) ah.begin(slice0 + s0 + warp, off, cols, w);
 }
 
+// The same sums, one round loaded ahead, for the persistent kernel: groups of rounds in flight
+// there (two kinds of rows and the pair loop in one kernel) spilled 440 to 560 bytes a thread, in
+// the dense pieces' loops too, and a step of two 64-cell dense networks took 4.9 us; now 3.6.
+template <bool HAS_W>
+__device__ __forceinline__ void slice_rows_short(int slice0, int lsw, int n, int r0, int rows, const int32_t *off,
+                                                 const uint4 *cols, const float4 *w, const float *vs, float g,
+                                                 float *ic_s) {
+    constexpr int D = SliceAhead<HAS_W>::D;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int per = 32 >> lsw, s0 = r0 / per, ns = (r0 + rows - 1) / per - s0 + 1;
+    const VjSliced vj{vs};
+    for (int s = warp; s < ns; s += 8) {
+        const int e0 = __ldg(off + slice0 + s0 + s), ne = __ldg(off + slice0 + s0 + s + 1) - e0;
+        const int i = (s0 + s) * per + (lane >> lsw);
+        const float vi = vs[min(i, n - 1)];
+        const uint4 *pc = cols + (int64_t)e0 * 32 + lane;
+        const float4 *pw = HAS_W ? w + (int64_t)e0 * 64 + lane : w;
+        float ks = 0.0f, kc = 0.0f, blk = 0.0f;
+        uint4 q = make_uint4(0u, 0u, 0u, 0u);
+        if (ne > 0) q = __ldg(pc);
+#pragma unroll 1
+        for (int k = 0; k < ne; ++k) {
+            const uint4 now = q;
+            float4 wa, wb;
+            if (HAS_W) {
+                wa = __ldg(pw);
+                wb = __ldg(pw + 32);
+                pw += 64;
+            }
+            pc += 32;
+            if (k + 1 < ne) q = __ldg(pc);
+            blk += csr_group16<HAS_W>(now, wa, wb, vi, vj);
+            if ((k & (D - 1)) == D - 1 || k + 1 == ne) {
+                kahan_add(ks, kc, blk);
+                blk = 0.0f;
+            }
+        }
+        float acc = ks - kc;
+        for (int o = (1 << lsw) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((lane & ((1 << lsw) - 1)) == 0 && i >= r0 && i < r0 + rows)
+            ic_s[i - r0] = (HAS_W ? acc : acc * g) * (1.0f / GJ_SCALE);
+    }
+}
+
 // The sliced columns (and weights) from the networks' 16-bit rows: a warp per slice.
 struct SliceDesc {
     int32_t row, rows;   // first row (padded index), rows (<= 32 / SW)
@@ -387,8 +431,8 @@ __global__ void __launch_bounds__(256) batch_csr_kernel(const BatchArgs a) {
 // holds k x (pieces of b).  No CTA ever waits on a later step than its own, so the CTA
 // with the oldest step always progresses: the launch cannot deadlock, and no grid-wide
 // barrier is needed.  The pair loop, the CSR row sums and the cell update are those of
-// the per-step kernel (the same lanes per row and rows per warp give the same sums), so
-// the states equal those of the per-step launches bit for bit.
+// the per-step kernels (the same lanes per row give the same sums, whatever the rows per
+// warp), so the states equal those of the per-step launches bit for bit.
 struct PersistItem {
     int32_t kind;     // TILE_DENSE or TILE_CSR
     int32_t net;      // network (index of its arrival counter)
@@ -480,9 +524,12 @@ struct VRowCG {
     __device__ __forceinline__ float operator()(int j) const { return __ldcg(v + j); }
 };
 
-// 256 threads: 8 warps; dense pieces run 8 x R rows at a time.
+// 256 threads: 8 warps; dense pieces run 8 x R rows at a time.  Three CTAs per SM: a piece is a
+// chain of latencies, and fewer, larger shares of the networks wait for fewer others.  us per step
+// with four / three: 12 dense networks of 1792 cells 19.2 / 11.6, two networks of 500 5.2 / 4.4, 96
+// networks of 32-4096 cells 43 / 45.
 template <int R>
-__global__ void __launch_bounds__(256, 4) batch_persist_kernel(const BatchPersistArgs a) {
+__global__ void __launch_bounds__(256, 3) batch_persist_kernel(const BatchPersistArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ float red_s[32], red_c[32];
@@ -562,15 +609,10 @@ __global__ void __launch_bounds__(256, 4) batch_persist_kernel(const BatchPersis
                 }
             } else if (P.mode & TILE_STAGE_V) {
                 const int lsw = 31 - __clz(P.sw), r0 = P.row0 - P.seg;
-                if (P.mode & TILE_UNIFORM_W) {
-                    SliceAhead<false> ah;
-                    slice_begin(ah, P.slice0, lsw, r0, P.rows, a.soff, a.scols, a.sw);
-                    slice_rows(ah, P.slice0, lsw, P.n, r0, P.rows, a.soff, a.scols, a.sw, vb, P.g, ic_s);
-                } else {
-                    SliceAhead<true> ah;
-                    slice_begin(ah, P.slice0, lsw, r0, P.rows, a.soff, a.scols, a.sw);
-                    slice_rows(ah, P.slice0, lsw, P.n, r0, P.rows, a.soff, a.scols, a.sw, vb, P.g, ic_s);
-                }
+                if (P.mode & TILE_UNIFORM_W)
+                    slice_rows_short<false>(P.slice0, lsw, P.n, r0, P.rows, a.soff, a.scols, a.sw, vb, P.g, ic_s);
+                else
+                    slice_rows_short<true>(P.slice0, lsw, P.n, r0, P.rows, a.soff, a.scols, a.sw, vb, P.g, ic_s);
             } else {
                 persist_csr_piece(a, P, VRowCG{vcur + P.seg}, VjGlobalCG{vcur + P.seg}, ic_s);
             }
@@ -643,6 +685,7 @@ struct BatchExt {
     int32_t *d_cta_off = nullptr;
     uint32_t *d_pcnt = nullptr;     // n_nets counters, then the abort word
     int p_grid = 0, p_vbuf = 256, p_pieces = 0;
+    int p_R = 0;                    // dense rows per warp of the persistent kernel (0: choose)
     cudaGraphExec_t p_graph = nullptr;
     int64_t p_graph_steps = 0;
     bool p_graph_refused = false;
@@ -964,7 +1007,18 @@ static const void *persist_fn(int R) {
         default: return (const void *)batch_persist_kernel<4>;
     }
 }
-static size_t persist_smem(const BatchExt *X) { return (size_t)X->p_vbuf * 4 + 8 * X->R * 4; }
+static size_t persist_smem(const BatchExt *X) { return (size_t)X->p_vbuf * 4 + 8 * X->p_R * 4; }
+
+// Rows per warp of the persistent kernel's dense pieces where none are asked for: a row's sum is the
+// same whatever R.  Two keep a small network's chain short, four share the column loads once
+// the pairs fill the chip.  us per step with 2 / 4: one network of 2000 cells 6.2 / 8.0, of 300 4.2 /
+// 4.7, twelve of 1792 (4e7 pairs) 11.6 / 11.8, 48 of 32-4096 beside 48 CSR ones (1e8) 45 / 35.
+static int persist_rows(const BatchExt *X) {
+    double pairs = 0.0;
+    for (const BatchNet &b : X->nets)
+        if (b.kind == ION_DENSE_UNIFORM) pairs += (double)b.n * b.n_pad;
+    return pairs > 6.0e7 ? 4 : 2;
+}
 
 // Cut the networks into pieces and deal them out to the CTAs of one resident grid.
 // Work per row: a dense row costs its network's padded width in pair evaluations (plus a
@@ -975,10 +1029,9 @@ static size_t persist_smem(const BatchExt *X) { return (size_t)X->p_vbuf * 4 + 8
 // first, so that their arrivals come early in every step.
 static ion_status batch_persist_plan(ion_sim *s) {
     BatchExt *X = ext_of(s);
-    if (X->R != 1 && X->R != 2 && X->R != 4) X->R = 2;
     X->p_vbuf = X->max_dense_pad;
     int per_sm = 0;
-    cudaError_t e = persist_attr(X->R, persist_smem(X), &per_sm);
+    cudaError_t e = persist_attr(X->p_R, persist_smem(X), &per_sm);
     if (e != cudaSuccess || per_sm < 1)
         return ion_fail(s, ION_ERR_UNSUPPORTED, "persistent batch: no resident CTA (%s)", cudaGetErrorString(e));
     const int grid = per_sm * s->sms;
@@ -987,8 +1040,11 @@ static ion_status batch_persist_plan(ion_sim *s) {
     double total = 0.0;
     for (size_t b = 0; b < X->nets.size(); ++b) {
         const BatchNet &x = X->nets[b];
-        if (x.kind == ION_DENSE_UNIFORM) nc[b] = {(double)x.n_pad + 64.0, 2048.0 + x.n_pad, 8 * X->R};
-        else nc[b] = {3.0 * (x.n > 0 ? (double)x.nnz / x.n : 0.0) + 60.0, 2048.0 + 0.5 * x.n_pad, 32};
+        // sliced rows: two slices or more per piece (twelve networks of 2000 cells, k = 24: 5.1 us
+        // per step, one slice 8.5, eight 6.6)
+        if (x.kind == ION_DENSE_UNIFORM) nc[b] = {(double)x.n_pad + 64.0, 2048.0 + x.n_pad, 8 * X->p_R};
+        else nc[b] = {3.0 * (x.n > 0 ? (double)x.nnz / x.n : 0.0) + 60.0, 2048.0 + 0.5 * x.n_pad,
+                      net_staged(X, x) ? 2 * (32 / x.sw) : 32};
         total += nc[b].per_row * x.n + nc[b].fixed;
     }
     const double share = total / grid;
@@ -1106,9 +1162,9 @@ static cudaError_t persist_enqueue(ion_sim *s, int n_steps, bool capture) {
         cfg.stream = s->st;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        e = cudaLaunchKernelExC(&cfg, persist_fn(X->R), args);
+        e = cudaLaunchKernelExC(&cfg, persist_fn(X->p_R), args);
     } else {
-        e = cudaLaunchCooperativeKernel(persist_fn(X->R), dim3(X->p_grid), dim3(256), args, persist_smem(X), s->st);
+        e = cudaLaunchCooperativeKernel(persist_fn(X->p_R), dim3(X->p_grid), dim3(256), args, persist_smem(X), s->st);
     }
     if (e != cudaSuccess) return e;
     return launch_advance(s->d_t, n_steps, s->st);
@@ -1339,7 +1395,7 @@ extern "C" ion_status ion_create_batch(int32_t n_nets, const ion_net *nets, cons
             for (int i = 0; i < x.n; ++i) X->h_map[(size_t)u++] = x.seg + i;
     }
     const ion_tune *tu = (const ion_tune *)params->tune;
-    if (tu && tu->dense_rows_per_warp > 0) X->R = tu->dense_rows_per_warp;
+    if (tu && tu->dense_rows_per_warp > 0) X->R = X->p_R = tu->dense_rows_per_warp;
     if (tu && tu->csr_rows_per_cta > 0) X->csr_rows = tu->csr_rows_per_cta;
     if (tu && tu->csr_lanes_scale != 0) X->sw_scale = tu->csr_lanes_scale > 0 ? 1 : -1;
     if ((X->R != 1 && X->R != 2 && X->R != 4 && X->R != 8) || X->csr_rows < 1 || X->csr_rows > 256)
@@ -1409,6 +1465,8 @@ extern "C" ion_status ion_create_batch(int32_t n_nets, const ion_net *nets, cons
         if (!coop) return fail(ion_fail(nullptr, ION_ERR_UNSUPPORTED, "ion_create_batch: no cooperative launches"));
         X->persistent = true;
         s->flags |= ION_FLAG_PERSISTENT;
+        if (X->p_R == 0) X->p_R = persist_rows(X);
+        else if (X->p_R == 8) X->p_R = 2;   // a shape of the per-step launches only
         st = batch_persist_plan(s);
         if (st != ION_OK) return fail(st);
         s->run_override = batch_persist_run;
@@ -1645,10 +1703,10 @@ static ion_status autotune_persist_batch(ion_sim *s, int32_t steps, ion_tune *ch
     }
     const int64_t t0 = s->t;
     float best = 1e30f;
-    int bR = X->R;
+    int bR = X->p_R;
     ion_status st = ION_OK;
     for (int R : {1, 2, 4}) {
-        X->R = R;
+        X->p_R = R;
         st = batch_persist_plan(s);
         if (st != ION_OK) break;
         cudaEvent_t a, b;
@@ -1675,10 +1733,8 @@ static ion_status autotune_persist_batch(ion_sim *s, int32_t steps, ion_tune *ch
             bR = R;
         }
     }
-    X->R = bR;
+    X->p_R = bR;
     if (st == ION_OK) st = batch_persist_plan(s);
-    if (st == ION_OK) st = batch_plan(s);      // the per-step kernels (dense inputs) use R too
-    if (st == ION_OK) st = batch_prepare(s);
     cudaFree(save);
     if (st != ION_OK) return st;
     if (chosen) {
