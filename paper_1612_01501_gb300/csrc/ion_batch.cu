@@ -35,8 +35,9 @@ namespace ion {
 
 enum TileKind : int32_t { TILE_DENSE = 0, TILE_CSR = 1 };
 // CSR tile modes: every weight of the network equals T.g; 16-bit network-local columns
-// (col16); the network's V_dend staged in shared memory (with TILE_C16)
-enum TileMode : int32_t { TILE_UNIFORM_W = 1, TILE_C16 = 2, TILE_STAGE_V = 4 };
+// (col16); the network's V_dend staged in shared memory (with TILE_C16); its rows stored in
+// slices (with TILE_STAGE_V)
+enum TileMode : int32_t { TILE_UNIFORM_W = 1, TILE_C16 = 2, TILE_STAGE_V = 4, TILE_SLICED = 8 };
 
 struct BatchTile {
     int32_t kind;
@@ -48,7 +49,7 @@ struct BatchTile {
     int32_t sw;      // CSR: lanes per row
     float g;         // dense: pair weight; CSR with TILE_UNIFORM_W: every edge weight
     int32_t mode;    // CSR: TileMode bits
-    int32_t slice0;  // CSR with TILE_STAGE_V: the network's first slice
+    int32_t slice0;  // TILE_SLICED: the network's first slice
 };
 
 struct BatchArgs {
@@ -204,7 +205,30 @@ __global__ void __launch_bounds__(128) batch_slice_fill_kernel(const SliceDesc *
         }
 }
 
-// CSR rows of a TILE_C16 tile: 16-bit local columns, V_dend from `vj` (global memory)
+// A row's sum by SW lanes, each lane's part of it; a row of more than eight rounds (64 SW edges) by
+// its whole warp, one such row after the other (its sum in the row's lane 0).  All lanes of the
+// warp call it; e0 == e1: no row.
+template <int SW, bool HAS_W, class VJ>
+__device__ __forceinline__ float batch_row16(const uint16_t *col16, const float *w, int e0, int e1, float vi, int li,
+                                             VJ vj) {
+    const bool far = SW < 32 && e1 - e0 > 64 * SW;
+    float acc = far || e0 == e1 ? 0.0f : csr_row_sum16<SW, HAS_W, false>(col16, w, e0, e1, vi, li, vj);
+    if (SW < 32) {
+        const int lane = threadIdx.x & 31;
+        for (uint32_t left = __ballot_sync(0xffffffffu, far && li == 0); left != 0; left &= left - 1) {
+            const int src = __ffs(left) - 1;
+            float sum = csr_row_sum16<32, HAS_W, false>(col16, w, __shfl_sync(0xffffffffu, e0, src),
+                                                        __shfl_sync(0xffffffffu, e1, src),
+                                                        __shfl_sync(0xffffffffu, vi, src), lane, vj);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            if (lane == src) acc = sum;
+        }
+    }
+    return acc;
+}
+
+// CSR rows of a TILE_C16 tile: 16-bit local columns, V_dend from `vj`
 template <int SW, bool HAS_W, class VJ>
 __device__ __forceinline__ void batch_csr_rows16(const BatchArgs &a, const BatchTile &T, const float *vcur, VJ vj,
                                                  float *ic_s) {
@@ -226,8 +250,8 @@ __device__ __forceinline__ void batch_csr_rows16(const BatchArgs &a, const Batch
             e1n = a.row_ptr[T.row0 + rr + nsub + 1];
             vin = vcur[T.row0 + rr + nsub];
         }
-        float acc = 0.0f;
-        if (rr < T.rows) acc = csr_row_sum16<SW, HAS_W, false>(a.col16, a.w, e0, e1, vi, li, vj);
+        const bool has = rr < T.rows;
+        float acc = batch_row16<SW, HAS_W>(a.col16, a.w, has ? e0 : 0, has ? e1 : 0, vi, li, vj);
 #pragma unroll
         for (int off = SW / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
         if (li == 0 && rr < T.rows) ic_s[rr] = (HAS_W ? acc : acc * T.g) * (1.0f / GJ_SCALE);
@@ -373,12 +397,13 @@ __global__ void __launch_bounds__(256) batch_csr_kernel(const BatchArgs a) {
     const TileRow row = tile_row(a, T);
     float *vs = reinterpret_cast<float *>(smem_raw), *cs = vs + a.vbuf;
     const bool staged = (T.mode & TILE_STAGE_V) != 0, uniform = (T.mode & TILE_UNIFORM_W) != 0;
+    const bool sliced = (T.mode & TILE_SLICED) != 0;
     const int lsw = 31 - __clz(T.sw), local0 = T.row0 - T.seg;
     // the first slice of this warp, before the wait too
     SliceAhead<false> au;
     SliceAhead<true> aw;
-    if (staged && uniform) slice_begin(au, T.slice0, lsw, local0, T.rows, a.soff, a.scols, a.sw);
-    else if (staged) slice_begin(aw, T.slice0, lsw, local0, T.rows, a.soff, a.scols, a.sw);
+    if (sliced && uniform) slice_begin(au, T.slice0, lsw, local0, T.rows, a.soff, a.scols, a.sw);
+    else if (sliced) slice_begin(aw, T.slice0, lsw, local0, T.rows, a.soff, a.scols, a.sw);
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         fence_mbar_init();
@@ -402,7 +427,8 @@ __global__ void __launch_bounds__(256) batch_csr_kernel(const BatchArgs a) {
             cp_async_wait_all();
             return;
         }
-        if (uniform) slice_rows(au, T.slice0, lsw, T.n, local0, T.rows, a.soff, a.scols, a.sw, vs, T.g, ic_s);
+        if (!sliced) batch_csr_tile16(a, T, vcur, VjSliced{vs}, ic_s);
+        else if (uniform) slice_rows(au, T.slice0, lsw, T.n, local0, T.rows, a.soff, a.scols, a.sw, vs, T.g, ic_s);
         else slice_rows(aw, T.slice0, lsw, T.n, local0, T.rows, a.soff, a.scols, a.sw, vs, T.g, ic_s);
     } else if (T.mode & TILE_C16) {
         batch_csr_tile16(a, T, vcur, VjGlobal{vcur + T.seg}, ic_s);
@@ -442,7 +468,7 @@ struct PersistItem {
     int32_t pieces;   // pieces of this network (arrivals per step)
     int32_t sw;       // CSR: lanes per row
     int32_t mode;     // CSR: TileMode bits
-    int32_t slice0;   // CSR with TILE_STAGE_V: the network's first slice
+    int32_t slice0;   // TILE_SLICED: the network's first slice
     float g;
 };
 
@@ -491,12 +517,15 @@ __device__ __forceinline__ void persist_csr_rows(const BatchPersistArgs &a, cons
                                                  float *ic_s) {
     const int sub = threadIdx.x / SW, li = threadIdx.x % SW, nsub = blockDim.x / SW;
     for (int rr = sub; rr - sub < P.rows; rr += nsub) {   // the same trip count in every lane
-        float acc = 0.0f;
+        int e0 = 0, e1 = 0;
+        float vi = 0.0f;
         if (rr < P.rows) {
             const int i = P.row0 + rr;
-            const int e0 = a.row_ptr[i], e1 = a.row_ptr[i + 1];
-            if (e1 > e0) acc = csr_row_sum16<SW, HAS_W, false>(a.col16, a.w, e0, e1, vrow(i - P.seg), li, vj);
+            e0 = a.row_ptr[i];
+            e1 = a.row_ptr[i + 1];
+            vi = vrow(i - P.seg);
         }
+        float acc = batch_row16<SW, HAS_W>(a.col16, a.w, e0, e1, vi, li, vj);
 #pragma unroll
         for (int off = SW / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
         if (li == 0 && rr < P.rows) ic_s[rr] = (HAS_W ? acc : acc * P.g) * (1.0f / GJ_SCALE);
@@ -519,6 +548,10 @@ __device__ __forceinline__ void persist_csr_piece(const BatchPersistArgs &a, con
 #undef ION_CSR_SW
 }
 
+struct VRowSmem {
+    const float *v;
+    __device__ __forceinline__ float operator()(int j) const { return v[j]; }
+};
 struct VRowCG {
     const float *v;
     __device__ __forceinline__ float operator()(int j) const { return __ldcg(v + j); }
@@ -607,12 +640,14 @@ __global__ void __launch_bounds__(256, 3) batch_persist_kernel(const BatchPersis
                                                                  P.n, U, P.g);
                     __syncthreads();   // part[] is rewritten by the next row block
                 }
-            } else if (P.mode & TILE_STAGE_V) {
+            } else if (P.mode & TILE_SLICED) {
                 const int lsw = 31 - __clz(P.sw), r0 = P.row0 - P.seg;
                 if (P.mode & TILE_UNIFORM_W)
                     slice_rows_short<false>(P.slice0, lsw, P.n, r0, P.rows, a.soff, a.scols, a.sw, vb, P.g, ic_s);
                 else
                     slice_rows_short<true>(P.slice0, lsw, P.n, r0, P.rows, a.soff, a.scols, a.sw, vb, P.g, ic_s);
+            } else if (P.mode & TILE_STAGE_V) {
+                persist_csr_piece(a, P, VRowSmem{vb}, VjSliced{vb}, ic_s);
             } else {
                 persist_csr_piece(a, P, VRowCG{vcur + P.seg}, VjGlobalCG{vcur + P.seg}, ic_s);
             }
@@ -668,7 +703,8 @@ struct BatchNet {
     float g;          // dense: pair weight; CSR with uniform weights: every edge weight
     int64_t e0, nnz;  // CSR edges in the global arrays
     int sw;
-    int slice0 = 0;         // staged CSR: first slice
+    int slice0 = 0;         // sliced CSR: first slice
+    bool sliced = false;    // CSR: rows in slices
     bool uniform = false;   // CSR: every weight bitwise equal (g)
     bool c16 = false;       // CSR: 16-bit network-local columns in col16
 };
@@ -742,6 +778,18 @@ static bool net_staged(const BatchExt *X, const BatchNet &b) {
     return b.kind == ION_CSR && b.c16 && b.n_pad <= X->max_dense_pad;   // fits the launches' shared memory
 }
 
+// A slice lasts as long as its longest row, with the few lanes of a mean row.  Networks with a
+// row of more than four times the mean's rounds (at least four) keep their 16-bit rows: more lanes
+// per row, a whole warp for the long ones (batch_row16), no slices.  us per step of six networks
+// of 4000 cells, k = 10, two cells with 2000 partners each: sliced 61, so 6.8.
+static bool net_sliced(const BatchExt *X, const BatchNet &b, int sw) {
+    if (!net_staged(X, b)) return false;
+    const int most = 4 * std::max(1, (int)std::ceil((double)b.nnz / b.n / (8 * sw)));
+    for (int r = b.seg; r < b.seg + b.n; ++r)
+        if (X->h_rp[(size_t)r + 1] - X->h_rp[(size_t)r] > 8 * sw * most) return false;
+    return true;
+}
+
 // The sliced layout for the current lanes-per-row scale (kept while that does not change).
 static ion_status batch_build_slices(ion_sim *s) {
     BatchExt *X = ext_of(s);
@@ -752,8 +800,9 @@ static ion_status batch_build_slices(ion_sim *s) {
     bool weights = false;
     for (BatchNet &b : X->nets) {
         const double deg = b.n > 0 ? (double)b.nnz / b.n : 0.0;
-        if (b.kind == ION_CSR) b.sw = net_staged(X, b) ? slice_sw_for(deg, X->sw_scale) : csr_sw_for(deg, X->sw_scale);
-        if (!net_staged(X, b)) continue;
+        b.sliced = net_sliced(X, b, slice_sw_for(deg, X->sw_scale));
+        if (b.kind == ION_CSR) b.sw = b.sliced ? slice_sw_for(deg, X->sw_scale) : csr_sw_for(deg, X->sw_scale);
+        if (!b.sliced) continue;
         weights = weights || !b.uniform;
         b.slice0 = (int)desc.size();
         int lsw = 0;
@@ -844,7 +893,7 @@ static ion_status batch_plan(ion_sim *s) {
         } else {
             const double deg = b.n > 0 ? (double)b.nnz / b.n : 0.0;
             int mode = (b.uniform ? TILE_UNIFORM_W : 0) | (b.c16 ? TILE_C16 : 0);
-            if (net_staged(X, b)) mode |= TILE_STAGE_V;
+            if (net_staged(X, b)) mode |= TILE_STAGE_V | (b.sliced ? TILE_SLICED : 0);
             int crows = X->csr_rows;
             while (crows > 32 && crows * deg > csr_work) crows = (crows + 1) / 2;
             for (int r = 0; r < b.n; r += crows) {
@@ -1044,7 +1093,7 @@ static ion_status batch_persist_plan(ion_sim *s) {
         // per step, one slice 8.5, eight 6.6)
         if (x.kind == ION_DENSE_UNIFORM) nc[b] = {(double)x.n_pad + 64.0, 2048.0 + x.n_pad, 8 * X->p_R};
         else nc[b] = {3.0 * (x.n > 0 ? (double)x.nnz / x.n : 0.0) + 60.0, 2048.0 + 0.5 * x.n_pad,
-                      net_staged(X, x) ? 2 * (32 / x.sw) : 32};
+                      x.sliced ? 2 * (32 / x.sw) : 32};
         total += nc[b].per_row * x.n + nc[b].fixed;
     }
     const double share = total / grid;
@@ -1074,7 +1123,7 @@ static ion_status batch_persist_plan(ion_sim *s) {
                 it.sw = x.sw;
                 it.mode = (x.uniform ? TILE_UNIFORM_W : 0) | (x.c16 ? TILE_C16 : 0);
                 it.slice0 = x.slice0;
-                if (net_staged(X, x)) it.mode |= TILE_STAGE_V;
+                if (net_staged(X, x)) it.mode |= TILE_STAGE_V | (x.sliced ? TILE_SLICED : 0);
             }
             pieces.push_back({it, nc[b].per_row * it.rows + nc[b].fixed});
         }

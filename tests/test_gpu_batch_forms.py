@@ -8,6 +8,7 @@ import pytest
 from paper_1612_01501_gb300 import inputs
 from paper_1612_01501_gb300 import ion
 
+from test_gpu_long_rows import hub_graph
 from test_gpu_parity import torch_cuda  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -20,6 +21,14 @@ def _dense(n):
 def _csr(n, k, weights="uniform", seed=5):
     rp, col = inputs.random_symmetric_csr(n, k, seed)
     w = np.full(len(col), inputs.junction_weight(0.04, k), np.float32)
+    if weights == "random":
+        w = (w * inputs.uniform(inputs.stream_seed(len(col), "batch_forms"), len(col), 0.5, 1.5)).astype(np.float32)
+    return dict(n=n, kind=ion.CSR, row_ptr=rp, col=col, w=w)
+
+
+def _hub(n, k, hubs, length, weights="uniform"):
+    rp, col = hub_graph(n, k, hubs, length)
+    w = np.full(len(col), 0.0005, np.float32)
     if weights == "random":
         w = (w * inputs.uniform(inputs.stream_seed(len(col), "batch_forms"), len(col), 0.5, 1.5)).astype(np.float32)
     return dict(n=n, kind=ion.CSR, row_ptr=rp, col=col, w=w)
@@ -41,6 +50,9 @@ SETS = {
     "dense": [_dense(n) for n in (1, 31, 64, 500, 1792)],
     "mixed": [_dense(300), _csr(1000, 50), _csr(300, 12, "random"), dict(n=200, kind=ion.NO_GJ), _dense(2000)],
     "csr": [_csr(2000, 24), _csr(33, 8), _csr(3000, 150, "random"), _csr(500, 70)],
+    # a row just within and just beyond four times the mean's rounds, and far beyond
+    "long_rows": [_hub(4000, 10, 2, 2000), _hub(400, 6, 1, 60), _hub(400, 6, 1, 66), _hub(3000, 40, 3, 900, "random"),
+                  _csr(1000, 24), _dense(200)],
 }
 
 
@@ -88,3 +100,35 @@ def test_persistent_step_is_within_twice_a_replayed_step(torch_cuda, nets):
         finally:
             ion.ion_destroy(h)
     assert us[1] <= 2.0 * us[0], us
+
+
+def test_batch_with_long_rows_matches_single_networks(torch_cuda):
+    nets = SETS["long_rows"]
+    S0 = _state(nets)
+    h = ion.ion_create_batch(nets, init_state=S0)
+    try:
+        ion.ion_step(h, 20)
+        got = ion.ion_read_state(h, S0.shape[1])
+    finally:
+        ion.ion_destroy(h)
+    off = 0
+    for b in nets:
+        n = b["n"]
+        with ion.Simulation(**b, init_state=S0[:, off:off + n]) as sim:
+            sim.step(20)
+            ref = sim.state()
+        assert np.abs(got[:3, off:off + n] - ref[:3]).max() <= 1e-3   # the sums' order, 20 steps
+        off += n
+
+
+# 18 times as long with one lane per row for every row
+@pytest.mark.parametrize("flags,most", [(0, 8), (ion.FLAG_PERSISTENT, 8)])
+def test_long_rows_do_not_hold_a_batch(torch_cuda, flags, most):
+    us = []
+    for nets in ([_csr(4000, 10)] * 6, [_hub(4000, 10, 2, 2000)] * 6):
+        h = ion.ion_create_batch(nets, init_state=_state(nets), flags=ion.FLAG_KAHAN | flags)
+        try:
+            us.append(us_per_step(h, 1, 200))
+        finally:
+            ion.ion_destroy(h)
+    assert us[1] <= most * us[0], us
