@@ -946,8 +946,8 @@ static cudaError_t enqueue_one_step(ion_sim *s, int k_off, const float *iapp) {
 
 // Enqueue k consecutive steps from offset 0 of the device step counter (iapp_base: their dense
 // evoked input), between the extension's fork and join if it has them.
-static cudaError_t enqueue_run(ion_sim *s, int k, const float *iapp_base) {
-    cudaError_t e = s->fork_hook ? s->fork_hook(s) : cudaSuccess;
+static cudaError_t enqueue_run(ion_sim *s, int k, const float *iapp_base, bool captured) {
+    cudaError_t e = s->fork_hook ? s->fork_hook(s, k, captured) : cudaSuccess;
     for (int j = 0; j < k && e == cudaSuccess; ++j)
         e = enqueue_one_step(s, j, iapp_base ? iapp_base + (int64_t)j * s->n : nullptr);
     if (s->join_hook) {
@@ -957,16 +957,16 @@ static cudaError_t enqueue_run(ion_sim *s, int k, const float *iapp_base) {
     return e;
 }
 
-// The counter's advance follows a step kernel (not, with an extension's join, an event): it may
-// be scheduled while that drains.
-static bool advance_pdl(const ion_sim *s) { return !(s->flags & ION_FLAG_NO_PDL) && !s->pdl_off && !s->join_hook; }
+// The counter's advance follows a step kernel (not, after a join, an event): it may be scheduled
+// while that drains.
+static bool advance_pdl(const ion_sim *s) { return !(s->flags & ION_FLAG_NO_PDL) && !s->pdl_off && !s->forked; }
 
 // Enqueue k steps directly (no graph) followed by the device counter advance.
 static cudaError_t enqueue_steps_direct(ion_sim *s, int64_t k, const float *iapp_base) {
     int64_t done = 0;
     while (done < k) {
         const int64_t chunk = std::min<int64_t>(k - done, 1 << 20);
-        cudaError_t e = enqueue_run(s, (int)chunk, iapp_base ? iapp_base + done * (int64_t)s->n : nullptr);
+        cudaError_t e = enqueue_run(s, (int)chunk, iapp_base ? iapp_base + done * (int64_t)s->n : nullptr, false);
         if (e != cudaSuccess) return e;
         e = launch_advance(s->d_t, chunk, s->st, advance_pdl(s));
         s->launches++;
@@ -982,7 +982,7 @@ static ion_status build_graph_once(ion_sim *s) {
     cudaGraph_t g = nullptr;
     const int64_t launches0 = s->launches;
     ION_CK(s, cudaStreamBeginCapture(s->st, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = enqueue_run(s, K, nullptr);
+    cudaError_t e = enqueue_run(s, K, nullptr, true);
     if (e == cudaSuccess) e = launch_advance(s->d_t, K, s->st, advance_pdl(s));
     cudaError_t e2 = cudaStreamEndCapture(s->st, &g);
     s->launches = launches0;

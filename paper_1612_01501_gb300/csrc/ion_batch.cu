@@ -738,6 +738,9 @@ struct BatchExt {
         int vbuf = 256, rows_max = 32;  // shared memory of its launches
     };
     std::vector<Chain> chains;
+    std::vector<Chain> whole;           // the same tiles, one list per kind: runs on one stream
+    int one_steps = 0;                  // direct runs of up to so many steps are
+    bool on_one = false;                // the present run is one
     cudaStream_t side[BATCH_CHAINS - 1] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[BATCH_CHAINS - 1] = {};
     bool forked_now = false;            // the next step is the first after a fork
@@ -943,6 +946,24 @@ static ion_status batch_plan(ion_sim *s) {
         if (T.kind == TILE_DENSE || (T.mode & TILE_STAGE_V)) C.vbuf = std::max(C.vbuf, T.n_pad);
         C.rows_max = std::max(C.rows_max, T.rows);
     }
+    X->whole.clear();
+    for (const BatchExt::Chain &C : X->chains) {   // the chains of a kind lie one after the other
+        if (X->whole.empty() || X->whole.back().dense != C.dense) {
+            X->whole.push_back(C);
+            continue;
+        }
+        BatchExt::Chain &W = X->whole.back();
+        W.n += C.n;
+        W.vbuf = std::max(W.vbuf, C.vbuf);
+        W.rows_max = std::max(W.rows_max, C.rows_max);
+    }
+    // Forking and joining costs the host 4 to 5 us per call, more than the chains save in a few
+    // steps.  us per step of a call of k steps, chains / one stream: two dense networks of 64 cells
+    // 9.1 / 5.3 (k = 1), 4.1 / 3.7 (40); twelve of 1792 14.7 / 12.4 (1), 11.4 / 10.9 (4), 10.0 / 10.6
+    // (10); a dense and a CSR network of 500 9.6 / 7.8 (1), 6.5 / 7.0 (2); 96 networks of 32-4096 33.2
+    // / 35.5 (1).
+    const double total = std::accumulate(net_cost.begin(), net_cost.end(), 0.0);
+    X->one_steps = total > 6.0e7 ? 0 : X->whole.size() > 1 ? 1 : (int)sorted.size() <= s->sms ? INT32_MAX : 4;
     s->lps = (int64_t)X->chains.size();
     cudaError_t e = cudaStreamSynchronize(s->st);
     ion_drop_graphs(s);   // the captured steps hold the old tile list
@@ -999,14 +1020,15 @@ static cudaError_t batch_step(ion_sim *s, int k_off, const float *iapp) {
     a.soff = X->d_soff;
     a.kahan = 1;
     cudaError_t e = cudaSuccess;
-    for (size_t q = 0; q < X->chains.size() && e == cudaSuccess; ++q) {
-        const BatchExt::Chain &C = X->chains[q];
+    const std::vector<BatchExt::Chain> &run = X->on_one ? X->whole : X->chains;
+    for (size_t q = 0; q < run.size() && e == cudaSuccess; ++q) {
+        const BatchExt::Chain &C = run[q];
         a.tiles = X->d_tiles + C.off;
         a.rows_max = C.rows_max;
         a.vbuf = C.vbuf;
         // a side stream's first launch follows the fork event, not a kernel: an ordinary launch
         const bool pdl = a.c.pdl && !(q > 0 && X->forked_now);
-        e = batch_launch(a, C.dense, X->R, C.n, batch_smem(X, C), pdl, q == 0 ? s->st : X->side[q - 1]);
+        e = batch_launch(a, C.dense, X->R, C.n, batch_smem(X, C), pdl, q == 0 || X->on_one ? s->st : X->side[q - 1]);
         s->launches++;
     }
     X->forked_now = false;
@@ -1014,19 +1036,22 @@ static cudaError_t batch_step(ion_sim *s, int k_off, const float *iapp) {
 }
 
 // Before the steps of a captured graph or of a direct run: the side streams start after the
-// handle's stream; after them the handle's stream continues when every chain is done.
-static cudaError_t batch_fork(ion_sim *s) {
+// handle's stream; after them the handle's stream continues when every chain is done.  A direct run
+// of few steps stays on the handle's stream (one_steps).
+static cudaError_t batch_fork(ion_sim *s, int steps, bool captured) {
     BatchExt *X = ext_of(s);
-    if (X->chains.size() < 2) return cudaSuccess;
+    X->on_one = !captured && steps <= X->one_steps;
+    s->forked = !X->on_one && X->chains.size() > 1;
+    X->forked_now = s->forked;
+    if (!s->forked) return cudaSuccess;
     cudaError_t e = cudaEventRecord(X->ev_fork, s->st);
     for (size_t q = 1; q < X->chains.size() && e == cudaSuccess; ++q) e = cudaStreamWaitEvent(X->side[q - 1], X->ev_fork, 0);
-    X->forked_now = true;
     return e;
 }
 static cudaError_t batch_join(ion_sim *s) {
     BatchExt *X = ext_of(s);
     cudaError_t e = cudaSuccess;
-    for (size_t q = 1; q < X->chains.size(); ++q) {   // every side stream joins, also after an error
+    for (size_t q = 1; s->forked && q < X->chains.size(); ++q) {   // every side stream joins, also after an error
         cudaError_t e1 = cudaEventRecord(X->ev_join[q - 1], X->side[q - 1]);
         if (e1 == cudaSuccess) e1 = cudaStreamWaitEvent(s->st, X->ev_join[q - 1], 0);
         if (e == cudaSuccess) e = e1;
@@ -1274,8 +1299,8 @@ static ion_status batch_persist_run(ion_sim *s, int64_t n_steps, const float *ia
 static ion_status batch_prepare(ion_sim *s) {
     BatchExt *X = ext_of(s);
     cudaError_t e = cudaSuccess;
-    for (size_t q = 0; q < X->chains.size() && e == cudaSuccess; ++q)
-        e = batch_allow_smem(X->chains[q].dense, X->R, batch_smem(X, X->chains[q]));
+    for (size_t q = 0; q < X->whole.size() && e == cudaSuccess; ++q)   // as large as any chain's need
+        e = batch_allow_smem(X->whole[q].dense, X->R, batch_smem(X, X->whole[q]));
     if (e == cudaSuccess && !X->ev_fork) e = cudaEventCreateWithFlags(&X->ev_fork, cudaEventDisableTiming);
     for (size_t q = 1; q < X->chains.size() && e == cudaSuccess; ++q) {
         if (!X->side[q - 1]) e = cudaStreamCreateWithFlags(&X->side[q - 1], cudaStreamNonBlocking);

@@ -96,8 +96,10 @@ struct ion_sim {
 
     // extension points (persistent, batched and surrogate variants)
     cudaError_t (*step_override)(ion_sim *, int k_off, const float *iapp) = nullptr;
-    cudaError_t (*fork_hook)(ion_sim *) = nullptr;   // around a run of step_override calls
+    // around a run of `steps` step_override calls, captured into a graph or launched now
+    cudaError_t (*fork_hook)(ion_sim *, int steps, bool captured) = nullptr;
     cudaError_t (*join_hook)(ion_sim *) = nullptr;
+    bool forked = false;            // the run uses streams beside st
     ion_status (*run_override)(ion_sim *, int64_t n_steps, const float *iapp) = nullptr;
     ion_status (*prepare_hook)(ion_sim *) = nullptr;
     ion_status (*state_sync_hook)(ion_sim *) = nullptr;

@@ -74,6 +74,56 @@ def test_persistent_launch_gives_the_bits_of_step_launches(torch_cuda, which, tu
     assert np.array_equal(out[0], out[1])
 
 
+@pytest.mark.parametrize("which", SETS)
+def test_calls_of_few_steps_give_the_bits_of_replays(torch_cuda, which):
+    """Direct runs of 1, 2, 4, 5 and 9 steps (on one stream or on chains beside it), with a device
+    input rewritten on the stream right before a call and a state read after it, against graph
+    replays and ordinary launches."""
+    torch = torch_cuda
+    nets = SETS[which]
+    S0 = _state(nets)
+    n = S0.shape[1]
+    stream = torch.cuda.Stream()
+    calls = [1, 1, 2, 4, 5, 9, 1, 2, 1] * 2
+    out = []
+    for flags in (0, ion.FLAG_NO_PDL, ion.FLAG_NO_GRAPH):
+        big = torch.zeros(32 << 20, dtype=torch.float32, device="cuda")
+        drive = torch.zeros((9, n), dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        h = ion.ion_create_batch(nets, init_state=S0, flags=ion.FLAG_KAHAN | flags, stream=stream.cuda_stream)
+        try:
+            ion.ion_set_input(h, _pulses(n))
+            with torch.cuda.stream(stream):
+                for q, k in enumerate(calls):
+                    if q % 3 == 1:
+                        big.add_(0.25)
+                        drive.copy_(big[-9 * n:].view(9, n))
+                        ion.ion_step(h, k, dense=drive[:k])
+                    else:
+                        ion.ion_step(h, k)
+                    if q % 4 == 3:
+                        ion.ion_read_state(h, n, 2)
+                ion.ion_step(h, 103)
+            out.append(ion.ion_read_state(h, n))
+        finally:
+            ion.ion_destroy(h)
+    assert np.isfinite(out[0]).all()
+    assert np.array_equal(out[0], out[1])
+    assert np.array_equal(out[0], out[2])
+
+
+def test_a_call_of_one_step_costs_few_launches(torch_cuda):
+    """One launch per kind of network and the counter's, without forking to other streams."""
+    for nets, launches in ((SETS["dense"][1:4], 2), ([_dense(500), _csr(500, 20)], 3)):
+        h = ion.ion_create_batch(nets, init_state=_state(nets))
+        try:
+            before = ion.ion_launch_count(h)
+            ion.ion_step(h, 1)
+            assert ion.ion_launch_count(h) - before == launches
+        finally:
+            ion.ion_destroy(h)
+
+
 def us_per_step(h, calls, steps):
     def run():
         for _ in range(calls):
