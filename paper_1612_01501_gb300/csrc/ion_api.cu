@@ -866,6 +866,17 @@ StepCommon ion_step_common(ion_sim *s, int k_off, const float *iapp) {
     return c;
 }
 
+// The update launch of a step whose currents are a launch of their own.  After dense currents of more
+// than 2500 cells it is an ordinary launch: scheduled early, its CTAs go where the currents' CTAs
+// leave room, several to an SM, and the update then runs on a part of the chip.  us per step early
+// / ordinary: learned rates 2 000 cells 11.8 / 11.8, 4 096 17.0 / 13.7, 8 192 23.6 / 20.3; SPLIT 2 000
+// 4.9 / 5.4, 2 999 7.3 / 6.0, 8 192 14.9 / 13.8, 16 384 39.6 / 40.2.
+StepCommon ion_update_common(const ion_sim *s, const StepCommon &c) {
+    StepCommon u = c;
+    if (s->kind == ION_DENSE_UNIFORM && s->n > 2500) u.pdl = 0;
+    return u;
+}
+
 // Enqueue one step (offset k_off from the device step counter).
 static cudaError_t enqueue_one_step(ion_sim *s, int k_off, const float *iapp) {
     if (s->step_override) return s->step_override(s, k_off, iapp);
@@ -908,7 +919,7 @@ static cudaError_t enqueue_one_step(ion_sim *s, int k_off, const float *iapp) {
         e = launch_dense_step(a, s->dense_R, s->dense_W, s->dense_GJ, s->st);
         s->launches++;
         if (e == cudaSuccess && split) {
-            CellArgs ca{c, s->d_ic, s->d_cellp};
+            CellArgs ca{ion_update_common(s, c), s->d_ic, s->d_cellp};
             e = launch_cell_step(ca, s->st);
             s->launches++;
         }
@@ -932,7 +943,7 @@ static cudaError_t enqueue_one_step(ion_sim *s, int k_off, const float *iapp) {
         e = ion_launch_csr(s, a);
         s->launches++;
         if (e == cudaSuccess && split) {
-            CellArgs ca{c, s->d_ic, s->d_cellp};
+            CellArgs ca{ion_update_common(s, c), s->d_ic, s->d_cellp};
             e = launch_cell_step(ca, s->st);
             s->launches++;
         }

@@ -122,6 +122,7 @@ inline cudaError_t ion_alloc(T **p, size_t bytes) {
 
 // shared helpers (ion_api.cu)
 void ion_csr_fill(const ion_sim *s, ion::CsrArgs &a, bool staged);
+ion::StepCommon ion_update_common(const ion_sim *s, const ion::StepCommon &c);
 cudaError_t ion_launch_csr(const ion_sim *s, const ion::CsrArgs &a);
 ion_status ion_prepare_csr_chunk(ion_sim *s);
 ion::SliceLayout ion_plan_sliced(int32_t n, int32_t n_pad, int64_t nnz, int sms, int lanes);
