@@ -167,7 +167,10 @@ typedef struct {
     const void *tune;           /* ion_tune* launch shape override, NULL = built-in choice */
     int64_t debug_delay_ns;     /* test hook, 0 in production: with ION_FLAG_PERSISTENT one CTA
                                    sleeps this long before its first grid barrier (a short
-                                   barrier_timeout_ns then yields ION_ERR_TIMEOUT)          */
+                                   barrier_timeout_ns then yields ION_ERR_TIMEOUT); with
+                                   ION_FLAG_SURROGATE on tcgen05, k = 1..6: the k-th of a step's
+                                   six tensor-core completions is never signalled to the first
+                                   128 cells' CTA (its 0.5 s wait then yields the same)     */
     const float *cell_params;   /* per-cell model constants (Table "reqs": every neuron has its
                                    own conductances), or NULL for the model table's values in
                                    every cell.  Host FP32 array of ION_NCELLPARAMS x n_cells,

@@ -377,7 +377,8 @@ size_t dense_smem_bytes(int n_pad, int rows_per_warp, int warps);
 size_t surrogate_tc_weights_bytes();
 cudaError_t surrogate_tc_prepare();
 cudaError_t surrogate_tc_pack(const ion_surrogate_weights *d_w, void *d_out, cudaStream_t st);
-cudaError_t launch_surrogate_tc(const StepCommon &c, const void *W, const float *ic, cudaStream_t st);
+// withhold: test hook, 1..6: CTA 0's withhold-th tensor-core completion is never signalled
+cudaError_t launch_surrogate_tc(const StepCommon &c, const void *W, const float *ic, int withhold, cudaStream_t st);
 cudaError_t launch_mlp_eval_tc(const void *W, int64_t n, const float *V, const float *ca, float *out,
                                uint32_t *status, cudaStream_t st);
 

@@ -942,7 +942,8 @@ static cudaError_t surrogate_step(ion_sim *s, int k_off, const float *iapp) {
     s->launches++;
     const float *ic = s->kind == ION_NO_GJ ? nullptr : s->d_ic;
     const StepCommon cu = ion_update_common(s, c);
-    if (!(s->flags & ION_FLAG_SURROGATE_WARP_MMA)) return launch_surrogate_tc(cu, s->d_mlp_tc, ic, s->st);
+    if (!(s->flags & ION_FLAG_SURROGATE_WARP_MMA)) 
+        return launch_surrogate_tc(cu, s->d_mlp_tc, ic, (int)std::min<int64_t>(s->debug_delay_ns, 7), s->st);
     SurrArgs sa{cu, (const MlpDev *)s->d_mlp, ic};
     return launch_k(surrogate_cell_kernel, dim3((unsigned)((s->n + 2 * SURR_CPW - 1) / (2 * SURR_CPW))), dim3(64), 0,
                     s->st, c.pdl != 0, sa);

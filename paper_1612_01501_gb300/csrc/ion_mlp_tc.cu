@@ -28,8 +28,10 @@
 // (8 g + c) 128, so the K-direction core-matrix stride (leading byte offset) is 128 B and
 // the row-group stride (stride byte offset) 1024 B.
 // Every wait is bounded: a tensor-core completion that does not arrive within ~0.5 s sets
-// the timeout status bit; the CTA then waits (again bounded) once more, frees its TMEM and
-// returns.
+// the timeout status bit.  A warp whose wait ran out neither reads the accumulators nor writes
+// the operands from there on, and thread 0 issues nothing once its own has; at the end the CTA
+// waits (again bounded) once more for what is in flight, frees its TMEM and returns without
+// having stored a word: its cells keep step t.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -130,23 +132,30 @@ __device__ __forceinline__ uint32_t tanh_bf16x2(uint32_t x) {
 }
 
 // Hand buffer b to the tensor core (all threads): its generic writes are ordered before the
-// asynchronous reads, then thread 0 issues the layer's four K = 16 steps and the commit.
-__device__ __forceinline__ void tc_issue(Smem &sm, int b, const __nv_bfloat16 *B, uint32_t idesc) {
+// asynchronous reads, then thread 0 issues the layer's four K = 16 steps and the commit, unless one
+// of its own waits has run out (`ok`: those before it have then not been seen to complete).
+// issued[b] counts thread 0's layers.  withhold: test hook, the commit is left out, so that the
+// wait for this layer runs out.
+__device__ __forceinline__ void tc_issue(Smem &sm, int b, const __nv_bfloat16 *B, uint32_t idesc, bool ok,
+                                         uint32_t (&issued)[2], bool withhold) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && ok) {
+        issued[b]++;
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < KH / 16; ++kk)
             tc_mma(sm.tmem + b * N2, smem_desc(sm.a[b] + kk * 16 * 8, 128, 1024), smem_desc(B + kk * 16 * 8, 128, 1024),
                    idesc, kk > 0 ? 1u : 0u);
-        tc_commit(&sm.bar[b]);
+        if (!withhold) tc_commit(&sm.bar[b]);
     }
 }
-// Wait (bounded) for the layer last issued on buffer b; false if it did not complete in time.
-__device__ __forceinline__ bool tc_wait(Smem &sm, int b, uint32_t phase) {
-    const bool done = mbar_wait_bounded(&sm.bar[b], phase);
+// Wait (bounded) for the layer last issued on buffer b; false, in every lane of the warp, if a lane
+// of it did not see the completion in time, or (ok) an earlier wait of the warp ran out.
+__device__ __forceinline__ bool tc_wait(Smem &sm, int b, uint32_t phase, bool ok) {
+    if (!ok) return false;
+    const bool done = __all_sync(0xffffffffu, mbar_wait_bounded(&sm.bar[b], phase));
     tc_fence_after();
     return done;
 }
@@ -191,7 +200,7 @@ __device__ __forceinline__ void layer2_epilogue(Smem &sm, int c, uint32_t lane_a
 }
 
 // CTA prologue: TMEM columns (warp 0), weights into shared memory by one bulk copy, mbarriers.
-// The weights are waited for where they are first read (tc_weights).
+// The weights are waited for where they are first read (wbar).
 __device__ __forceinline__ void tc_setup(Smem &sm, const Weights *Wg) {
     if (threadIdx.x < 32) {
         tmem_alloc(&sm.tmem, TMEM_COLS);
@@ -226,14 +235,15 @@ __device__ __forceinline__ void tc_outputs(Smem &sm, int b, float (&y)[NOUT]) {
 #pragma unroll
     for (int o = 0; o < NOUT; ++o) y[o] = fmaf(v[o] + sm.W.b3[o], sm.W.out_scale[o], sm.W.out_shift[o]);
 }
-// After the last wait (all threads): reports a completion that did not come in time and waits
-// once more (bounded) for both buffers' MMAs, so that the TMEM they write can be freed.
-__device__ __forceinline__ bool tc_finish(Smem &sm, bool ok, uint32_t *status, uint32_t phase0, uint32_t phase1) {
+// After the last wait (all threads): true if every wait of the CTA succeeded.  Else reports the
+// timeout and waits once more (bounded) for the layers and the copy in flight, so that the TMEM they
+// write can be freed.
+__device__ __forceinline__ bool tc_finish(Smem &sm, bool ok, uint32_t *status, const uint32_t (&issued)[2]) {
     if (!__syncthreads_or(!ok)) return true;
     if (threadIdx.x == 0) {
         if (status != nullptr) atomicOr(status, (uint32_t)ST_TIMEOUT);
-        (void)mbar_wait_bounded(&sm.bar[0], phase0);
-        (void)mbar_wait_bounded(&sm.bar[1], phase1);
+        for (int b = 0; b < 2; ++b)
+            if (issued[b] > 0) (void)mbar_wait_bounded(&sm.bar[b], (issued[b] - 1u) & 1u);
         (void)mbar_wait_bounded(&sm.wbar, 0u);
     }
     return false;
@@ -252,6 +262,7 @@ struct SurrTcArgs {
     StepCommon c;
     const tc::Weights *W;
     const float *ic;    // gap currents of this step (NULL: none)
+    int32_t withhold;   // test hook: CTA 0 leaves out its withhold-th commit (0: none)
 };
 
 // The cell update with learned rates: 128 cells per CTA, three tensor-core tiles (dendrite and
@@ -275,68 +286,82 @@ __global__ void __launch_bounds__(128) surrogate_tc_kernel(const SurrTcArgs a) {
     const float ic = valid && a.ic != nullptr ? a.ic[i] : 0.0f;
     float iapp = pulse_current(c.pulses, pa, t);
     if (c.iapp != nullptr && valid) iapp += c.iapp[i];
-    bool ok = mbar_wait_bounded(&sm.wbar, 0u);   // the weights
-    const int row = threadIdx.x;
-    const float dt = c.P.dt, x1 = (logf(cell.ca) - sm.W.in_shift[1]) * sm.W.in_scale[1];
+    const int row = threadIdx.x, hook = blockIdx.x == 0 ? a.withhold : 0;
+    const float dt = c.P.dt;
     auto x0 = [&](float V) { return (V - sm.W.in_shift[0]) * sm.W.in_scale[0]; };
     constexpr uint32_t L2 = tc::idesc_bf16(tc::ROWS, tc::N2), L3 = tc::idesc_bf16(tc::ROWS, tc::N3);
     float y[tc::NOUT];
+    // The new words stay in registers until every completion has been seen: nothing of a cell is
+    // stored if one does not arrive (0.2 us of a step's 21.4 at 65 536 cells, k = 100).
+    DendNext d{};
+    float r1 = 0.0f, s1 = 0.0f, q1 = 0.0f, ms = 0.0f, vs = 0.0f, k1 = 0.0f, l1 = 0.0f, hs1 = 0.0f, ns1 = 0.0f, xs1 = 0.0f;
+    uint32_t issued[2] = {0u, 0u};
+    bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&sm.wbar, 0u));   // the weights
+    const float x1 = (logf(cell.ca) - sm.W.in_shift[1]) * sm.W.in_scale[1];
     tc::layer1_row(sm, 0, row, x0(cell.vd), x1);
-    tc::tc_issue(sm, 0, sm.W.w2, L2);
+    tc::tc_issue(sm, 0, sm.W.w2, L2, ok, issued, hook == 1);
     tc::layer1_row(sm, 1, row, x0(cell.vs), x1);
-    tc::tc_issue(sm, 1, sm.W.w2, L2);
-    ok = tc::tc_wait(sm, 0, 0u) && ok;
-    tc::layer2_epilogue(sm, 0, tc::tc_lane(sm, 0), row);
-    tc::tc_issue(sm, 0, sm.W.w3, L3);
-    ok = tc::tc_wait(sm, 1, 0u) && ok;
-    tc::layer2_epilogue(sm, 1, tc::tc_lane(sm, 1), row);
-    tc::tc_issue(sm, 1, sm.W.w3, L3);
+    tc::tc_issue(sm, 1, sm.W.w2, L2, ok, issued, hook == 2);
+    ok = tc::tc_wait(sm, 0, 0u, ok);
+    if (ok) tc::layer2_epilogue(sm, 0, tc::tc_lane(sm, 0), row);
+    tc::tc_issue(sm, 0, sm.W.w3, L3, ok, issued, hook == 3);
+    ok = tc::tc_wait(sm, 1, 0u, ok);
+    if (ok) tc::layer2_epilogue(sm, 1, tc::tc_lane(sm, 1), row);
+    tc::tc_issue(sm, 1, sm.W.w3, L3, ok, issued, hook == 4);
     // dendrite: its outputs, then the axon's layer 1 into the buffer they leave
-    ok = tc::tc_wait(sm, 0, 1u) && ok;
-    tc::tc_outputs(sm, 0, y);
-    tc::layer1_row(sm, 0, row, x0(cell.va), x1);
-    tc::tc_issue(sm, 0, sm.W.w2, L2);
-    bool finite = true;
-    if (valid) {
-        const DendNext d = dend_step(c.P, cell, ic, iapp);
-        vnext[i] = d.vd;
-        c.S.f(F_CA)[i] = d.ca;
-        c.S.f(F_ICAH)[i] = d.icah;
-        c.S.f(F_IC)[i] = ic;
-        c.S.f(F_R)[i] = relax(cell.r, tc::learned_rate(y, G_R), dt);
-        c.S.f(F_S)[i] = relax(cell.s, tc::learned_rate(y, G_S), dt);
-        c.S.f(F_Q)[i] = relax(cell.q, tc::learned_rate(y, G_Q), dt);
-        finite = isfinite(d.vd) && isfinite(d.ca);
+    ok = tc::tc_wait(sm, 0, 1u, ok);
+    if (ok) {
+        tc::tc_outputs(sm, 0, y);
+        tc::layer1_row(sm, 0, row, x0(cell.va), x1);
+    }
+    tc::tc_issue(sm, 0, sm.W.w2, L2, ok, issued, hook == 5);
+    if (ok) {
+        d = dend_step(c.P, cell, ic, iapp);
+        r1 = relax(cell.r, tc::learned_rate(y, G_R), dt);
+        s1 = relax(cell.s, tc::learned_rate(y, G_S), dt);
+        q1 = relax(cell.q, tc::learned_rate(y, G_Q), dt);
     }
     // soma
-    ok = tc::tc_wait(sm, 1, 1u) && ok;
-    tc::tc_outputs(sm, 1, y);
-    if (valid) {
-        const float ms = tc::learned_xinf(y, G_MS), vs = soma_step(c.P, cell, ms);
-        c.S.f(F_VSOMA)[i] = vs;
-        c.S.f(F_MS)[i] = ms;
-        c.S.f(F_K)[i] = relax(cell.k, tc::learned_rate(y, G_K), dt);
-        c.S.f(F_L)[i] = relax(cell.l, tc::learned_rate(y, G_L), dt);
-        c.S.f(F_HS)[i] = relax(cell.hs, tc::learned_rate(y, G_HS), dt);
-        c.S.f(F_NS)[i] = relax(cell.ns, tc::learned_rate(y, G_NS), dt);
-        c.S.f(F_XS)[i] = relax(cell.xs, tc::learned_rate(y, G_XS), dt);
-        finite = finite && isfinite(vs);
+    ok = tc::tc_wait(sm, 1, 1u, ok);
+    if (ok) {
+        tc::tc_outputs(sm, 1, y);
+        ms = tc::learned_xinf(y, G_MS);
+        vs = soma_step(c.P, cell, ms);
+        k1 = relax(cell.k, tc::learned_rate(y, G_K), dt);
+        l1 = relax(cell.l, tc::learned_rate(y, G_L), dt);
+        hs1 = relax(cell.hs, tc::learned_rate(y, G_HS), dt);
+        ns1 = relax(cell.ns, tc::learned_rate(y, G_NS), dt);
+        xs1 = relax(cell.xs, tc::learned_rate(y, G_XS), dt);
     }
     // axon
-    ok = tc::tc_wait(sm, 0, 0u) && ok;
-    tc::layer2_epilogue(sm, 0, tc::tc_lane(sm, 0), row);
-    tc::tc_issue(sm, 0, sm.W.w3, L3);
-    ok = tc::tc_wait(sm, 0, 1u) && ok;
-    tc::tc_outputs(sm, 0, y);
-    ok = tc::tc_finish(sm, ok, c.status, 1u, 1u);
+    ok = tc::tc_wait(sm, 0, 0u, ok);
+    if (ok) tc::layer2_epilogue(sm, 0, tc::tc_lane(sm, 0), row);
+    tc::tc_issue(sm, 0, sm.W.w3, L3, ok, issued, hook == 6);
+    ok = tc::tc_wait(sm, 0, 1u, ok);
+    if (ok) tc::tc_outputs(sm, 0, y);
+    const bool all = tc::tc_finish(sm, ok, c.status, issued);
     tc::tc_teardown(sm);
-    if (!ok || !valid) return;
+    if (!all || !valid) return;
     const float ma = tc::learned_xinf(y, G_MA), va = axon_step(c.P, cell, ma);
+    vnext[i] = d.vd;
+    c.S.f(F_CA)[i] = d.ca;
+    c.S.f(F_ICAH)[i] = d.icah;
+    c.S.f(F_IC)[i] = ic;
+    c.S.f(F_R)[i] = r1;
+    c.S.f(F_S)[i] = s1;
+    c.S.f(F_Q)[i] = q1;
+    c.S.f(F_VSOMA)[i] = vs;
+    c.S.f(F_MS)[i] = ms;
+    c.S.f(F_K)[i] = k1;
+    c.S.f(F_L)[i] = l1;
+    c.S.f(F_HS)[i] = hs1;
+    c.S.f(F_NS)[i] = ns1;
+    c.S.f(F_XS)[i] = xs1;
     c.S.f(F_VAXON)[i] = va;
     c.S.f(F_MA)[i] = ma;
     c.S.f(F_HA)[i] = relax(cell.ha, tc::learned_rate(y, G_HA), dt);
     c.S.f(F_XA)[i] = relax(cell.xa, tc::learned_rate(y, G_XA), dt);
-    if (!finite || !isfinite(va)) atomicOr(c.status, (uint32_t)ST_NONFINITE);
+    if (!(isfinite(d.vd) && isfinite(d.ca) && isfinite(vs) && isfinite(va))) atomicOr(c.status, (uint32_t)ST_NONFINITE);
     if (c.par >= 0 && (int)(t & 1) != c.par) atomicOr(c.status, (uint32_t)ST_SLOT);
     if (c.trace != nullptr && ((t + 1) % c.trace_stride) == 0) {
         const int64_t sample = (t + 1) / c.trace_stride - 1;
@@ -352,26 +377,22 @@ __global__ void __launch_bounds__(128) mlp_eval_tc_kernel(const tc::Weights *Wg,
     tc::tc_setup(sm, Wg);
     const int64_t k = (int64_t)blockIdx.x * tc::ROWS + threadIdx.x;
     const bool valid = k < n;
-    bool ok = mbar_wait_bounded(&sm.wbar, 0u);   // the weights
+    const uint32_t lane = tc::tc_lane(sm, 0);
+    uint32_t issued[2] = {0u, 0u};
+    float y[tc::NOUT];
+    bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&sm.wbar, 0u));   // the weights
     const float x0 = valid ? (V[k] - sm.W.in_shift[0]) * sm.W.in_scale[0] : 0.0f;
     const float x1 = valid ? (logf(ca[k]) - sm.W.in_shift[1]) * sm.W.in_scale[1] : 0.0f;
-    float y[tc::NOUT];
     tc::layer1_row(sm, 0, threadIdx.x, x0, x1);
-    tc::tc_issue(sm, 0, sm.W.w2, tc::idesc_bf16(tc::ROWS, tc::N2));
-    ok = tc::tc_wait(sm, 0, 0u) && ok;
-    tc::layer2_epilogue(sm, 0, tc::tc_lane(sm, 0), threadIdx.x);
-    tc::tc_issue(sm, 0, sm.W.w3, tc::idesc_bf16(tc::ROWS, tc::N3));
-    ok = tc::tc_wait(sm, 0, 1u) && ok;
-    tc::tc_outputs(sm, 0, y);
-    if (!__syncthreads_or(!ok)) {
-        if (valid)
+    tc::tc_issue(sm, 0, sm.W.w2, tc::idesc_bf16(tc::ROWS, tc::N2), ok, issued, false);
+    ok = tc::tc_wait(sm, 0, 0u, ok);
+    if (ok) tc::layer2_epilogue(sm, 0, lane, threadIdx.x);
+    tc::tc_issue(sm, 0, sm.W.w3, tc::idesc_bf16(tc::ROWS, tc::N3), ok, issued, false);
+    ok = tc::tc_wait(sm, 0, 1u, ok);
+    if (ok) tc::tc_outputs(sm, 0, y);
+    if (tc::tc_finish(sm, ok, status, issued) && valid)
 #pragma unroll
-            for (int o = 0; o < tc::NOUT; ++o) out[k * tc::NOUT + o] = y[o];
-    } else if (threadIdx.x == 0) {
-        atomicOr(status, (uint32_t)ST_TIMEOUT);
-        (void)mbar_wait_bounded(&sm.bar[0], 1u);
-        (void)mbar_wait_bounded(&sm.wbar, 0u);
-    }
+        for (int o = 0; o < tc::NOUT; ++o) out[k * tc::NOUT + o] = y[o];
     tc::tc_teardown(sm);
 }
 
@@ -421,8 +442,8 @@ cudaError_t surrogate_tc_pack(const ion_surrogate_weights *d_w, void *d_out, cud
     return cudaGetLastError();
 }
 
-cudaError_t launch_surrogate_tc(const StepCommon &c, const void *W, const float *ic, cudaStream_t st) {
-    SurrTcArgs a{c, static_cast<const tc::Weights *>(W), ic};
+cudaError_t launch_surrogate_tc(const StepCommon &c, const void *W, const float *ic, int withhold, cudaStream_t st) {
+    SurrTcArgs a{c, static_cast<const tc::Weights *>(W), ic, withhold};
     return launch_k(surrogate_tc_kernel, dim3((unsigned)((c.n + tc::ROWS - 1) / tc::ROWS)), dim3(tc::ROWS), kTcSmem,
                     st, c.pdl != 0, a);
 }
