@@ -32,3 +32,23 @@ def test_direct_csr_fuses_the_product_into_the_sum(torch_cuda):
     twice = p[:, 0].astype(np.float32) + p[:, 1].astype(np.float32)
     assert (fused != twice).mean() > 0.1
     assert np.array_equal(ic, fused)
+
+
+def test_one_cta_sums_are_as_accurate_as_the_step_launches(torch_cuda):
+    """Gap currents of the one-CTA kernel and of the per-step launches (both compensated) against 64
+    bits, relative to the sum of the terms' magnitudes, over 240 random states: the mean of the
+    rms errors is the same to 0.8 % (plain chains of up to 24 terms: 1.6 % larger)."""
+    rms = np.zeros(2)
+    for n in (64, 99, 130, 192):
+        for seed in range(60):
+            S = ion.ion_default_state(n)
+            S[0] = (-60 + np.random.default_rng(seed + n).normal(0, 8, n)).astype(np.float32)
+            V = S[0].astype(np.float64)
+            d = V[:, None] - V[None, :]
+            f = float(np.float32(1e-3)) * (0.8 * np.exp(-d * d / 100) + 0.2) * d
+            for q, flags in enumerate((0, ion.FLAG_PERSISTENT)):
+                with ion.Simulation(n, ion.DENSE_UNIFORM, g=1e-3, init_state=S, flags=ion.FLAG_KAHAN | flags) as sim:
+                    sim.step(1)
+                    e = (sim.state(18) - f.sum(1)) / np.abs(f).sum(1)
+                rms[q] += np.sqrt((e * e).mean())
+    assert rms[1] <= 1.008 * rms[0], rms
