@@ -45,13 +45,13 @@ static MatrixShape matrix_shape(int n, int n_pad, int sms) {
     s.GR = MX_WARPS / s.GJ;
     return s;
 }
-// u of the rows, [rows][GJ] partial sums, the rows' state words
-static size_t matrix_smem_bytes(const MatrixShape &s) { return (size_t)s.rows * (1 + s.GJ + NCW) * sizeof(float); }
+// u of the rows, [rows][GJ] partial sums and their compensations, the rows' state words
+static size_t matrix_smem_bytes(const MatrixShape &s) { return (size_t)s.rows * (1 + 2 * s.GJ + NCW) * sizeof(float); }
 
 template <int R>
 __global__ void __launch_bounds__(MX_THREADS, 1) matrix_step_kernel(const MatrixArgs a, const MatrixShape S) {
     extern __shared__ __align__(16) float mx_smem[];
-    float *u_s = mx_smem, *part = u_s + S.rows, *cs = part + S.rows * S.GJ;
+    float *u_s = mx_smem, *part = u_s + S.rows, *comp = part + S.rows * S.GJ, *cs = comp + S.rows * S.GJ;
     const StepCommon &c = a.c;
     const int n = c.n, n_pad = c.n_pad;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -123,7 +123,12 @@ __global__ void __launch_bounds__(MX_THREADS, 1) matrix_step_kernel(const Matrix
                     float v = acc.x + acc.y;
 #pragma unroll
                     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-                    if (lane == 0) part[r * S.GJ + sp] = tile > 0 ? part[r * S.GJ + sp] + v : v;
+                    if (lane == 0) {   // further column tiles (n > 8192) are added with compensation
+                        float ks = tile > 0 ? part[r * S.GJ + sp] : 0.0f, kc = tile > 0 ? comp[r * S.GJ + sp] : 0.0f;
+                        kahan_add(ks, kc, v);
+                        part[r * S.GJ + sp] = ks;
+                        comp[r * S.GJ + sp] = kc;
+                    }
                 }
             }
         }
@@ -132,14 +137,14 @@ __global__ void __launch_bounds__(MX_THREADS, 1) matrix_step_kernel(const Matrix
     __syncthreads();
     if (!has_row) return;
     float ks = 0.0f, kc = 0.0f;
-    for (int q = 0; q < S.GJ; ++q) kahan_add(ks, kc, part[mine * S.GJ + q]);
+    for (int q = 0; q < S.GJ; ++q) kahan_add(ks, kc, part[mine * S.GJ + q] - comp[mine * S.GJ + q]);
     const float ic = (ks - kc) * (1.0f / GJ_SCALE);
     const CellNext o = cell_step(c.P, staged_cell(cs, S.rows, mine), ic, iapp);
     finish_cell(c, t, vd_next(c), row0 + mine, o);
 }
 
 cudaError_t prepare_matrix_step() {
-    const int smem = MX_THREADS * (1 + MX_WARPS + NCW) * (int)sizeof(float);   // the largest shape's
+    const int smem = MX_THREADS * (1 + 2 * MX_WARPS + NCW) * (int)sizeof(float);   // the largest shape's
     cudaError_t e = cudaFuncSetAttribute(matrix_step_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(matrix_step_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(matrix_step_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

@@ -52,3 +52,23 @@ def test_one_cta_sums_are_as_accurate_as_the_step_launches(torch_cuda):
                     e = (sim.state(18) - f.sum(1)) / np.abs(f).sum(1)
                 rms[q] += np.sqrt((e * e).mean())
     assert rms[1] <= 1.008 * rms[0], rms
+
+
+@pytest.mark.parametrize("n", [8193, 8448, 16640])
+def test_matrix_beyond_one_column_tile(torch_cuda, n):
+    """Two and three column tiles per row.  A term is good to about 2^-22 of its size (the
+    transform, ex2 and two products), a lane's chain has 8 terms, and the rest is pairwise or
+    compensated: 2^-21 of the sum of the terms' magnitudes."""
+    torch = torch_cuda
+    S = ion.ion_default_state(n)
+    S[0] = (-60 + np.random.default_rng(n).normal(0, 8, n)).astype(np.float32)
+    W = torch.rand((n, n), device="cuda", generator=torch.Generator("cuda").manual_seed(1)) * 1e-4
+    torch.cuda.synchronize()
+    with ion.Simulation(n, ion.DENSE_MATRIX, w=W, init_state=S) as sim:
+        sim.step(1)
+        ic = torch.from_numpy(sim.state(18)).cuda().double()
+    V = torch.from_numpy(S[0]).cuda().double()
+    for a in range(0, n, 1000):
+        d = V[a:a + 1000, None] - V[None]
+        f = (0.8 * torch.exp(-d * d / 100) + 0.2) * d * W[a:a + 1000].double()
+        assert bool(((ic[a:a + 1000] - f.sum(1)).abs() <= 2.0 ** -21 * f.abs().sum(1)).all())
