@@ -248,7 +248,8 @@ static int num_sms() {
 // 18 688 cells: the choice is within 0.9 % of the best on average, 4.6 % at worst.  us per
 // step, this choice / rows and warps alone as before: 1 003 cells 2.88 / 3.47; 2 999: 4.60 /
 // 4.64; 8 192: 12.4 / 12.7; 9 000: 15.4 / 15.6; 12 000: 22.6 / 22.9.
-void ion_choose_dense_shape(int n, int sms, int *R_out, int *W_out, int *GJ_out) {
+// max_threads: what a CTA of R rows per warp may have; the modelled cost is returned.
+double ion_choose_dense_shape(int n, int sms, int *R_out, int *W_out, int *GJ_out, int (*max_threads)(int)) {
     static const int Rs[] = {1, 2, 4, 6, 8};
     static const int GJs[] = {1, 2, 4};
     double best = -1.0;
@@ -257,7 +258,7 @@ void ion_choose_dense_shape(int n, int sms, int *R_out, int *W_out, int *GJ_out)
         for (int GJ : GJs)
             for (int GR = 1; GR <= 32; ++GR) {
                 const int W = GR * GJ;
-                if (W * 32 > dense_max_threads(R)) continue;
+                if (W * 32 > max_threads(R)) continue;
                 const long rows = (long)GR * R;
                 const long waves = ((n + rows - 1) / rows + sms - 1) / sms;
                 const double few = W >= 24 ? 1.0 : (W >= 18 ? 1.02 : (W >= 12 ? 1.06 : (W >= 8 ? 1.1 : 1.4)));
@@ -273,6 +274,7 @@ void ion_choose_dense_shape(int n, int sms, int *R_out, int *W_out, int *GJ_out)
     *R_out = bR;
     *W_out = bW;
     *GJ_out = bGJ;
+    return best;
 }
 
 // CSR: lanes per row from the mean degree (about two edges per lane per pass, four per

@@ -87,7 +87,10 @@ static ion_status persist_run(ion_sim *s, int64_t n_steps, const float *iapp) {
 
 // Shape of a persistent launch: one CTA of its own kernel for small networks; else the
 // per-step shape, if the persistent kernel allows that many threads and all its CTAs
-// can be resident at once.
+// can be resident at once.  Where the built-in per-step shape has too many threads, the best
+// within the limit takes its place if the model puts it level (11 553-12 160, 12 769-13 376 and
+// 13 985-14 592 cells: four rows per warp instead of eight); a shape that costs more is left to
+// the per-step launches.
 static bool choose_persist_shape(ion_sim *s) {
     if (s->n <= DENSE_SMALL) {
         s->persist_R = s->persist_W = s->persist_GJ = 1;   // not used
@@ -96,8 +99,13 @@ static bool choose_persist_shape(ion_sim *s) {
     PersistArgs probe{};
     probe.c.n = s->n;
     probe.c.n_pad = s->n_pad;
-    const int R = s->dense_R, W = s->dense_W, GJ = s->dense_GJ;
-    if (W * 32 > persist_max_threads(R)) return false;
+    int R = s->dense_R, W = s->dense_W, GJ = s->dense_GJ;
+    if (W * 32 > persist_max_threads(R)) {
+        int R0, W0, GJ0;
+        const double step = ion_choose_dense_shape(s->n, s->sms, &R0, &W0, &GJ0);
+        if (R != R0 || W != W0 || GJ != GJ0) return false;   // asked for by hand
+        if (ion_choose_dense_shape(s->n, s->sms, &R, &W, &GJ, persist_max_threads) > 1.005 * step) return false;
+    }
     int grid = 0;
     if (persist_dense(probe, R, W, GJ, &grid, false, s->st) != cudaSuccess || grid <= 0) return false;
     s->persist_R = R;

@@ -134,7 +134,8 @@ ion_status ion_cell_params_to_f32(const float *cp, int32_t n, const ion_model &m
 ion::StepCommon ion_step_common(ion_sim *s, int k_off, const float *iapp);
 float *ion_field_ptr(ion_sim *s, int32_t field);
 ion_status ion_validate_csr(int32_t n, const ion_conn *c);
-void ion_choose_dense_shape(int n, int sms, int *R, int *W, int *GJ);
+double ion_choose_dense_shape(int n, int sms, int *R, int *W, int *GJ,
+                              int (*max_threads)(int) = ion::dense_max_threads);
 void ion_choose_csr_shape(double mean_deg, int *SW, int *rows);
 // 16-bit columns of a sorted host CSR in shared-memory bank order (ion_bank.cu)
 bool ion_csr_bank_col16(int32_t n, int32_t n_pad, const int32_t *row_ptr, const int32_t *col,

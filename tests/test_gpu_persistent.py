@@ -163,3 +163,18 @@ def test_one_cta_network_matches_step_launches(cuda, O, n):
     assert np.abs(out[0][:3] - out[1][:3]).max() <= 1e-4
     assert (np.abs(out[0] - out[1])[3:18] / scale[3:18]).max() <= 1e-4
     assert np.abs(out[0][18] - out[1][18]).max() <= 1e-4
+
+
+@pytest.mark.parametrize("n", [11600, 12100, 13000, 14200])
+@pytest.mark.parametrize("half", [False, True])
+def test_persistent_launch_where_the_step_shape_has_too_many_threads(cuda, O, n, half):
+    """The per-step shape of these sizes has eight rows per warp, more threads than the persistent
+    kernel allows: it takes a shape of its own, one launch (and one counter advance) per call.
+    The sums' order differs, so close, not equal."""
+    g = inputs.junction_weight(0.04, n)
+    S0 = initial_state(O, dict(n=n, jitter=inputs.vdend_jitter(n, 9)))
+    flags = ion.FLAG_KAHAN | ion.FLAG_PERSISTENT | (ion.FLAG_HALF_WORK if half else 0)
+    a, _ = _run(n, g, S0, 40, ion.FLAG_KAHAN, chunks=2)
+    b, lb = _run(n, g, S0, 40, flags, chunks=2)
+    assert lb == 4
+    assert np.abs(a[:3] - b[:3]).max() <= 1e-3
