@@ -68,7 +68,7 @@ class ion_params(ctypes.Structure):
 
 
 class ion_input(ctypes.Structure):
-    _fields_ = [("kind", ctypes.c_int32), ("mem", ctypes.c_int32), ("dense", ctypes.c_void_p), ("n_pulses", ctypes.c_int32),
+    _fields_ = [("kind", ctypes.c_int32), ("mem", ctypes.c_int32), ("dense", c_f32p), ("n_pulses", ctypes.c_int32),
                 ("pulse_cell", c_i32p), ("pulse_begin", c_i64p), ("pulse_end", c_i64p), ("pulse_amp", c_f32p)]
 
 
@@ -105,7 +105,7 @@ _SIGS = {
     "ion_set_input": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ion_input)]),
     "ion_step": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64, ctypes.POINTER(ion_input)]),
     "ion_sync": (ctypes.c_int, [ctypes.c_void_p]),
-    "ion_read_state": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p, ctypes.c_int64]),
+    "ion_read_state": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, c_f32p, ctypes.c_int64]),
     "ion_write_state": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, c_f32p, ctypes.c_int64]),
     "ion_state_device_ptr": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, ctypes.POINTER(ctypes.c_void_p)]),
     "ion_set_trace": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32]),
@@ -172,6 +172,12 @@ def _ptr(a, ctype):
     if hasattr(a, "data_ptr"):
         return ctypes.cast(ctypes.c_void_p(a.data_ptr()), ctypes.POINTER(ctype))
     return a.ctypes.data_as(ctypes.POINTER(ctype))
+
+
+def _f32_at(address: int):
+    """The float pointer to an address (the calls of a closed loop: a cast costs several times as
+    much; nothing is read through it here)."""
+    return ctypes.pointer(ctypes.c_float.from_address(address))
 
 
 def _is_device(a) -> bool:
@@ -310,7 +316,7 @@ def _input_struct(pulses=None, dense=None):
         else:
             dense = np.ascontiguousarray(dense, np.float32)
             inp.mem = HOST
-        inp.dense = dense.data_ptr() if hasattr(dense, "data_ptr") else dense.ctypes.data
+        inp.dense = _f32_at(dense.data_ptr() if hasattr(dense, "data_ptr") else dense.ctypes.data)
         keep.append(dense)
     elif pulses is not None:
         inp.kind = INPUT_PULSES
@@ -350,7 +356,7 @@ def ion_sync(h):
 
 def ion_read_state(h, n: int, field: int = FIELD_ALL) -> np.ndarray:
     out = np.zeros((NFIELDS, n) if field == FIELD_ALL else (n,), np.float32)
-    _check(lib().ion_read_state(h, int(field), out.ctypes.data, out.size), h)
+    _check(lib().ion_read_state(h, int(field), _f32_at(out.ctypes.data), out.size), h)
     return out
 
 
