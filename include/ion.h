@@ -256,9 +256,10 @@ ion_status ion_create(const ion_net *net, const ion_conn *conn, const ion_params
 /* Several independent networks advanced together: one to three launches per time step cover
  * all of them (lists of tiles, each one network's rows; the launches of different lists run
  * side by side, on streams of the handle that are forked from and joined to its stream within
- * ion_step), and ion_step replays CUDA graphs of graph_steps steps.  Cells are numbered consecutively across networks (network b's
- * cell i is global cell offset_b + i, offset_b = n_0 + ... + n_{b-1}); init_state, the
- * state read and written, pulse cells and trace samples all use this numbering.
+ * ion_step; a call of a few steps may run them one after the other on the handle's stream), and
+ * ion_step replays CUDA graphs of graph_steps steps.  Cells are numbered consecutively across
+ * networks (network b's cell i is global cell offset_b + i, offset_b = n_0 + ... + n_{b-1});
+ * init_state, the state read and written, pulse cells and trace samples all use this numbering.
  * Dense networks may have at most 8192 cells; CSR arrays must be host memory.
  * ION_FLAG_PERSISTENT: each ion_step call is one cooperative launch (replayed from a CUDA
  * graph) that advances every network by all its steps.  The networks are cut into pieces
@@ -286,7 +287,9 @@ ion_status ion_sync(ion_sim *sim);
 
 /* Copy state to host memory `out` (count floats: n_cells for one field, 19 * n_cells
  * for ION_FIELD_ALL).  Synchronises; returns a sticky device error if there is one
- * (the copy is still made). */
+ * (the copy is still made).  A single network's fourth read of at most 16 384 floats makes a
+ * pinned buffer (about 0.3 ms, once), through which later such reads and host inputs of that
+ * size go: a loop with a deadline makes four reads before it begins. */
 ion_status ion_read_state(ion_sim *sim, int32_t field, float *out, int64_t count);
 
 /* Overwrite state from host memory `in` (same sizes as ion_read_state).  Ordered on
@@ -318,8 +321,9 @@ ion_status ion_trace_wait(ion_sim *sim);
  * and keep the fastest (the state and step count are restored afterwards).  Single
  * dense networks: (R, W, GJ) near the cost model's optimum; single CSR networks: lanes
  * per row and rows per CTA around the degree-based choice; batches: rows per dense tile,
- * rows per CSR tile and the lanes-per-row scale.  *chosen (nullable) receives the table.
- * Not for ION_FLAG_PERSISTENT handles.  Synchronises. */
+ * rows per CSR tile and the lanes-per-row scale, or, with ION_FLAG_PERSISTENT, the rows per
+ * warp of that launch's dense pieces.  *chosen (nullable) receives the table.
+ * Not for single ION_FLAG_PERSISTENT networks.  Synchronises. */
 ion_status ion_autotune(ion_sim *sim, int32_t steps, ion_tune *chosen);
 
 /* Storage the handle streams per stored edge of a CSR network (host-copied CSR only; a

@@ -31,7 +31,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t phase) {
 // stream is still draining.  pdl_enter() first waits until that kernel has completed and
 // its writes are visible (at once for an ordinary launch), then allows the next kernel
 // launched that way to be scheduled.  Every kernel so launched calls it before its first
-// access to memory that the launch before it writes.
+// access to memory that a launch or the caller may write (launch_k has the rule).
 __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -13,10 +13,11 @@
 // long ones first; the launches of K steps are captured into one CUDA graph and replayed.
 // ion_autotune times the tile shapes and keeps the fastest.
 //
-// What bounds it: instruction issue (the 96-network sweep of 32-4096 cells: 70 % issued).
-// That sweep, us per step: 20.3 (the 48 dense networks alone 17.5, the 48 CSR ones 8.8); one
-// launch per step with fixed tiles, 16-bit rows with heads and tails, state and pulses read
-// after the sums took 30.4.
+// What bounds it: the dense chains' pair loops and the updates between them (256 networks: the
+// dense launches keep the XU pipe 53 % and issue 63 % busy, the CSR launch is bound by latency
+// beside them).  A sweep of 96 networks of 32-4096 cells, us per step: 20.3 (the 48 dense networks
+// alone 17.5, the 48 CSR ones 8.8); one launch per step with fixed tiles, 16-bit rows with heads
+// and tails, state and pulses read after the sums took 30.4.
 #include <cuda_runtime.h>
 
 #include <algorithm>

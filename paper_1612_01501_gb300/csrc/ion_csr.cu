@@ -148,10 +148,10 @@ cudaError_t prepare_csr_step() {
 // caller (a.borrowed) are read after the wait: the caller may rewrite them on the handle's
 // stream between two calls, and only the wait orders this kernel after such a write.  A row of
 // more than a.long_rounds rounds (a multiple of the mean row) is finished by its whole warp:
-// 65 536 cells, k = 10, 8 rows of 3000 edges: 75.7 us per step with SW lanes for every row, 26.6 now.  256 threads, SW lanes
-// per row, four gathers in flight per lane; then one thread per row runs the update.  C16:
-// 16-bit columns.  LIN: linear junctions, w (V_i - V_j).
-// 65 536 cells, k = 10: 5.6 us per step (4 lanes, 128 rows per CTA); the kernel that read
+// 65 536 cells, k = 10, 8 rows of 3000 edges: 75.7 us per step with SW lanes for every row, 26.6
+// now.  256 threads, SW lanes per row, four gathers in flight per lane; then one thread per row
+// runs the update.  C16: 16-bit columns.  LIN: linear junctions, w (V_i - V_j).
+// 65 536 cells, k = 10: 5.5 us per step (4 lanes, 128 rows per CTA); the kernel that read
 // bounds, columns, gathers, state and pulses one after the other took 9.5 (7.1 tuned).
 constexpr int SHORT_E = 4;
 

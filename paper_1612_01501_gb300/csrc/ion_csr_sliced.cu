@@ -11,8 +11,9 @@
 // rows small (sorted sliced ELLPACK, Kreutzer et al. 2014).  A row far longer than the mean
 // gets more lanes, up to the whole warp: a warp walking it with SW lanes would hold every
 // other warp at the chunk's barrier (65 536 cells, k = 100, 8 rows of 3000 edges: 37.5 us per
-// step with the mean row's lanes, 10.3 now, 10.0 without such rows).  Columns are 16-bit offsets into the staged buffer; padding entries point at the
-// row's own V_dend behind the buffers (dV = 0: they add exactly 0).
+// step with the mean row's lanes, 10.3 now, 10.0 without such rows).  Columns are 16-bit
+// offsets into the staged buffer; padding entries point at the row's own V_dend behind the
+// buffers (dV = 0: they add exactly 0).
 //
 // Bank order: one gather reads entry t of all 32 lanes, from 32 random banks about 3.5
 // wavefronts, and these bound the sums.  The order of a lane's edges is free, so the fill

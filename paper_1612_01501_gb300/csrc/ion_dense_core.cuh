@@ -10,8 +10,6 @@
 
 namespace ion {
 
-constexpr float PAD_U = 1.0e6f;   // |u| of padded columns: 2^{-PAD_U^2} is exactly 0 (matrix kernel)
-
 // u = s V - C of a row, C = fl(s m) with m the step's shift (V_dend of cell 0): one fused
 // operation, the columns' negated x = C - s V the same bits with the other sign.  C is rounded,
 // but the same C enters every u, so differences and N u_i - sum u_j are free of it; each u is

@@ -24,7 +24,7 @@ static cudaError_t reset_barrier(ion_sim *s) {
 }
 
 // Multi-CTA networks use the half-work kernel (each unordered pair once, two barriers per
-// step); one-CTA networks the full-work kernel with V_dend kept in shared memory.
+// step); networks of up to DENSE_SMALL cells the one-CTA kernel.
 static ion_status half_run(ion_sim *s, int64_t n_steps, const float *iapp) {
     (void)iapp;
     int64_t done = 0;

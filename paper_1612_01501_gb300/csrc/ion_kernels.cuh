@@ -42,8 +42,12 @@ struct StepCommon {
 };
 
 // Launch a per-step kernel; with `pdl`, with programmatic stream serialization, so that
-// its CTAs may be scheduled while the kernel before it drains (the kernel starts with
-// pdl_enter(), which waits for that kernel's completion before any global access).
+// its CTAs may be scheduled while the kernel before it drains.  Before pdl_enter() returns, a
+// kernel so launched reads only what the handle owns and no launch writes while steps are in
+// flight: its copy of the connectivity, pulses, tile lists, learned weights.  State, the step
+// counter, evoked input, another launch's results and arrays borrowed from the caller are read
+// after it: the wait is what makes earlier writes visible, also those of launches before the one
+// waited for.
 template <class... P, class... A>
 inline cudaError_t launch_k(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl,
                             A... args) {
