@@ -22,3 +22,14 @@ def test_dense_input_points_at_the_array():
     inp, keep = ion._input_struct(dense=x)
     assert ctypes.addressof(inp.dense.contents) == x.ctypes.data and keep[0] is x
     assert [inp.dense[k] for k in range(6)] == list(range(6))
+
+
+def test_dense_input_from_a_read_only_array_and_a_tensor():
+    x = np.arange(6, dtype=np.float32)
+    x.flags.writeable = False
+    inp, _ = ion._input_struct(dense=x)
+    assert ctypes.addressof(inp.dense.contents) == x.ctypes.data
+    torch = pytest.importorskip("torch")
+    t = torch.arange(6, dtype=torch.float32)
+    assert ctypes.addressof(ion._f32(t)) == t.data_ptr()
+    ion._f32(np.zeros((0,), np.float32))               # an empty array has an address too
