@@ -315,7 +315,9 @@ void ion_choose_direct_shape(int32_t n, double mean_deg, int sms, int *SW, int *
 // Shared-memory staging of V_dend for a CSR network (mode 0: choose, 1: off, 2: on).
 // The sliced kernel pays per chunk of V_dend (about 1.7 us: the copy, the slices' bookkeeping),
 // the direct kernel per edge (a 32-byte sector from L2, 4.4 us per million; 1.8 where V_dend
-// fits L1 beside the rest) and, up to about a wave of CTAs, per row; us per step direct / staged:
+// fits L1 beside the rest).  Networks of 40 000 to 50 000 cells with ten edges per row gather
+// although staging is 3 to 5 % faster there: the slices cost 14 ms at creation, 70 000 steps' worth
+// of that gain.  us per step direct / staged:
 // 2 000 cells, k = 200: 3.1 / 4.3; 4 000: 4.0 / 4.3 (100); 10 000: 3.7 / 4.2 (24), 4.5 / 4.3 (40);
 // 20 000: 3.5 / 4.5 (10), 4.6 / 4.6 (24), 6.5 / 4.7 (40); 30 000: 4.1 / 4.6 (10); 40 000: 5.1 /
 // 4.9 (10), 7.4 / 5.1 (24); 50 000: 5.4 / 5.1 (10); 65 536: 5.5 / 8.1 (10), 8.9 / 8.4 (24);
@@ -331,7 +333,7 @@ static bool stage_by_default(const ion_sim *s, double deg, double csr_bytes) {
     const SliceLayout L = ion_plan_sliced(s->n, s->n_pad, s->nnz, s->sms, 0);
     const double waves = std::ceil((double)s->n / L.rows / s->sms);
     const double staged = 2.5 + 1.7 * L.n_chunks * waves + 2.0e-5 * s->n;
-    const double direct = 2.2 + 3.0e-5 * std::min(s->n, 50000) + (s->n <= 4000 ? 1.8e-6 : 4.4e-6) * (double)s->nnz;
+    const double direct = 2.2 + (s->n <= 4000 ? 1.8e-6 : 4.4e-6) * (double)s->nnz;
     return staged < direct;
 }
 // The 16-bit columns serve the staged kernel (columns relative to a chunk of at most 2^16

@@ -99,9 +99,9 @@ def test_unstaged_16_bit_rows_one_step(torch_cuda, O, n, k, weights, linear):
     assert err.max() <= STEP_RTOL, err.max(axis=1)
 
 
-# both sides of the line between gathering and staging, each at least as fast there as the other
-# (the figures are beside the rule)
-@pytest.mark.parametrize("n,k,staged", [(2000, 200, 0), (10000, 24, 0), (30000, 10, 0), (40000, 10, 1), (50000, 10, 1),
+# both sides of the line between gathering and staging (the figures are beside the rule); short
+# rows of 40 000 to 50 000 cells gather although staging gains 3 to 5 %
+@pytest.mark.parametrize("n,k,staged", [(2000, 200, 0), (10000, 24, 0), (30000, 10, 0), (20000, 24, 0), (40000, 10, 0), (50000, 10, 0),
                                         (20000, 40, 1), (65536, 10, 0), (65536, 24, 1), (100000, 24, 1), (300000, 10, 0)])
 def test_default_staging(torch_cuda, n, k, staged):
     rp, col = inputs.random_symmetric_csr(n, k, 3)
