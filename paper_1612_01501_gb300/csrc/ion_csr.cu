@@ -525,8 +525,8 @@ constexpr int CELL_THREADS = 128;   // CTA of the kernels that only update cells
 // 256 of them held every CTA of the update for 2 us), the cells' words are on their way before
 // the sum is known, the pulses before the wait, and the update walks the cells in opposite directions on even
 // and odd steps (cell_step_kernel).
-// Per step before / now: 200 cells 2.6 / 2.0 us, 8192 5.1 / 2.9, 16 384 7.1 / 3.7 (one launch),
-// 16 385 5.3 / 3.8, 100 003 7.4 / 5.5, 600 011 24.8 / 16.1, 1 211 904 57.4 / 30.1.
+// Per step before / now: 200 cells 3.1 / 2.1 us, 8192 5.2 / 3.0, 16 384 7.1 / 3.6 (one launch),
+// 16 385 5.5 / 4.5, 100 003 7.8 / 6.0, 600 011 25.9 / 16.6, 1 211 904 62.7 / 31.0.
 __device__ __forceinline__ void two_sum_add(float &s, float &e, float so, float eo) {   // (s + e) += so + eo
     const float t = s + so, b = t - s;
     e = (e + eo) + ((s - (t - b)) + (so - b));
