@@ -63,23 +63,23 @@ TRAFFIC = {   # an entry is removed when its kernel changes, until it is capture
     ("c2", "dense_step_kernel"): (530688, "profiles/dense_step_kernel_c2_8192.md",
                                   dict(dense_rows_per_warp=4, dense_warps=28, dense_col_splits=2)),
     ("k3", "cell_step_kernel"): (285282816 + 242117120, "profiles/cell_step_kernel_k3_4194304.md", {}),
-    ("c3_k10", "csr_direct_step_kernel"): (7364096, "profiles/csr_direct_step_kernel_c3_k10.md",
+    ("c3_k10", "csr_direct_step_kernel"): (7366144, "profiles/csr_direct_step_kernel_c3_k10.md",
                                            dict(csr_lanes_per_row=4, csr_rows_per_cta=128)),
     # the DRAM bytes of a cold launch are those of the layout (each index byte and state word
     # read once), the same for any lane count
-    ("c3_k100", "csr_sliced_step_kernel"): (21719808, "profiles/csr_sliced_step_kernel_c3_k100.md", dict(csr_staging=2)),
-    ("c3_k1000", "csr_sliced_step_kernel"): (139095296 + 2982656, "profiles/csr_sliced_step_kernel_c3_k1000.md",
+    ("c3_k100", "csr_sliced_step_kernel"): (21719552, "profiles/csr_sliced_step_kernel_c3_k100.md", dict(csr_staging=2)),
+    ("c3_k1000", "csr_sliced_step_kernel"): (139092480 + 2791424, "profiles/csr_sliced_step_kernel_c3_k1000.md",
                                              dict(csr_staging=2)),
     # the chunked kernel on the compact layout: networks kept in the opt-in bank order only, which
     # no workload asks for (the default staged network runs the sliced kernel)
     ("c3_k1000", "csr_chunk_step_kernel"): (135862784 + 2681600, "profiles/csr_chunk_step_kernel_c3_k1000.md",
                                             dict(csr_staging=2)),
-    ("c2_sgj", "sgj_dense_update_kernel"): (515584, "profiles/sgj_dense_update_kernel_c2_sgj_8192.md", {}),
+    ("c2_sgj", "sgj_dense_update_kernel"): (515328, "profiles/sgj_dense_update_kernel_c2_sgj_8192.md", {}),
     # one of the step's two dense launches
     ("c4", "batch_dense_kernel"): (3876352, "profiles/batch_kernels_c4.md", {}),
-    ("c5", "surrogate_tc_kernel"): (4796416, "profiles/surrogate_tc_kernel_c5.md", {}),
+    ("c5", "surrogate_tc_kernel"): (4798464, "profiles/surrogate_tc_kernel_c5.md", {}),
     # captured at four rows in flight: every weight is streamed once whatever their number
-    ("c2_matrix", "matrix_step_kernel"): (268974848 + 3223040, "profiles/matrix_step_kernel_c2_matrix_8192.md", {}),
+    ("c2_matrix", "matrix_step_kernel"): (268976640 + 3687680, "profiles/matrix_step_kernel_c2_matrix_8192.md", {}),
 }
 
 
